@@ -103,7 +103,7 @@ typedef enum {
                                     else STREAM */
     FLOOD_KERNEL_REFERENCE = 1,  /* one thread per cell, IEEE ops in the oracle's order */
     FLOOD_KERNEL_ROWS = 2,       /* one warp per 128-column strip, float4 row streaming */
-    FLOOD_KERNEL_TILED = 3,      /* pipeline of K warps per strip, K steps per launch (temporal blocking) */
+    FLOOD_KERNEL_TILED = 3,      /* one warp per strip and chunk, K steps per launch in registers (temporal blocking) */
     FLOOD_KERNEL_STREAM = 4,     /* one warp per 128-column strip, rows staged by bulk copies (default) */
     FLOOD_KERNEL_TMA = 5         /* as STREAM, rows staged as 2D tiles by tensor-map (TMA) copies */
 } flood_kernel;
@@ -118,7 +118,8 @@ typedef struct {
     int32_t epoch_steps;         /* E: steps per CFL epoch (1..1024) */
     int32_t bc_form;             /* 0 cell discharge dx h^(5/3) sqrt(S)/n, 1 literal dx^2 h^(2/3) sqrt(S)/n */
     int32_t kernel;              /* flood_kernel */
-    int32_t steps_per_launch;    /* K for FLOOD_KERNEL_TILED: 1..4 or 8, must divide E (0 = 4) */
+    int32_t steps_per_launch;    /* K for FLOOD_KERNEL_TILED: 1..4 or 8, must divide E (0 = 4; 8 runs as two
+                                    launches of 4) */
     int32_t tile_x, tile_y;      /* launch shape, 0 = chosen by the library.  STREAM: warps per block (1..4),
                                     rows per chunk.  TILED: at most tile_x pipelines (blocks), tile_y rows
                                     per work item (a chunk of one 120-column strip).  Negative: invalid. */
@@ -326,10 +327,11 @@ flood_status flood_ensemble_create(int32_t n, const flood_grid *grids, const voi
                                    const void *const *mannings, const flood_bc_section *const *sections,
                                    const int32_t *n_sections, const flood_opts *opts, flood_ensemble **out);
 /* Launch shape: warps per block (1..4, stream kernel), rows per chunk (stream
- * blocks; for the tiled kernel the rows per (chunk, strip) item of a grid of
- * 2^20 cells, scaled by sqrt(cells / 2^20) for the others, at least 32 and at
- * most the grid's rows: the largest grids come first with the longest items
- * and the small ones fill the end of the launch), steps per graph replay,
+ * blocks; for the tiled kernel the most rows per (chunk, strip) item of a grid
+ * of 2^20 cells, scaled by sqrt(cells / 2^20) for the others: the library takes
+ * fewer where the scenarios give too few items to fill the GPU evenly; the
+ * largest grids come first with the longest items and the small ones fill the
+ * end of the launch), steps per graph replay,
  * graph on/off.  FLOOD_ERR_ARG on values out of range. */
 flood_status flood_ensemble_set_launch(flood_ensemble *e, int32_t warps, int32_t rows, int32_t steps_per_graph,
                                        int32_t use_graph);
@@ -452,14 +454,14 @@ int64_t flood_debug_alloc_count(void);
 flood_status flood_debug_padding(flood_handle *h, int32_t fill, int64_t *bad);
 
 /*
- * flood_debug_tiled_split: the work items the temporal-blocking kernel would
- * split an nx x ny grid into (host only, no device): k_steps 1..4 or 8, mode
- * bit 0 theta weighting and bit 1 vector-norm friction (they narrow the
- * strips), resident >= 1 the pipelines the GPU holds at once (912 on a GB300
- * for K = 4 as printed).  *chunk_rows the rows per item, *blocks the
- * pipelines launched, *n_items the (chunk, strip) items.  FLOOD_ERR_ARG (no
- * message) for arguments out of range, NULL outputs or more than 2^31 - 1
- * items.
+ * flood_debug_tiled_split: the work items the temporal-blocking kernel splits
+ * an nx x ny grid into when the caller holds it to `resident` pipelines
+ * (flood_opts.tile_x) that walk the items in turn (host only, no device):
+ * k_steps 1..4 or 8, mode bit 0 theta weighting and bit 1 vector-norm friction
+ * (they narrow the strips), resident >= 1.  *chunk_rows the rows per item,
+ * *blocks the pipelines launched, *n_items the (chunk, strip) items.
+ * FLOOD_ERR_ARG (no message) for arguments out of range, NULL outputs or more
+ * than 2^31 - 1 items.
  */
 flood_status flood_debug_tiled_split(int32_t nx, int32_t ny, int32_t k_steps, int32_t mode, int32_t resident,
                                      int32_t *chunk_rows, int32_t *blocks, int32_t *n_items);

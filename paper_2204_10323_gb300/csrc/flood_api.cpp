@@ -344,7 +344,6 @@ flood_status advance(flood_handle *h, int64_t n, const int64_t *gcells, int ng, 
         int k = 1;
         if (h->prec == FLOOD_F32 && h->kernel == FLOOD_KERNEL_TILED && !gcells) {
             k = std::min<int64_t>(h->k_per_launch, std::min<int64_t>(E - s, n - done));
-            if (k > 4 && k < 8) k = 4;   // the kernel exists for 1..4 and 8 steps per launch
         }
         int want = (s + k == E) ? 1 : 0;
         flood_status st = launch_steps(h, s, k, want, gcells, ng, gcells ? gbuf + done * ng : nullptr);
@@ -540,7 +539,8 @@ flood_status create_handle(const flood_grid *grid, const void *dem, const void *
     h->tile_x = o.tile_x;
     h->tile_y = o.tile_y;
     if (h->kernel == FLOOD_KERNEL_TILED)
-        h->k_per_launch = (o.kernel == FLOOD_KERNEL_TILED && o.steps_per_launch > 0) ? o.steps_per_launch : 4;
+        // 8 steps run as two launches of 4: the state of 8 time levels does not fit a warp's registers
+        h->k_per_launch = (o.kernel == FLOOD_KERNEL_TILED && o.steps_per_launch > 0) ? std::min(o.steps_per_launch, 4) : 4;
 
     auto bail = [&](flood_status st, const char *msg) {
         std::string m = msg;

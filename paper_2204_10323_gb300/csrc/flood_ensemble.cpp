@@ -28,21 +28,20 @@ struct flood_ensemble {
     int64_t step = 0;
     cudaStream_t stream = nullptr;
     int warps = 4, rows = 64, steps_per_graph = 16;
-    int kernel = FLOOD_KERNEL_STREAM, k_steps = 4;   // TILED: k_steps per launch, rows per item
+    int base_rows = 64;                    // tiled: rows per item of a grid of 2^20 cells (choose_rows)
+    int kernel = FLOOD_KERNEL_STREAM, k_steps = 4;   // TILED: k_steps per launch (1..4), rows per item
     int mode = 0;                          // scheme options: bit 0 theta weighting, bit 1 vector-norm friction
     StepArgs<float> *table[2] = {nullptr, nullptr};   // per parity of the ping-pong buffers
     int *base = nullptr;                   // block prefix, n + 1
     int total_blocks = 0;
     int *tbase = nullptr;                  // tiled item prefix, n + 1
     int total_items = 0;
-    int *next_item = nullptr;              // tiled: the item counter of the launch (zeroed before each)
     // tiled: the members in two groups of about equal cells, each launched on a stream of its
     // own from one epoch start to the next, so that one group's launches fill the other's tails
     static constexpr int kGroups = 2;
     std::vector<int> group_of;             // per member
     StepArgs<float> *gtable[kGroups][2] = {{nullptr, nullptr}, {nullptr, nullptr}};   // [group][parity]
     int *gtbase[kGroups] = {nullptr, nullptr};
-    int *gnext[kGroups] = {nullptr, nullptr};
     int gn[kGroups] = {0, 0}, gtotal[kGroups] = {0, 0};
     EpochArgs<float> *getab[kGroups] = {nullptr, nullptr};   // the group's members' epoch arguments
     int2 *gtasks[kGroups] = {nullptr, nullptr};              // (member in the group, inflow section)
@@ -100,27 +99,56 @@ EpochArgs<float> epoch_args(const flood_handle *h)
     return A;
 }
 
-// Rows per work item of the temporal-blocking kernel for a member grid: the
-// launch shape's rows for a grid of 2^20 cells, scaled by the square root of
-// the grid's cells over that, at least 32 and at most the grid's rows.  The
-// grids come largest first, so the items shrink towards the end of a launch,
-// where the pipelines, taking items as they come free, fill the tail with the
-// small ones (the measured best of several rules on uneven scenario mixes).
+// Rows per work item of the temporal-blocking kernel for a member grid (an edge
+// strip's items have five eighths of them): base_rows for a grid of 2^20 cells, scaled
+// by the square root of the grid's cells over that, at least 8 and at most the
+// grid's rows.  The grids come largest first, so the items shrink towards the end of
+// a launch, where the small ones fill the tail.
 int item_rows(const flood_ensemble *e, const Geom &g)
 {
     const double cells = (double)g.nx * g.ny;
-    const int r = (int)(e->rows * std::sqrt(cells / (double)(1 << 20)) + 0.5);
-    return std::min(std::max(r, 32), g.ny);
+    const int r = (int)(e->base_rows * std::sqrt(cells / (double)(1 << 20)) + 0.5);
+    return std::min(std::max(r, 8), g.ny);
+}
+
+int edge_rows(int rows) { return (5 * rows + 7) / 8; }
+
+// base_rows, at most the launch shape's rows: each item repeats 2K rows, and the launch ends
+// with its longest items' last rows, so few rows cost work and many leave warps idle.  The cost is
+// the items' ticks over the warps that the GPU holds, plus half the longest item.
+void choose_rows(flood_ensemble *e)
+{
+    const double resident = 152.0 * 12.0;      // one-warp items the GPU holds at once
+    const int K = e->k_steps;
+    double best = -1.0;
+    int rows = e->rows;
+    for (int b : {8, 12, 16, 20, 24, 32, 40, 48, 64, 80, 96, 128, 160, 192, 256, 320, 384, 512, e->rows}) {
+        if (b > e->rows) continue;
+        e->base_rows = b;
+        double ticks = 0.0, longest = 0.0;
+        for (const flood_handle *h : e->members) {
+            const int r = item_rows(e, h->geo);
+            ticks += (double)tiled_items(h->geo, r, edge_rows(r), K) * (r + 2 * K);
+            longest = std::max(longest, (double)(r + 2 * K));
+        }
+        const double cost = std::max(ticks / resident, longest) + 0.5 * longest;
+        if (best < 0.0 || cost < best) {
+            best = cost;
+            rows = b;
+        }
+    }
+    e->base_rows = rows;
 }
 
 flood_status build_tables(flood_ensemble *e)
 {
     const int n = (int)e->members.size();
+    choose_rows(e);
     std::vector<int> base(n + 1, 0), tbase(n + 1, 0);
     for (int k = 0; k < n; k++) {
         const Geom &g = e->members[e->order[k]]->geo;
         base[k + 1] = base[k] + stream_blocks(g, e->warps, e->rows);
-        tbase[k + 1] = tbase[k] + tiled_items(g, item_rows(e, g), e->k_steps);
+        tbase[k + 1] = tbase[k] + tiled_items(g, item_rows(e, g), edge_rows(item_rows(e, g)), e->k_steps);
     }
     e->total_blocks = base[n];
     e->total_items = tbase[n];
@@ -132,6 +160,7 @@ flood_status build_tables(flood_ensemble *e)
             h->cur = p;
             t[k] = step_args_f32(h, 0);
             t[k].tile_y = item_rows(e, h->geo);
+            t[k].tile_x = edge_rows(t[k].tile_y);
             h->cur = cur;
         }
         cudaError_t c = cudaMemcpyAsync(e->table[p], t.data(), n * sizeof(StepArgs<float>), cudaMemcpyHostToDevice,
@@ -157,7 +186,7 @@ flood_status build_tables(flood_ensemble *e)
             std::vector<int> gb(ng + 1, 0);
             for (int i = 0; i < ng; i++) {
                 const Geom &G = e->members[members[g][i]]->geo;
-                gb[i + 1] = gb[i] + tiled_items(G, item_rows(e, G), e->k_steps);
+                gb[i + 1] = gb[i] + tiled_items(G, item_rows(e, G), edge_rows(item_rows(e, G)), e->k_steps);
             }
             e->gn[g] = ng;
             e->gtotal[g] = gb[ng];
@@ -169,6 +198,7 @@ flood_status build_tables(flood_ensemble *e)
                     h->cur = p;
                     t[i] = step_args_f32(h, 0);
                     t[i].tile_y = item_rows(e, h->geo);
+                    t[i].tile_x = edge_rows(t[i].tile_y);
                     h->cur = cur;
                 }
                 if (ng && (c = cudaMemcpyAsync(e->gtable[g][p], t.data(), ng * sizeof(StepArgs<float>),
@@ -231,7 +261,7 @@ flood_status ensemble_step(flood_ensemble *e, int64_t limit, cudaStream_t st, in
 {
     const int E = e->E;
     const int s = (int)(e->step % E);
-    const bool grouped = e->kernel == FLOOD_KERNEL_TILED && !(e->k_steps == 8 && (int)std::min<int64_t>(E - s, limit) < 8);
+    const bool grouped = e->kernel == FLOOD_KERNEL_TILED;
     if (s == 0 && grouped) {
         // each group starts its members' epoch on its own stream
         flood_status fs = fork_groups(e, st);
@@ -254,18 +284,14 @@ flood_status ensemble_step(flood_ensemble *e, int64_t limit, cudaStream_t st, in
     if (e->kernel == FLOOD_KERNEL_TILED) {
         steps = (int)std::min<int64_t>(e->k_steps, std::min<int64_t>(E - s, limit));
     }
-    // the item table is laid out for k_steps: 8-step tables (wider halos) take
-    // only whole 8-step launches, anything shorter runs single stream steps
-    if (e->kernel == FLOOD_KERNEL_TILED && !(e->k_steps == 8 && steps < 8)) {
+    if (grouped) {
         flood_status fs = fork_groups(e, st);
         if (fs) return fs;
         c = cudaSuccess;
         for (int g = 0; g < flood_ensemble::kGroups && c == cudaSuccess; g++) {
             if (e->gn[g] == 0) continue;
-            c = cudaMemsetAsync(e->gnext[g], 0, sizeof(int), e->lane[g]);
-            if (c == cudaSuccess)
-                c = launch_step_tiled_ensemble(e->gtable[g][parity], e->gtbase[g], e->gn[g], e->gtotal[g], steps, s,
-                                               s + steps == E ? 1 : 0, e->gnext[g], e->mode, e->lane[g]);
+            c = launch_step_tiled_ensemble(e->gtable[g][parity], e->gtbase[g], e->gn[g], e->gtotal[g], steps, s,
+                                           s + steps == E ? 1 : 0, e->mode, e->lane[g]);
         }
     } else {
         flood_status fs = join_groups(e, st);
@@ -386,16 +412,14 @@ extern "C" flood_status flood_ensemble_create(int32_t n, const flood_grid *grids
     }
     e->base = (int *)dev_alloc(e->owner, (n + 1) * sizeof(int));
     e->tbase = (int *)dev_alloc(e->owner, (n + 1) * sizeof(int));
-    e->next_item = (int *)dev_alloc(e->owner, sizeof(int));
     for (int g = 0; g < flood_ensemble::kGroups; g++) {
         for (int p = 0; p < 2; p++) e->gtable[g][p] = (StepArgs<float> *)dev_alloc(e->owner, n * sizeof(StepArgs<float>));
         e->gtbase[g] = (int *)dev_alloc(e->owner, (n + 1) * sizeof(int));
-        e->gnext[g] = (int *)dev_alloc(e->owner, sizeof(int));
         e->getab[g] = (EpochArgs<float> *)dev_alloc(e->owner, n * sizeof(EpochArgs<float>));
         int n_sec_all = 0;
         for (flood_handle *h : e->members) n_sec_all += h->n_in;
         e->gtasks[g] = (int2 *)dev_alloc(e->owner, std::max(n_sec_all, 1) * sizeof(int2));
-        if (!e->gtable[g][0] || !e->gtable[g][1] || !e->gtbase[g] || !e->gnext[g] || !e->getab[g] || !e->gtasks[g] ||
+        if (!e->gtable[g][0] || !e->gtable[g][1] || !e->gtbase[g] || !e->getab[g] || !e->gtasks[g] ||
             cudaStreamCreateWithFlags(&e->lane[g], cudaStreamNonBlocking) != cudaSuccess ||
             cudaEventCreateWithFlags(&e->lane_ev[g], cudaEventDisableTiming) != cudaSuccess) {
             flood_ensemble_destroy(e);
@@ -430,7 +454,7 @@ extern "C" flood_status flood_ensemble_create(int32_t n, const flood_grid *grids
     }
     e->n_tasks = (int)tk.size();
     e->tasks = (int2 *)dev_alloc(e->owner, std::max<size_t>(tk.size(), 1) * sizeof(int2));
-    if (!e->base || !e->tbase || !e->next_item || !e->etab || !e->tasks ||
+    if (!e->base || !e->tbase || !e->etab || !e->tasks ||
         cudaMemcpyAsync(e->etab, et.data(), n * sizeof(EpochArgs<float>), cudaMemcpyHostToDevice, e->stream) ||
         (tk.size() &&
          cudaMemcpyAsync(e->tasks, tk.data(), tk.size() * sizeof(int2), cudaMemcpyHostToDevice, e->stream))) {
@@ -469,7 +493,7 @@ extern "C" flood_status flood_ensemble_set_kernel(flood_ensemble *e, int32_t ker
     if (kernel == FLOOD_KERNEL_TILED && (!(K <= 4 || K == 8) || e->E % K != 0))
         return efail(e, FLOOD_ERR_ARG, "steps_per_launch must be 1..4 or 8 and divide epoch_steps");
     e->kernel = kernel;
-    e->k_steps = kernel == FLOOD_KERNEL_TILED ? K : 1;
+    e->k_steps = kernel == FLOOD_KERNEL_TILED ? std::min(K, 4) : 1;   // 8 steps run as two launches of 4
     return build_tables(e);                  // item counts depend on K; drops the graphs
 }
 
@@ -527,12 +551,10 @@ extern "C" flood_status flood_ensemble_destroy(flood_ensemble *e)
             if (e->table[p]) dev_free(e->owner, e->table[p]);
         if (e->base) dev_free(e->owner, e->base);
         if (e->tbase) dev_free(e->owner, e->tbase);
-        if (e->next_item) dev_free(e->owner, e->next_item);
         for (int g = 0; g < flood_ensemble::kGroups; g++) {
             for (int p = 0; p < 2; p++)
                 if (e->gtable[g][p]) dev_free(e->owner, e->gtable[g][p]);
             if (e->gtbase[g]) dev_free(e->owner, e->gtbase[g]);
-            if (e->gnext[g]) dev_free(e->owner, e->gnext[g]);
             if (e->getab[g]) dev_free(e->owner, e->getab[g]);
             if (e->gtasks[g]) dev_free(e->owner, e->gtasks[g]);
         }

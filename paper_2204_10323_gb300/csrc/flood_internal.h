@@ -28,7 +28,7 @@ struct Ctrl {
     double cfl_exceed;            // epochs whose dt broke dx / sqrt(g h_max) at their end
     unsigned long long hmax_bits; // running max of h (bits of a non-negative double)
     int status;                   // kStatus* bits
-    int next_item;                // the temporal-blocking kernel's work-item counter (zeroed before each launch)
+    int pad;
 };
 
 // One inflow section as seen by the Eq. 6 solver.
@@ -84,7 +84,8 @@ struct StepArgs {
     const int64_t *gauge_cells;   // flat j*nx+i; h after each step -> gauge_out
     int n_gauges;
     double *gauge_out;            // (k_steps) x n_gauges rows for this launch, or null
-    int tile_x, tile_y;           // launch shape (stream/TMA: warps, rows; tiled: strips, rows per item)
+    int tile_x, tile_y;           // launch shape (stream/TMA: warps, rows; tiled: rows per item of the edge
+                                  // strips and of the others; on its way in: cap on pipelines, rows per item)
 };
 
 // ---------------------------------------------------------------- launchers
@@ -101,13 +102,11 @@ cudaError_t launch_step_stream_ensemble(const StepArgs<float> *table, const int 
 // Blocks of one grid for the stream kernel, and the (warps, rows) a tile pair selects.
 int stream_blocks(const Geom &g, int warps, int rows);
 cudaError_t launch_step_tma(const StepArgs<float> &a, cudaStream_t st);
-// Temporal blocking over many grids: the (chunk, strip) items of grid k are
-// base[k] .. base[k+1] - 1 (tiled_items per grid, table[k].tile_y rows per item), k_steps steps from s0.
-int tiled_items(const Geom &g, int chunk_rows, int k_steps);
-// next_item (device, zero before the launch): the pipelines take their items after
-// the first from this counter (dynamic scheduling); null: block b takes b, b + grid, ...
+// Temporal blocking over many grids: the items of grid k are base[k] .. base[k+1] - 1 (tiled_items per
+// grid, table[k].tile_y rows per item, tile_x in the edge strips), k_steps steps from s0.
+int tiled_items(const Geom &g, int rows, int rows_edge, int k_steps);
 cudaError_t launch_step_tiled_ensemble(const StepArgs<float> *table, const int *base, int n, int total_items,
-                                       int k_steps, int s0, int want_hmax, int *next_item, int mode, cudaStream_t st);
+                                       int k_steps, int s0, int want_hmax, int mode, cudaStream_t st);
 void stream_launch_shape(const Geom &g, int tile_x, int tile_y, int *warps, int *rows);
 cudaError_t launch_step_tiled(const StepArgs<float> &a, cudaStream_t st);
 

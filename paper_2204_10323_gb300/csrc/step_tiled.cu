@@ -5,12 +5,41 @@
 
 namespace flood {
 
-// Row chunks for the (chunk, strip) work items of a grid of n_strips strips and
-// ny rows on `resident` pipelines: the chunk count minimises the ticks of the
-// busiest pipeline, (items per pipeline) x (chunk rows + 3K - 1), an item
-// costing its rows plus 2K - 1 staged halo rows and the 2(K - 1) ticks by
-// which level K lags level 1.
-void tiled_split(int n_strips, int ny, int resident, int K, int *chunk_rows, int *blocks)
+// Rows per item.  An item of r rows takes r + 2K ticks; a tick of a warp alone on its quarter of an SM
+// takes about 1650 cycles, beside others about 1150 + 490 per warp (K = 4, measured with the clock
+// register at 1024^2 .. 4096^2), and 1000 more in an edge strip, whose items are therefore shorter.  The
+// rows minimise the waves of items, the last one with the warps it has: few rows fill the GPU evenly but
+// repeat 2K rows each.  us per step with rows chosen so / fixed at 96: 11.0 / 36.8 (1024^2), 15.9 / 37.3
+// (2048^2), 39 / 50 (4096^2), 131 / 131 (8192^2), 465 / 477 (16384^2).
+void tiled_rows(int nx, int ny, int K, int mode, int *rows, int *rows_edge)
+{
+    static constexpr int kTry[] = {4,  6,  8,  10, 12, 14, 16,  18,  20,  22,  24,  28,  32, 36,
+                                   40, 44, 48, 56, 64, 80, 96, 112, 128, 144, 160, 192, 256};
+    const int sms = 152, resident = sms * tiled_warps(mode);
+    const int out = out_cols(K, mode), n_strips = (nx + out - 1) / out, n_edge = n_strips < 2 ? n_strips : 2;
+    const auto tick = [](double warps) { return 1150.0 + 490.0 * (warps > 1.0 ? warps : 1.0); };
+    const auto even = [&](int r) { return (ny + (ny + r - 1) / r - 1) / ((ny + r - 1) / r); };   // equal chunks of at most r
+    double best = -1.0;
+    for (int t : kTry) {
+        const int r = even(t), re = even((5 * t + 7) / 8);
+        const long long n = (long long)n_edge * ((ny + re - 1) / re) + (long long)(n_strips - n_edge) * ((ny + r - 1) / r);
+        const long long full = n / resident, rest = n % resident;
+        double cost = (r + 2 * K) * (full * tick(tiled_warps(mode) / 4.0) + (rest ? tick(rest / (4.0 * sms)) : 0.0));
+        const double edge = (re + 2 * K) * (tick(full ? tiled_warps(mode) / 4.0 : rest / (4.0 * sms)) + 1000.0);
+        if (edge > cost) cost = edge;
+        if (best < 0.0 || cost < best) {
+            best = cost;
+            *rows = r;
+            *rows_edge = re;
+        }
+        if (t >= ny) break;
+    }
+}
+
+// Row chunks for the items of a grid of n_strips strips and ny rows on `resident` pipelines that walk
+// them in turn (a caller's cap on the pipelines): the chunk count minimises the ticks of the busiest
+// pipeline, (items per pipeline) x (chunk rows + 3K - 1).
+static void tiled_split(int n_strips, int ny, int resident, int K, int *chunk_rows, int *blocks)
 {
     static thread_local int memo[4] = {-1, -1, -1, -1}, memo_rows = 0;   // per thread: no race between handles
     if (memo[0] == n_strips && memo[1] == ny && memo[2] == resident && memo[3] == K) {
@@ -43,14 +72,8 @@ void tiled_split(int n_strips, int ny, int resident, int K, int *chunk_rows, int
     *blocks = (int)(items < resident ? items : resident);
 }
 
-// The same when the pipelines take their items from a counter as they come free:
-// about eight items per pipeline, so that the ones that finish early take more
-// and the launch ends evenly, of at least 24 K rows (an item costs its rows plus
-// the 3K - 1 ticks of filling the pipeline); a grid that would get fewer than four
-// such items per pipeline keeps the round-robin split.  Measured against fixed
-// rows per item of 64 ... 384 on the fractal workload at 16384^2 (304 rows: 8
-// items per pipeline) and 8192^2 (96 rows: 6.5), and against the round-robin
-// split at 4096^2 and 2048^2.
+// The same with about eight items per pipeline of at least 24 K rows, so that the launch ends
+// evenly; a grid that would get fewer than four such items per pipeline keeps the split above.
 void tiled_split_dynamic(int n_strips, int ny, int resident, int K, int *chunk_rows, int *blocks)
 {
     const long long target = 8LL * resident;
@@ -69,12 +92,10 @@ void tiled_split_dynamic(int n_strips, int ny, int resident, int K, int *chunk_r
     *blocks = (int)(items < resident ? items : resident);
 }
 
-int tiled_items(const Geom &g, int chunk_rows, int k_steps)
+int tiled_items(const Geom &g, int rows, int rows_edge, int k_steps)
 {
     const int mode = (g.theta != 1.0 ? 1 : 0) | (g.friction != 0 ? 2 : 0);
-    const int out = out_cols(k_steps, mode);
-    const int n_strips = (g.nx + out - 1) / out;
-    return n_strips * ((g.ny + chunk_rows - 1) / chunk_rows);
+    return tiled_item_count(g.nx, g.ny, out_cols(k_steps, mode), rows, rows_edge);
 }
 
 // Scheme mode of a grid: bit 0 theta weighting, bit 1 vector-norm friction.
@@ -83,16 +104,15 @@ static int tiled_mode(const Geom &g) { return (g.theta != 1.0 ? 1 : 0) | (g.fric
 // step_tiled_opts.cu: the same launchers for modes 1..3.
 cudaError_t launch_step_tiled_opts(const StepArgs<float> &a, int mode, cudaStream_t st);
 cudaError_t launch_step_tiled_ensemble_opts(const StepArgs<float> *table, const int *base, int n, int total_items,
-                                            int k_steps, int s0, int want_hmax, int *next_item, int mode,
+                                            int k_steps, int s0, int want_hmax, int mode,
                                             cudaStream_t st);
 
 cudaError_t launch_step_tiled_ensemble(const StepArgs<float> *table, const int *base, int n, int total_items,
-                                       int k_steps, int s0, int want_hmax, int *next_item, int mode, cudaStream_t st)
+                                       int k_steps, int s0, int want_hmax, int mode, cudaStream_t st)
 {
     if (mode != 0)
-        return launch_step_tiled_ensemble_opts(table, base, n, total_items, k_steps, s0, want_hmax, next_item, mode,
-                                               st);
-    return launch_tiled_ensemble_mode<0>(table, base, n, total_items, k_steps, s0, want_hmax, next_item, st);
+        return launch_step_tiled_ensemble_opts(table, base, n, total_items, k_steps, s0, want_hmax, mode, st);
+    return launch_tiled_ensemble_mode<0>(table, base, n, total_items, k_steps, s0, want_hmax, st);
 }
 
 cudaError_t launch_step_tiled(const StepArgs<float> &a, cudaStream_t st)
