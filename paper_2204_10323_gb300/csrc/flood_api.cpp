@@ -176,19 +176,35 @@ void field_shape(const flood_handle *h, int field, int *rows, int *cols)
     *cols = h->geo.nx + (field == FLOOD_FIELD_QX ? 1 : 0);
 }
 
+cudaError_t copy_rows(void *dst, size_t dpitch, const void *src, size_t spitch, size_t width, size_t rows, int on_device,
+                      bool to_device, int device, cudaStream_t st)
+{
+    if (!on_device)
+        return cudaMemcpy2DAsync(dst, dpitch, src, spitch, width, rows,
+                                 to_device ? cudaMemcpyHostToDevice : cudaMemcpyDeviceToHost, st);
+    // memory of this device: the copy kernel; anything else that the caller calls device memory is
+    // left to the runtime's copy, which checks it
+    cudaPointerAttributes at;
+    const cudaError_t e = cudaPointerGetAttributes(&at, to_device ? src : dst);
+    if (e == cudaSuccess && at.type == cudaMemoryTypeDevice && at.device == device)
+        return launch_copy_rows(dst, dpitch, src, spitch, width, rows, st);
+    if (e != cudaSuccess) (void)cudaGetLastError();
+    return cudaMemcpy2DAsync(dst, dpitch, src, spitch, width, rows, cudaMemcpyDeviceToDevice, st);
+}
+
 flood_status copy_in(flood_handle *h, void *dst_pitched, const void *src, int rows, int cols, int src_on_device)
 {
     size_t e = h->esz;
-    CK(cudaMemcpy2DAsync(dst_pitched, (size_t)h->geo.pitch * e, src, (size_t)cols * e, (size_t)cols * e, rows,
-                         src_on_device ? cudaMemcpyDeviceToDevice : cudaMemcpyHostToDevice, h->stream));
+    CK(copy_rows(dst_pitched, (size_t)h->geo.pitch * e, src, (size_t)cols * e, (size_t)cols * e, rows, src_on_device, true,
+                 h->device, h->stream));
     return FLOOD_OK;
 }
 
 flood_status copy_out(flood_handle *h, void *dst, const void *src_pitched, int rows, int cols, int dst_on_device)
 {
     size_t e = h->esz;
-    CK(cudaMemcpy2DAsync(dst, (size_t)cols * e, src_pitched, (size_t)h->geo.pitch * e, (size_t)cols * e, rows,
-                         dst_on_device ? cudaMemcpyDeviceToDevice : cudaMemcpyDeviceToHost, h->stream));
+    CK(copy_rows(dst, (size_t)cols * e, src_pitched, (size_t)h->geo.pitch * e, (size_t)cols * e, rows, dst_on_device, false,
+                 h->device, h->stream));
     return FLOOD_OK;
 }
 

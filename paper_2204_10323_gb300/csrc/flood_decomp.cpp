@@ -345,7 +345,6 @@ extern "C" flood_status flood_decomp_read(flood_decomp *d, int32_t field, void *
     const int rows_all = d->ny + (field == FLOOD_FIELD_QY ? 1 : 0);
     const int cols = d->nx + (field == FLOOD_FIELD_QX ? 1 : 0);
     if (bytes != (size_t)rows_all * cols * d->esz) return dfail(d, FLOOD_ERR_ARG, "dst size does not match the field");
-    const cudaMemcpyKind kind = dst_on_device ? cudaMemcpyDeviceToDevice : cudaMemcpyDeviceToHost;
     for (int r = 0; r < d->n_parts; r++) {
         flood_handle *h = d->parts[r];
         const int y0 = d->rows[4 * r], y1 = d->rows[4 * r + 1], a = d->rows[4 * r + 2];
@@ -353,9 +352,9 @@ extern "C" flood_status flood_decomp_read(flood_decomp *d, int32_t field, void *
         const int n = (y1 - y0) + ((field == FLOOD_FIELD_QY && r == d->n_parts - 1) ? 1 : 0);
         const void *plane = field == FLOOD_FIELD_Z ? h->z : field == FLOOD_FIELD_N ? h->n : field_plane(h, field);
         const size_t pitch_b = (size_t)h->geo.pitch * d->esz;
-        DCK(cudaMemcpy2DAsync((char *)dst + (size_t)y0 * cols * d->esz, (size_t)cols * d->esz,
-                              (const char *)plane + (size_t)(y0 - a) * pitch_b, pitch_b, (size_t)cols * d->esz, n, kind,
-                              d->stream));
+        DCK(copy_rows((char *)dst + (size_t)y0 * cols * d->esz, (size_t)cols * d->esz,
+                      (const char *)plane + (size_t)(y0 - a) * pitch_b, pitch_b, (size_t)cols * d->esz, n, dst_on_device,
+                      false, h->device, d->stream));
     }
     DCK(cudaStreamSynchronize(d->stream));
     return FLOOD_OK;

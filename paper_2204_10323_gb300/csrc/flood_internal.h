@@ -147,6 +147,9 @@ cudaError_t launch_epoch_batched(const EpochArgs<T> *tab, int n, const int2 *tas
 // h_max of a state into ctrl->hmax_bits (max with what is there).
 template <typename T>
 cudaError_t launch_hmax(const Geom &g, const T *h, Ctrl *ctrl, cudaStream_t st);
+// rows of `width` bytes from src to dst (device memory of the current device), pitches in bytes.
+cudaError_t launch_copy_rows(void *dst, size_t dpitch, const void *src, size_t spitch, size_t width, size_t rows,
+                             cudaStream_t st);
 // Block mean (f x f, partial blocks at the far edges) of a ny x nx field into ceil(ny/f) x ceil(nx/f).
 template <typename T>
 cudaError_t launch_coarsen(const T *src, int nx, int ny, int f, T *dst, cudaStream_t st);

@@ -120,6 +120,10 @@ size_t plane_elems(const flood_handle *h, int field);
 void field_shape(const flood_handle *h, int field, int *rows, int *cols);
 flood_status copy_in(flood_handle *h, void *dst_pitched, const void *src, int rows, int cols, int src_on_device);
 flood_status copy_out(flood_handle *h, void *dst, const void *src_pitched, int rows, int cols, int dst_on_device);
+// rows of `width` bytes between two arrays, the caller's on the host or (on_device) the device; to_device:
+// src is the caller's, else dst.
+cudaError_t copy_rows(void *dst, size_t dpitch, const void *src, size_t spitch, size_t width, size_t rows, int on_device,
+                      bool to_device, int device, cudaStream_t st);
 flood_status refresh_hmax(flood_handle *h);
 flood_status launch_inflow_epoch(flood_handle *h);
 flood_status launch_steps(flood_handle *h, int s, int k, int want_hmax, const int64_t *gcells, int ng,
