@@ -24,10 +24,8 @@
 #include <cstddef>
 #include <type_traits>
 
-#include <cuda.h>
-
 #include "fast_face.cuh"
-#include "tma_util.cuh"
+#include "step_tiled.cuh"
 
 namespace flood {
 
@@ -401,40 +399,9 @@ __global__ void __launch_bounds__(BX * TileRows<T>::v) adj_step_kernel(const Adj
 //   dW/dn_j   = (w_j/n_j) / sum_c (pe w_c/hh_c),
 // so dL/dn_j += (w_j/n_j) (sum_c nu_c pe w_c/hh_c / sum_c pe w_c/hh_c - nu_j).
 
-// Adjoint of the unclipped depth of cell (i, j) from global memory: its four new
-// faces, the update and the clip test with the arithmetic of the tile kernels'
-// phases A and B, the gauge seeds in gauge order.
-template <typename T>
-__device__ T cell_lhu(const AdjArgs<T> &A, const Fwd<T> &F, const int i, const int j)
-{
-    const StepArgs<T> &a = A.fwd;
-    const int nx = a.geo.nx, ny = a.geo.ny;
-    const size_t P = (size_t)a.geo.pitch, c = (size_t)j * P + i;
-    const T h = a.h[c], z = a.z[c], n = a.n[c];
-    T qW, qE, qS, qN;
-    if (i == 0) qW = bface(a, F, 0, j, h, n);
-    else qW = F.face(a.qx[c], a.h[c - 1], a.z[c - 1], a.n[c - 1], h, z, n);
-    if (i == nx - 1) qE = bface(a, F, 1, j, h, n);
-    else qE = F.face(a.qx[c + 1], h, z, n, a.h[c + 1], a.z[c + 1], a.n[c + 1]);
-    if (j == 0) qS = bface(a, F, 2, i, h, n);
-    else qS = F.face(a.qy[c], a.h[c - P], a.z[c - P], a.n[c - P], h, z, n);
-    if (j == ny - 1) qN = bface(a, F, 3, i, h, n);
-    else qN = F.face(a.qy[c + P], h, z, n, a.h[c + P], a.z[c + P], a.n[c + P]);
-    const T hu = F.update(h, qW, qE, qS, qN);
-    if (hu < T(0)) return T(0);
-    T v = A.lh[c];
-    const int64_t flat = (int64_t)j * nx + i;
-    for (int gk = 0; gk < A.n_gauges; gk++)
-        if (A.gauge_cells[gk] == flat) v = v + T(A.seed[gk]);
-    return v;
-}
-
-// Section k of pass 3 on the calling block.  kFused: the block runs beside the
-// tiles of the same launch, so it derives each cell's adjoint of the unclipped
-// depth itself (cell_lhu) and adds its dL/dn terms to gn_in (one double per
-// section cell, added to gn after the sweep); otherwise it reads lhu from the
+// Section k of pass 3 on the calling block (FP64 and the scheme options): reads lhu from the
 // finished tiles and adds into gn.
-template <typename T, bool kFused>
+template <typename T>
 __device__ void inflow_adjoint(const AdjArgs<T> &A, const int k, double *red)
 {
     const StepArgs<T> &a = A.fwd;
@@ -447,12 +414,8 @@ __device__ void inflow_adjoint(const AdjArgs<T> &A, const int k, double *red)
     const double pe = G.bc_form == 0 ? 5.0 / 3.0 : 2.0 / 3.0;
     const double inward = (double)inward_sign(S.side);
     const size_t P = (size_t)G.pitch;
-    const Fwd<T> F(G, a.ctrl->dt);
     const int tid = threadIdx.x + blockDim.x * threadIdx.y, nt = blockDim.x * blockDim.y;
-    auto lhu_of = [&](int64_t idx) -> double {
-        if constexpr (kFused) return (double)cell_lhu<T>(A, F, (int)(idx % (int64_t)P), (int)(idx / (int64_t)P));
-        else return (double)A.lhu[idx];
-    };
+    auto lhu_of = [&](int64_t idx) -> double { return (double)A.lhu[idx]; };
     auto lq_of = [&](int64_t idx) -> double {
         switch (S.side) {
         case 0: return (double)A.lqx[idx];
@@ -491,291 +454,548 @@ __device__ void inflow_adjoint(const AdjArgs<T> &A, const int k, double *red)
         if (!(hh > 0.0)) continue;
         const double w = (double)a.inflow_q[(size_t)a.s * a.n_slots + S.slot0 + c] * dx;
         const double nu = c == tid ? nu0 : inward * (lq_of(idx) + inward * dtdx * lhu_of(idx)) / dx;
-        const double term = (w / (double)a.n[idx]) * (Nn / D - nu);
-        if constexpr (kFused) A.gn_in[S.cell0 + c] += term;
-        else A.gn[idx] += term;
+        A.gn[idx] += (w / (double)a.n[idx]) * (Nn / D - nu);
     }
-}
-
-// The fused form's entry, kept out of line: its double-precision section sums
-// would otherwise raise the register count of the tile kernel that calls it.
-__device__ __noinline__ void inflow_adjoint_fused(const AdjArgs<float> &A, const int k, double *red)
-{
-    inflow_adjoint<float, true>(A, k, red);
 }
 
 template <typename T>
 __global__ void adj_inflow_kernel(const AdjArgs<T> A)
 {
     __shared__ double red[32];
-    inflow_adjoint<T, false>(A, blockIdx.x, red);
+    inflow_adjoint<T>(A, blockIdx.x, red);
 }
 
-// The FP32 reverse step with its inputs staged by the tensor-memory accelerator:
-// one thread issues eight 2D tensor copies (the forward state h, z, n, qx, qy and
-// the adjoint after the step lh, lqx, lqy, each box with its halo, zeros outside
-// the grid) onto one mbarrier, so the tile's staging costs no per-element index
-// arithmetic or load latency in the threads; phases A-D are those of
-// adj_step_kernel.  Staged rows start at column I0 - 4 (16-byte aligned) and
-// are kAW = 40 wide.
-struct AdjMaps {
-    CUtensorMap m[8];            // h, z, n, qx, qy, lh, lqx, lqy
-};
-enum { kMh = 0, kMz, kMn, kMqx, kMqy, kMlh, kMlqx, kMlqy };
-constexpr int kAW = 40;
-// A tensor copy's shared-memory destination must be 128-byte aligned: every box
-// starts on its own 128-byte boundary.  TB: rows of the tile.
-template <int TB>
-struct alignas(128) AdjStage {
-    alignas(128) float h[TB + 4][kAW];      // cells: rows J0-2 .., columns I0-4 ..
-    alignas(128) float z[TB + 4][kAW];
-    alignas(128) float n[TB + 4][kAW];
-    alignas(128) float qx[TB + 2][kAW];     // x-faces: rows J0-1 .., face columns I0-4 ..
-    alignas(128) float qy[TB + 3][kAW];     // y-faces: face rows J0-1 .., columns I0-4 ..
-    alignas(128) float lh[TB + 2][kAW];     // lambda_h': rows J0-1 .., columns I0-4 ..
-    alignas(128) float lqx[TB][kAW];        // lambda_qx': rows J0 .., face columns I0 ..
-    alignas(128) float lqy[TB + 1][BX];     // lambda_qy': face rows J0 .., columns I0 ..
-    uint64_t bar;
-};
-template <int TB>
-__host__ __device__ constexpr bool adj_stage_aligned()
-{
-    using S = AdjStage<TB>;
-    return offsetof(S, z) % 128 == 0 && offsetof(S, n) % 128 == 0 && offsetof(S, qx) % 128 == 0 &&
-           offsetof(S, qy) % 128 == 0 && offsetof(S, lh) % 128 == 0 && offsetof(S, lqx) % 128 == 0 &&
-           offsetof(S, lqy) % 128 == 0 && offsetof(S, bar) % 8 == 0;
-}
-static_assert(adj_stage_aligned<8>() && adj_stage_aligned<16>(), "tensor-copy destinations must be 128-byte aligned");
-// bytes the eight boxes deliver (the barrier's transaction count)
-template <int TB>
-__host__ __device__ constexpr uint32_t adj_bytes()
-{
-    return (uint32_t)sizeof(float) *
-           (3 * (TB + 4) * kAW + (TB + 2) * kAW + (TB + 3) * kAW + (TB + 2) * kAW + TB * kAW + (TB + 1) * BX);
-}
-// rows of the FP32 reverse step's tile, and its blocks per SM at 40 registers
-constexpr int kAdjTB = 8;
-constexpr uint64_t kAdjBudgetNs = 2000000000ull;
+// ---------------------------------------------------------------- FP32, Eq. 3 as printed
+// The FP32 reverse step: one warp walks the rows of a strip of 120 output columns (128 staged,
+// four per lane) south to north, as the temporal-blocking kernel does, in one pass.  At tick j:
+//  A. row j's new faces (the forward arithmetic) and, from the same intermediates, each face's
+//     derivatives with respect to its old discharge, its two depths and n; kept one tick;
+//  B. the adjoint lu of row j-1's unclipped depth: its update needs the south faces of row j;
+//  C. the x-faces of row j-1 and the y-faces between rows j-2 and j-1: mu, and its products with
+//     the kept derivatives;
+//  D. row j-2 is complete: its lambda_h and dL/dn.
+// A border face keeps the derivatives of Eq. 5 in the same places (its outer cell has lu = 0), so
+// that C and D know no borders; an inflow face leaves lu and lambda_q for pass 3.  Rows arrive by
+// asynchronous copies, every lane's shared memory is its own: no barrier, no index arithmetic per
+// element.
+//
+// At 1024^2 (20.2 us, 11 warps per SM) a lone warp's chain bounds it: a tick of 550 instructions takes
+// some 2300 cycles by itself, 3000 beside two others, and an item of six rows runs nine.  Eight warps per
+// SM without spills: 22.2 us; the derivatives kept in shared memory: 20.7.  A tile kernel (32 x 8 cells staged
+// by tensor copies, flat loops over the staged arrays between block barriers) executed 647 thread
+// instructions per cell, 285 of them integer, and took 28.8 us.
 
-template <int TB>
-__global__ void __launch_bounds__(BX * TB, TB == 8 ? 6 : 3) adj_step_tma_kernel(const AdjArgs<float> A, const int nbx,
-                                                                 const int n_tiles,
-                                                                 const __grid_constant__ AdjMaps maps)
+struct alignas(16) AdjSmem {
+    float raw[kAhead][8][128];           // rows in flight: h, z, n, qx, qy of row j; lambda_h, lambda_qx, lambda_qy of row j - 1
+    double gn[kAhead][128];              // dL/dn of row j - 2
+    int gauge[32][3];                    // gauges in the staged cells, in gauge order: row, column, index
+};
+
+// The derivatives of a row's faces.
+struct FaceRow {
+    Row4 q, L, R, n;                     // with respect to the old discharge, the depths of the two cells, n of either
+};
+
+__device__ __forceinline__ unsigned long long f2sel(bool x, bool y, unsigned long long a, unsigned long long b)
 {
-    using T = float;
-    const int n_sec = (int)gridDim.x - n_tiles;
-    if ((int)blockIdx.x < n_sec) {                   // the first blocks: pass 3, one section each, beside the tiles
-        __shared__ double red_in[32];
-        inflow_adjoint_fused(A, (int)blockIdx.x, red_in);
-        return;
+    const float2 u = f2unpack(a), v = f2unpack(b);
+    return f2pack(x ? u.x : v.x, y ? u.y : v.y);
+}
+
+__device__ __forceinline__ unsigned long long f2rcp(unsigned long long a)
+{
+    const float2 v = f2unpack(a);
+    return f2pack(rcp_fast(v.x), rcp_fast(v.y));
+}
+
+// Eq. 3 for two faces (the operations of face_fast_sel_x2, in its order), with what its derivatives
+// need.  A dry face is evaluated at depth 1 with a zero reciprocal of its denominator, which makes
+// its value and its derivatives zero.
+struct Faces2 {
+    unsigned long long hs, slope, q, nsum, cr, cq, m, inv, F;   // depth, eta_R - eta_L, old q, n_L + n_R, c r7, c |q| r7,
+                                                                // -a1 hs, 1 / den, the new value
+};
+
+__device__ __forceinline__ Faces2 faces2_value(unsigned long long hf, unsigned long long slope, unsigned long long q,
+                                               unsigned long long nsum, const FastConst &k)
+{
+    Faces2 f;
+    const float2 h0 = f2unpack(hf);
+    const bool w0 = h0.x > k.h_dry, w1 = h0.y > k.h_dry;
+    const float2 h = make_float2(w0 ? h0.x : 1.0f, w1 ? h0.y : 1.0f);
+    f.hs = f2pack(h.x, h.y);
+    f.slope = slope;
+    f.q = q;
+    f.nsum = nsum;
+    const float2 l = f2unpack(f2mul(f2pack(lg2_fast(h.x), lg2_fast(h.y)), f2dup(-7.0f / 3.0f)));
+    const unsigned long long r7 = f2pack(ex2_fast(l.x), ex2_fast(l.y));
+    const unsigned long long c = face_c(nsum, k), cq = face_cq(c, q);
+    f.m = f2mul(f2dup(-k.a1), f.hs);
+    const float2 rd = f2unpack(f2rcp(f2fma(cq, r7, f2dup(1.0f))));
+    f.inv = f2pack(w0 ? rd.x : 0.0f, w1 ? rd.y : 0.0f);
+    f.F = f2mul(f2fma(f.m, slope, q), f.inv);
+    f.cr = f2mul(c, r7);
+    f.cq = f2mul(cq, r7);
+    return f;
+}
+
+// face_lin's formulas.
+__device__ __forceinline__ void faces2_lin(const Faces2 &f, const FastConst &k, unsigned long long &dq, unsigned long long &dL,
+                                           unsigned long long &dR, unsigned long long &dn)
+{
+    // dF/dq = (1 - F c r7 sign(q)) / den, sign(0) = 0
+    const float2 qv = f2unpack(f.q), t = f2unpack(f2mul(f.F, f.cr));
+    const float t0 = qv.x != 0.0f ? __uint_as_float(__float_as_uint(t.x) ^ (__float_as_uint(qv.x) & 0x80000000u)) : 0.0f;
+    const float t1 = qv.y != 0.0f ? __uint_as_float(__float_as_uint(t.y) ^ (__float_as_uint(qv.y) & 0x80000000u)) : 0.0f;
+    dq = f2mul(f2sub(f2dup(1.0f), f2pack(t0, t1)), f.inv);
+    // dF/dhf, and the explicit dependence on the water levels; max sends hf's part to L on ties
+    const unsigned long long Ff = f2mul(f.F, f.cq);
+    const unsigned long long dh = f2mul(f2fma(f2mul(Ff, f2dup(7.0f / 3.0f)), f2rcp(f.hs), f2mul(f2dup(-k.a1), f.slope)), f.inv);
+    const unsigned long long ex = f2mul(f.m, f.inv);              // minus a1 hf / den
+    const float2 sv = f2unpack(f.slope);
+    const bool l0 = sv.x <= 0.0f, l1 = sv.y <= 0.0f;
+    dL = f2sub(f2sel(l0, l1, dh, 0ull), ex);
+    dR = f2add(f2sel(l0, l1, 0ull, dh), ex);
+    dn = f2mul(f2mul(Ff, f.inv), f2mul(f2dup(-2.0f), f2rcp(f.nsum)));
+}
+
+// A border face of Eq. 5 as a face between the cell (depth h, n) and an outer cell that does not
+// exist: its value, and its derivatives with respect to the depth and n of the cell.
+__device__ __forceinline__ float border_lin(int type, float inward, float h, float sqrtS, float n, const Geom &G, float inflow,
+                                            float &dh, float &dn)
+{
+    dh = dn = 0.0f;
+    if (type == kBcWall) return 0.0f;
+    if (type == kBcInflow) return inward * inflow;
+    const float q = outflow_fast(h, sqrtS, n, G.dx_f, G.h_dry_f, G.bc_form);
+    if (q > 0.0f) {
+        dh = __fdividef(-inward * (G.bc_form == 0 ? 5.0f / 3.0f : 2.0f / 3.0f) * q, h);
+        dn = __fdividef(inward * q, n);
     }
-    const int tile = (int)blockIdx.x - n_sec;
-    __shared__ AdjStage<TB> S;
-    __shared__ T sX[TB + 2][BX + 3];   // new x-faces: rows J0-1 .., face columns I0-1 ..
-    __shared__ T sY[TB + 3][BX + 2];   // new y-faces: face rows J0-1 .., columns I0-1 ..
-    __shared__ T sL[TB + 2][BX + 2];   // cells I0-1 .., J0-1 ..
-    __shared__ T cXl[TB][BX + 1], cXr[TB][BX + 1], cXn[TB][BX + 1];
-    __shared__ T cYl[TB + 1][BX], cYr[TB + 1][BX], cYn[TB + 1][BX];
-    __shared__ int s_ng, s_gk[kTileGauges];
-    const StepArgs<T> &a = A.fwd;
+    return -inward * q;
+}
+
+__device__ __forceinline__ void row_set(Row4 &v, int k, float x)
+{
+    const float2 a = f2unpack(v.a), b = f2unpack(v.b);
+    v = row_pack(k == 0 ? x : a.x, k == 1 ? x : a.y, k == 2 ? x : b.x, k == 3 ? x : b.y);
+}
+
+__device__ __forceinline__ Row4 row_add(const Row4 &x, const Row4 &y) { return Row4{f2add(x.a, y.a), f2add(x.b, y.b)}; }
+__device__ __forceinline__ Row4 row_mul(const Row4 &x, const Row4 &y) { return Row4{f2mul(x.a, y.a), f2mul(x.b, y.b)}; }
+
+__device__ __forceinline__ void adj_rows_item(const AdjArgs<float> &A, const int strip, const int y0, const int y1, AdjSmem &sm)
+{
+    constexpr int kOut = out_cols(2);
+    const StepArgs<float> &a = A.fwd;
     const Geom &G = a.geo;
+    const int lane = threadIdx.x;
     const int nx = G.nx, ny = G.ny;
     const size_t P = (size_t)G.pitch;
-    const double dtd = a.ctrl->dt;
-    const Fwd<T> F(G, dtd);
-    const T dt = T(dtd), dx = T(G.dx), g = T(G.g), hd = T(G.h_dry), dtdx = dt / dx;
-    const int tid = threadIdx.y * BX + threadIdx.x;
-    const int I0 = (tile % nbx) * BX, J0 = (tile / nbx) * TB;
+    const Fwd<float> FW(G, a.ctrl->dt);
+    const FastConst Kc = FW.K;
+    const int x0 = strip * kOut - 4;
+    const int c0 = x0 + 4 * lane;
+    const int own_lo = strip * kOut, own_hi = min(own_lo + kOut, nx);
+    const bool west = x0 < 0, east = x0 + 127 >= nx;
+    const bool in = c0 >= 0 && c0 < (int)P;
+    const int jb = max(y0 - 2, 0);
+    const int jhi = min(y1 + 1, ny - 1);               // last row of the state
+    const int jlast = y1 + 1;                          // last tick: row y1 - 1 is completed
+    const int steady_lo = jb > 0 ? jb : 2, steady_hi = nx >= 4 ? jhi : -1;
+    const bool full = c0 >= own_lo && c0 + 3 < own_hi;
+    const bool part = !full && c0 >= own_lo && (c0 < own_hi || (c0 == nx && own_hi == nx));
+    // the border face at x = 0 or x = nx in this lane's columns (with nx < 4 a lane can hold both, and every
+    // tick takes the general form); its type, inflow slot and sqrt(S) are read a tick ahead
+    const bool lane_w = west && c0 == 0, lane_e = east && nx - c0 >= 0 && nx - c0 < 4;
+    const int side = lane_e ? 1 : 0, kb = lane_e ? nx - c0 : lane_w ? 0 : -1;
+    int nb_t = kBcWall, nb_s = 0, pb_t = kBcWall, pb_s = 0;
+    float nb_q = 0.0f;
+    auto border_fetch = [&](int r) {
+        if (kb >= 0 && r <= jhi) {
+            nb_t = a.bc.type[(side ? ny : 0) + r];
+            nb_s = a.bc.slot[(side ? ny : 0) + r];
+            nb_q = a.bc.sqrtS_f[(side ? ny : 0) + r];
+        }
+    };
+    border_fetch(jb);
+    const size_t lane_off = in ? (size_t)c0 : 0;
 
-    // 0. the eight boxes onto one barrier; the gauge list is built meanwhile
-    if (tid == 0) {
-        mbar_init(&S.bar, 1);
-        fence_mbar_init();
-        s_ng = 0;
-        mbar_arrive_expect_tx(&S.bar, adj_bytes<TB>());
-        tma_load_2d(&S.h[0][0], &maps.m[kMh], I0 - 4, J0 - 2, &S.bar);
-        tma_load_2d(&S.z[0][0], &maps.m[kMz], I0 - 4, J0 - 2, &S.bar);
-        tma_load_2d(&S.n[0][0], &maps.m[kMn], I0 - 4, J0 - 2, &S.bar);
-        tma_load_2d(&S.qx[0][0], &maps.m[kMqx], I0 - 4, J0 - 1, &S.bar);
-        tma_load_2d(&S.qy[0][0], &maps.m[kMqy], I0 - 4, J0 - 1, &S.bar);
-        tma_load_2d(&S.lh[0][0], &maps.m[kMlh], I0 - 4, J0 - 1, &S.bar);
-        tma_load_2d(&S.lqx[0][0], &maps.m[kMlqx], I0, J0, &S.bar);
-        tma_load_2d(&S.lqy[0][0], &maps.m[kMlqy], I0, J0, &S.bar);
-    }
-    __syncthreads();
-    // B prelude: the gauges inside the tile and its halo, in gauge order (repeated
-    // gauges add up in order); a tile holding more than kTileGauges scans them all
-    for (int gk = tid; gk < A.n_gauges; gk += BX * TB) {
-        const int64_t flat = A.gauge_cells[gk];
-        const int gj = (int)(flat / nx), gi = (int)(flat - (int64_t)gj * nx);
-        if (gj >= J0 - 1 && gj <= J0 + TB && gi >= I0 - 1 && gi <= I0 + BX) {
-            const int slot = atomicAdd(&s_ng, 1);
-            if (slot < kTileGauges) s_gk[slot] = gk;
+    auto issue = [&](int j) {
+        float *d = &sm.raw[j & (kAhead - 1)][0][4 * lane];
+        if (j <= jhi) {
+            const size_t o = (size_t)j * P + lane_off;
+            copy16(d, a.h + o, in);
+            copy16(d + 128, a.z + o, in);
+            copy16(d + 256, a.n + o, in);
+            copy16(d + 384, a.qx + o, in);
+            copy16(d + 512, a.qy + o, in);
         }
-    }
-    const bool ok = mbar_wait_bounded(&S.bar, 0u, kAdjBudgetNs);
-    if (!__syncthreads_and(ok ? 1 : 0)) {
-        if (tid == 0) {
-            atomicOr(&a.ctrl->status, kStatusTimeout);
-            mbar_wait_bounded(&S.bar, 0u, kAdjBudgetNs);   // no copy may land after the block is gone
-        }
-        return;
-    }
-    if (tid == 0 && s_ng > 1 && s_ng <= kTileGauges) {
-        for (int x = 1; x < s_ng; x++)
-            for (int y = x; y > 0 && s_gk[y - 1] > s_gk[y]; y--) {
-                const int tmp = s_gk[y];
-                s_gk[y] = s_gk[y - 1];
-                s_gk[y - 1] = tmp;
+        if (j >= 1 && j <= jlast) {                    // face row ny has lambda_qy only
+            const size_t o = (size_t)(j - 1) * P + lane_off;
+            if (j - 1 < ny) {
+                copy16(d + 640, A.lh + o, in);
+                copy16(d + 768, A.lqx + o, in);
             }
-    }
-    // A. new face values.  x-face (lj, li): row J0-1+lj, face column fi = I0-1+li, between
-    // cells at staged columns li+2 (L) and li+3 (R) of staged row lj+1.
-    for (int t = tid; t < (TB + 2) * (BX + 3); t += BX * TB) {
-        const int lj = t / (BX + 3), li = t % (BX + 3);
-        const int j = J0 - 1 + lj, fi = I0 - 1 + li;
-        T v = T(0);
-        if (j >= 0 && j < ny && fi >= 0 && fi <= nx) {
-            const int sj = lj + 1, sl = li + 2, sr = li + 3;
-            if (fi == 0) v = bface(a, F, 0, j, S.h[sj][sr], S.n[sj][sr]);
-            else if (fi == nx) v = bface(a, F, 1, j, S.h[sj][sl], S.n[sj][sl]);
-            else
-                v = F.face(S.qx[lj][li + 3], S.h[sj][sl], S.z[sj][sl], S.n[sj][sl], S.h[sj][sr], S.z[sj][sr],
-                           S.n[sj][sr]);
+            copy16(d + 896, A.lqy + o, in);
         }
-        sX[lj][li] = v;
-    }
-    // y-face (lj, li): face row fj = J0-1+lj, column i = I0-1+li, between cells of
-    // staged rows lj (below) and lj+1 (above) at staged column li+3.
-    for (int t = tid; t < (TB + 3) * (BX + 2); t += BX * TB) {
-        const int lj = t / (BX + 2), li = t % (BX + 2);
-        const int fj = J0 - 1 + lj, i = I0 - 1 + li;
-        T v = T(0);
-        if (i >= 0 && i < nx && fj >= 0 && fj <= ny) {
-            const int sc = li + 3, sb = lj, st = lj + 1;
-            if (fj == 0) v = bface(a, F, 2, i, S.h[st][sc], S.n[st][sc]);
-            else if (fj == ny) v = bface(a, F, 3, i, S.h[sb][sc], S.n[sb][sc]);
-            else
-                v = F.face(S.qy[lj][li + 3], S.h[sb][sc], S.z[sb][sc], S.n[sb][sc], S.h[st][sc], S.z[st][sc],
-                           S.n[st][sc]);
+        if (j - 2 >= y0 && j - 2 < y1) {
+            const double *g = A.gn + (size_t)(j - 2) * P + lane_off;
+            copy16(reinterpret_cast<float *>(&sm.gn[j & (kAhead - 1)][4 * lane]), reinterpret_cast<const float *>(g), in);
+            copy16(reinterpret_cast<float *>(&sm.gn[j & (kAhead - 1)][4 * lane + 2]), reinterpret_cast<const float *>(g + 2), in);
         }
-        sY[lj][li] = v;
+        copy_commit();
+    };
+    for (int j = jb; j < jb + kAhead; j++) issue(j);
+
+    // the gauges in the staged cells, in gauge order (repeated gauges add up in order); an item with more
+    // than 32 scans them all at every row
+    int ng = 0;
+    for (int g0 = 0; g0 < A.n_gauges; g0 += 32) {
+        int gi = -1, gj = -1;
+        if (g0 + lane < A.n_gauges) {
+            const int2 rc = A.gauge_rc[g0 + lane];
+            gj = rc.x;
+            gi = rc.y;
+        }
+        const bool mine = gj >= jb && gj <= jhi && gi >= x0 && gi < x0 + 128;
+        const unsigned m = __ballot_sync(0xffffffffu, mine);
+        const int slot = ng + __popc(m & ((1u << lane) - 1));
+        if (mine && slot < 32) {
+            sm.gauge[slot][0] = gj;
+            sm.gauge[slot][1] = gi - x0;
+            sm.gauge[slot][2] = g0 + lane;
+        }
+        ng += __popc(m);
     }
-    __syncthreads();
-    // B. adjoint of the unclipped depth (gauge seeds included)
-    const int ng_tile = s_ng;
-    for (int t = tid; t < (TB + 2) * (BX + 2); t += BX * TB) {
-        const int lj = t / (BX + 2), li = t % (BX + 2);
-        const int j = J0 - 1 + lj, i = I0 - 1 + li;
-        T v = T(0);
-        if (i >= 0 && i < nx && j >= 0 && j < ny) {
-            const T hu = F.update(S.h[lj + 1][li + 3], sX[lj][li], sX[lj][li + 1], sY[lj][li], sY[lj + 1][li]);
-            if (!(hu < T(0))) {
-                v = S.lh[lj][li + 3];
-                if (ng_tile > 0) {
-                    const int64_t flat = (int64_t)j * nx + i;
-                    if (ng_tile <= kTileGauges) {
-                        for (int x = 0; x < ng_tile; x++)
-                            if (A.gauge_cells[s_gk[x]] == flat) v = v + T(A.seed[s_gk[x]]);
+    __syncwarp();
+
+    Row4 hp{0, 0}, zp{0, 0}, np_{0, 0};                // row j - 1: depth, bed, n
+    Row4 xp{0, 0}, yp{0, 0};                           // its new faces
+    FaceRow dx{}, dy{};                                // and their derivatives
+    Row4 lu2{0, 0}, acc2{0, 0}, gx2{0, 0}, gy2{0, 0};  // row j - 2: lu, and its sums so far
+
+    auto tick = [&](auto steady_t, auto edge_t, const int j) {
+        constexpr bool kSteady = decltype(steady_t)::value, kEdge = decltype(edge_t)::value;
+        const bool row = kSteady || j < ny, rowp = kSteady || (j >= 1 && j <= ny);   // rows j and j - 1 are cells
+        copy_wait<kAhead - 1>();
+        const float *d = &sm.raw[j & (kAhead - 1)][0][4 * lane];
+        const Row4 lq = row_load(d + 768), lqy = row_load(d + 896);
+        Row4 lu = row_load(d + 640);
+        double2 g01 = *reinterpret_cast<const double2 *>(&sm.gn[j & (kAhead - 1)][4 * lane]);
+        double2 g23 = *reinterpret_cast<const double2 *>(&sm.gn[j & (kAhead - 1)][4 * lane + 2]);
+        Row4 ch{0, 0}, cz{0, 0}, cn{0, 0}, cx{0, 0}, cy{0, 0};
+        if (row) {
+            ch = row_load(d);
+            cz = row_load(d + 128);
+            cn = row_load(d + 256);
+            cx = row_load(d + 384);
+            cy = row_load(d + 512);
+        }
+        issue(j + kAhead);
+        // ---- A. the new south faces of row j (their derivatives, and the west faces, after C has used
+        // those of row j - 1: they take the same registers)
+        const Row4 e = row_add(ch, cz);
+        const bool inner = kSteady || (j > 0 && j < ny);
+        Row4 qy{0, 0}, bR{0, 0}, bL{0, 0}, bn{0, 0};
+        Faces2 ya, yb;
+        if (inner) {
+            const Row4 ep = row_add(hp, zp);
+            ya = faces2_value(f2sub(f2max(ep.a, e.a), f2max(zp.a, cz.a)), f2sub(e.a, ep.a), cy.a, f2add(np_.a, cn.a), Kc);
+            yb = faces2_value(f2sub(f2max(ep.b, e.b), f2max(zp.b, cz.b)), f2sub(e.b, ep.b), cy.b, f2add(np_.b, cn.b), Kc);
+            qy = Row4{ya.F, yb.F};
+        } else if (j == 0 || j == ny) {
+            const int off = j == 0 ? 2 * ny : 2 * ny + nx;
+            const Row4 hb = j == 0 ? ch : hp, nb = j == 0 ? cn : np_;
+#pragma unroll 1
+            for (int k = 0; k < 4; k++) {
+                const int c = c0 + k;
+                if (c < 0 || c >= nx) continue;
+                const int t = a.bc.type[off + c];
+                float dh, dn;
+                const float v = border_lin(t, j == 0 ? 1.0f : -1.0f, row_get(hb, k), a.bc.sqrtS_f[off + c], row_get(nb, k), G,
+                                           t == kBcInflow ? a.inflow_q[(size_t)a.s * a.n_slots + a.bc.slot[off + c]] : 0.0f,
+                                           dh, dn);
+                row_set(qy, k, v);
+                if (j == 0) row_set(bR, k, dh);
+                else row_set(bL, k, dh);
+                row_set(bn, k, dn);
+            }
+        }
+        // ---- B. the adjoint of row j - 1's unclipped depth (tick y0 - 1 only readies row y0 - 1's faces)
+        const bool sums = !kSteady || j >= y0;
+        if (sums) {
+        if (rowp) {
+            const float2 x01 = f2unpack(xp.a), x23 = f2unpack(xp.b);
+            const float xe = from_right(xp);
+            const unsigned long long d0 = f2add(f2pack(__fsub_rn(x01.x, x01.y), __fsub_rn(x01.y, x23.x)), f2sub(yp.a, qy.a));
+            const unsigned long long d1 = f2add(f2pack(__fsub_rn(x23.x, x23.y), __fsub_rn(x23.y, xe)), f2sub(yp.b, qy.b));
+            const float2 u0 = f2unpack(f2fma(f2dup(Kc.dtdx), d0, hp.a)), u1 = f2unpack(f2fma(f2dup(Kc.dtdx), d1, hp.b));
+            const float u[4] = {u0.x, u0.y, u1.x, u1.y};
+            float v[4] = {row_get(lu, 0), row_get(lu, 1), row_get(lu, 2), row_get(lu, 3)};
+            if (ng > 0) {
+                const int n_scan = ng <= 32 ? ng : A.n_gauges;
+                for (int x = 0; x < n_scan; x++) {
+                    int gj, gc, gk = x;
+                    if (ng <= 32) {
+                        gj = sm.gauge[x][0];
+                        gc = sm.gauge[x][1];
+                        gk = sm.gauge[x][2];
                     } else {
-                        for (int gk = 0; gk < A.n_gauges; gk++)
-                            if (A.gauge_cells[gk] == flat) v = v + T(A.seed[gk]);
+                        gj = A.gauge_rc[x].x;
+                        gc = A.gauge_rc[x].y - x0;
+                    }
+                    if (gj != j - 1) continue;
+                    const float sd = (float)A.seed[gk];
+#pragma unroll
+                    for (int k = 0; k < 4; k++)
+                        if (gc == 4 * lane + k) v[k] = v[k] + sd;
+                }
+            }
+#pragma unroll
+            for (int k = 0; k < 4; k++) {
+                if (u[k] < 0.0f) v[k] = 0.0f;
+                if (kEdge && (c0 + k < 0 || c0 + k >= nx)) v[k] = 0.0f;
+            }
+            lu = row_pack(v[0], v[1], v[2], v[3]);
+        } else {
+            lu = Row4{0, 0};
+        }
+        // ---- C. the x-faces of row j - 1 and the y-faces below it
+        const float lul = from_left(lu);
+        const float2 a0 = f2unpack(lu.a), a1 = f2unpack(lu.b);
+        const unsigned long long dl0 = f2pack(__fsub_rn(a0.x, lul), __fsub_rn(a0.y, a0.x));
+        const unsigned long long dl1 = f2pack(__fsub_rn(a1.x, a0.y), __fsub_rn(a1.y, a1.x));
+        const Row4 mux{f2fma(f2dup(Kc.dtdx), dl0, lq.a), f2fma(f2dup(Kc.dtdx), dl1, lq.b)};
+        const Row4 muy{f2fma(f2dup(Kc.dtdx), f2sub(lu.a, lu2.a), lqy.a), f2fma(f2dup(Kc.dtdx), f2sub(lu.b, lu2.b), lqy.b)};
+        const Row4 xL = row_mul(mux, dx.L), xR = row_mul(mux, dx.R), xn = row_mul(mux, dx.n), xq = row_mul(mux, dx.q);
+        const Row4 yL = row_mul(muy, dy.L), yR = row_mul(muy, dy.R), yn = row_mul(muy, dy.n), yq = row_mul(muy, dy.q);
+        // ---- D. row j - 2 is complete
+        if (j - 2 >= y0 && j - 2 < y1) {
+            const Row4 out = row_add(acc2, yL), gs = row_add(gx2, row_add(gy2, yn));
+            const float2 s0 = f2unpack(gs.a), s1 = f2unpack(gs.b);
+            const size_t o = (size_t)(j - 2) * P + lane_off;
+            g01.x += (double)s0.x;
+            g01.y += (double)s0.y;
+            g23.x += (double)s1.x;
+            g23.y += (double)s1.y;
+            if (kEdge ? full : lane >= 1 && lane <= kOut / 4) {
+                row_store(A.lh_out + o, out);
+                *reinterpret_cast<double2 *>(A.gn + o) = g01;
+                *reinterpret_cast<double2 *>(A.gn + o + 2) = g23;
+            } else if (kEdge && part) {
+                const double g[4] = {g01.x, g01.y, g23.x, g23.y};
+#pragma unroll
+                for (int k = 0; k < 4; k++)
+                    if (c0 + k < own_hi) {
+                        A.lh_out[o + k] = row_get(out, k);
+                        A.gn[o + k] = g[k];
+                    }
+            }
+        }
+        // the adjoint of the old faces of row j - 1 (and of the grid's north faces, face row ny)
+        const int r = j - 1;
+        if (r >= y0 && (r < y1 || (r == ny && y1 == ny))) {
+            const size_t o = (size_t)r * P + lane_off;
+            const bool cells = r < ny;
+            if (kEdge ? full : lane >= 1 && lane <= kOut / 4) {
+                if (cells) row_store(A.lqx_out + o, xq);
+                row_store(A.lqy_out + o, yq);
+            } else if (kEdge && part) {
+#pragma unroll
+                for (int k = 0; k < 4; k++) {
+                    const int c = c0 + k;
+                    if (cells && (c < own_hi || c == nx)) A.lqx_out[o + k] = row_get(xq, k);
+                    if (c < own_hi) A.lqy_out[o + k] = row_get(yq, k);
+                }
+            }
+            // inflow faces: lu of the cell and lambda_q of the face, for pass 3
+            if (A.in_log) {
+                if (kEdge && cells && (west || east)) {
+                    const int kf = side ? nx - c0 : 0;
+                    if (kb >= 0 && pb_t == kBcInflow && (side ? own_hi == nx : own_lo == 0))
+                        A.in_log[pb_s] = make_float2(side ? (kf == 0 ? lul : row_get(lu, kf - 1)) : a0.x, row_get(lq, kf));
+                    if (!kSteady && lane_w && lane_e && a.bc.type[r] == kBcInflow)     // nx < 4: the west face too
+                        A.in_log[a.bc.slot[r]] = make_float2(a0.x, row_get(lq, 0));
+                }
+                if (!kSteady && (r == 0 || r == ny)) {
+                    const int off = r == 0 ? 2 * ny : 2 * ny + nx;
+                    const Row4 lb = r == 0 ? lu : lu2;
+#pragma unroll
+                    for (int k = 0; k < 4; k++) {
+                        const int c = c0 + k;
+                        if (c >= own_lo && c < own_hi && a.bc.type[off + c] == kBcInflow)
+                            A.in_log[a.bc.slot[off + c]] = make_float2(row_get(lb, k), row_get(lqy, k));
                     }
                 }
             }
         }
-        sL[lj][li] = v;
-    }
-    __syncthreads();
-    // C. each face touching the tile once.  x-face (lj, li): row J0+lj, face column
-    // fi = I0+li; cells at staged columns li+3 (L) and li+4 (R) of staged row lj+2.
-    for (int t = tid; t < TB * (BX + 1); t += BX * TB) {
-        const int lj = t / (BX + 1), li = t % (BX + 1);
-        const int j = J0 + lj, fi = I0 + li;
-        T cl = T(0), cr = T(0), cn = T(0);
-        if (j < ny && fi <= nx) {
-            const size_t r = (size_t)j * P;
-            const T lR = sL[lj + 1][li + 1], lL = sL[lj + 1][li];
-            const int sj = lj + 2, sl = li + 3, sr = li + 4;
-            if (fi == 0) {
-                const T mu = S.lqx[lj][li] + dtdx * lR;
-                outflow_adj(a, F, 0, j, S.h[sj][sr], S.n[sj][sr], mu, cr, cn);
-                A.lqx_out[r] = T(0);
-            } else if (fi == nx) {
-                const T mu = S.lqx[lj][li] - dtdx * lL;
-                outflow_adj(a, F, 1, j, S.h[sj][sl], S.n[sj][sl], mu, cl, cn);
-                A.lqx_out[r + nx] = T(0);
-            } else {
-                const T mu = S.lqx[lj][li] + dtdx * (lR - lL);
-                const T hL = S.h[sj][sl], zL = S.z[sj][sl], nL = S.n[sj][sl];
-                const T hR = S.h[sj][sr], zR = S.z[sj][sr], nR = S.n[sj][sr];
-                const T hf = F.hf(hL, zL, hR, zR);
-                T lq = T(0);
-                if (hf > hd && mu != T(0)) {
-                    FaceLin<T> d = face_lin<T>(S.qx[lj + 1][li + 4], hL, zL, nL, hR, zR, nR, hf, g, dt, dx);
-                    cl = mu * d.dhL;
-                    cr = mu * d.dhR;
-                    cn = mu * d.dn;
-                    lq = mu * d.dq;
-                }
-                if (li < BX) A.lqx_out[r + fi] = lq;        // the tile owns the west faces of its cells
-            }
+        // ---- the rows move on
+        acc2 = row_add(row_add(row_add(lu, xR), row_right(xL, from_right(xL))), yR);
+        gx2 = row_add(xn, row_right(xn, from_right(xn)));
+        gy2 = yn;
+        lu2 = lu;
         }
-        cXl[lj][li] = cl;
-        cXr[lj][li] = cr;
-        cXn[lj][li] = cn;
-    }
-    // y-face (lj, li): face row fj = J0+lj, column i = I0+li; cells of staged rows
-    // lj+1 (below) and lj+2 (above) at staged column li+4.
-    for (int t = tid; t < (TB + 1) * BX; t += BX * TB) {
-        const int lj = t / BX, li = t % BX;
-        const int fj = J0 + lj, i = I0 + li;
-        T cl = T(0), cr = T(0), cn = T(0);
-        if (i < nx && fj <= ny) {
-            const T lR = sL[lj + 1][li + 1], lL = sL[lj][li + 1];
-            const int sc = li + 4, sb = lj + 1, st = lj + 2;
-            if (fj == 0) {
-                const T mu = S.lqy[lj][li] + dtdx * lR;
-                outflow_adj(a, F, 2, i, S.h[st][sc], S.n[st][sc], mu, cr, cn);
-                A.lqy_out[i] = T(0);
-            } else if (fj == ny) {
-                const size_t c = (size_t)(ny - 1) * P + i;
-                const T mu = S.lqy[lj][li] - dtdx * lL;
-                outflow_adj(a, F, 3, i, S.h[sb][sc], S.n[sb][sc], mu, cl, cn);
-                A.lqy_out[c + P] = T(0);
-            } else {
-                const size_t c = (size_t)fj * P + i;
-                const T mu = S.lqy[lj][li] + dtdx * (lR - lL);
-                const T hL = S.h[sb][sc], zL = S.z[sb][sc], nL = S.n[sb][sc];
-                const T hR = S.h[st][sc], zR = S.z[st][sc], nR = S.n[st][sc];
-                const T hf = F.hf(hL, zL, hR, zR);
-                T lq = T(0);
-                if (hf > hd && mu != T(0)) {
-                    FaceLin<T> d = face_lin<T>(S.qy[lj + 1][li + 4], hL, zL, nL, hR, zR, nR, hf, g, dt, dx);
-                    cl = mu * d.dhL;
-                    cr = mu * d.dhR;
-                    cn = mu * d.dn;
-                    lq = mu * d.dq;
-                }
-                if (lj < TB) A.lqy_out[c] = lq;             // the tile owns the south faces of its cells
-            }
+        if (j == jlast) return;                        // row y1 + 1 only gave its south faces
+        yp = qy;
+        if (inner) {
+            faces2_lin(ya, Kc, dy.q.a, dy.L.a, dy.R.a, dy.n.a);
+            faces2_lin(yb, Kc, dy.q.b, dy.L.b, dy.R.b, dy.n.b);
+        } else {
+            dy = FaceRow{Row4{0, 0}, bL, bR, bn};
         }
-        cYl[lj][li] = cl;
-        cYr[lj][li] = cr;
-        cYn[lj][li] = cn;
+        if (row) {
+            const Row4 el = row_left(e, from_left(e)), zl = row_left(cz, from_left(cz));
+            const float nl = from_left(cn);
+            const float2 e0 = f2unpack(e.a), e1 = f2unpack(e.b), l0 = f2unpack(el.a), n0 = f2unpack(cn.a), n1 = f2unpack(cn.b);
+            const Faces2 xa = faces2_value(f2sub(f2max(el.a, e.a), f2max(zl.a, cz.a)),
+                                           f2pack(__fsub_rn(e0.x, l0.x), __fsub_rn(e0.y, e0.x)), cx.a,
+                                           f2pack(__fadd_rn(nl, n0.x), __fadd_rn(n0.x, n0.y)), Kc);
+            const Faces2 xb = faces2_value(f2sub(f2max(el.b, e.b), f2max(zl.b, cz.b)),
+                                           f2pack(__fsub_rn(e1.x, e0.y), __fsub_rn(e1.y, e1.x)), cx.b,
+                                           f2pack(__fadd_rn(n0.y, n1.x), __fadd_rn(n1.x, n1.y)), Kc);
+            xp = Row4{xa.F, xb.F};
+            faces2_lin(xa, Kc, dx.q.a, dx.L.a, dx.R.a, dx.n.a);
+            faces2_lin(xb, Kc, dx.q.b, dx.L.b, dx.R.b, dx.n.b);
+            if (kEdge && (west || east)) {
+                const float hl = from_left(ch);
+                // the border face of side sd in this lane's column kf
+                auto border = [&](int sd, int t, int slot, float sqrtS) {
+                    const int kf = sd ? nx - c0 : 0;
+                    const float h = sd ? (kf == 0 ? hl : row_get(ch, kf - 1)) : row_get(ch, 0);
+                    const float n = sd ? (kf == 0 ? nl : row_get(cn, kf - 1)) : n0.x;
+                    float dh, dn;
+                    const float v = border_lin(t, sd ? -1.0f : 1.0f, h, sqrtS, n, G,
+                                               t == kBcInflow ? a.inflow_q[(size_t)a.s * a.n_slots + slot] : 0.0f, dh, dn);
+                    row_set(xp, kf, v);
+                    row_set(dx.q, kf, 0.0f);
+                    row_set(dx.L, kf, sd ? dh : 0.0f);
+                    row_set(dx.R, kf, sd ? 0.0f : dh);
+                    row_set(dx.n, kf, dn);
+                };
+                if (kb >= 0) border(side, nb_t, nb_s, nb_q);
+                if (!kSteady && lane_w && lane_e) border(0, a.bc.type[j], a.bc.slot[j], a.bc.sqrtS_f[j]);
+                pb_t = nb_t;
+                pb_s = nb_s;
+                border_fetch(j + 1);
+            }
+        } else {
+            xp = Row4{0, 0};
+            dx = FaceRow{};
+            pb_t = kBcWall;
+        }
+        hp = ch;
+        zp = cz;
+        np_ = cn;
+    };
+
+    int j = jb;
+    if (jb > 0) {                                      // row y0 - 2 is only the row below
+        copy_wait<kAhead - 1>();
+        const float *d = &sm.raw[jb & (kAhead - 1)][0][4 * lane];
+        hp = row_load(d);
+        zp = row_load(d + 128);
+        np_ = row_load(d + 256);
+        border_fetch(jb + 1);
+        issue(jb + kAhead);
+        j++;
     }
+    while (j <= jlast) {
+        if (j >= steady_lo && j <= steady_hi) {
+            if (west || east) {
+#pragma unroll 1
+                for (; j <= steady_hi; j++) tick(std::true_type{}, std::true_type{}, j);
+            } else {
+#pragma unroll 1
+                for (; j <= steady_hi; j++) tick(std::true_type{}, std::false_type{}, j);
+            }
+        } else {
+            const int e = j < steady_lo ? min(jlast, steady_lo - 1) : jlast;
+#pragma unroll 1
+            for (; j <= e; j++) tick(std::false_type{}, std::true_type{}, j);
+        }
+    }
+    copy_wait<0>();
+}
+
+__global__ void __launch_bounds__(32, 12) adj_rows_kernel(const __grid_constant__ AdjArgs<float> A, const int rows, const int rows_edge)
+{
+    __shared__ AdjSmem sm;
+    constexpr int kOut = out_cols(2);
+    const int n_strips = (A.fwd.geo.nx + kOut - 1) / kOut, n_edge = min(n_strips, 2);
+    const int edge_items = n_edge * ((A.fwd.geo.ny + rows_edge - 1) / rows_edge), item = blockIdx.x;
+    int strip, y0, r;
+    if (item < edge_items) {
+        strip = item % n_edge ? n_strips - 1 : 0;
+        r = rows_edge;
+        y0 = (item / n_edge) * r;
+    } else {
+        strip = 1 + (item - edge_items) % (n_strips - n_edge);
+        r = rows;
+        y0 = (item - edge_items) / (n_strips - n_edge) * r;
+    }
+    adj_rows_item(A, strip, y0, min(y0 + r, A.fwd.geo.ny), sm);
+}
+
+// Pass 3 over the logged steps, block (entry, section): the formulas of inflow_adjoint on the logged lu
+// and lambda_q, each section cell's term into the entry's row of A.terms.
+__global__ void __launch_bounds__(64) adj_inflow_terms_kernel(const AdjInflowArgs A)
+{
+    __shared__ double red[32];
+    const int e = blockIdx.x, tid = threadIdx.x;
+    const InflowSec S = A.secs[blockIdx.y];
+    const int64_t step = A.first_step - e;           // global step of the entry
+    const int64_t ie = step / A.E - A.e0;
+    const int s = (int)(step % A.E);
+    const double Q = A.inflow_Q[ie * A.nQ + (size_t)s * A.n_sec + blockIdx.y];
+    const double W = A.inflow_W[ie * A.nQ + (size_t)s * A.n_sec + blockIdx.y];
+    const float *iq = A.inflow_q + ((size_t)ie * A.E + s) * A.n_slots;
+    const float2 *log = A.log + (size_t)e * A.n_slots;
+    double *terms = A.terms + (size_t)e * A.n_slots;
+    const double dx = A.geo.dx, dtdx = A.dt[ie] / A.geo.dx;
+    const double pe = A.geo.bc_form == 0 ? 5.0 / 3.0 : 2.0 / 3.0;
+    const double inward = (double)inward_sign(S.side);
+    auto nu_of = [&](int c) {
+        const float2 v = log[S.slot0 + c];
+        return inward * ((double)v.y + inward * dtdx * (double)v.x) / dx;
+    };
+    double D = 0.0, N = 0.0;
+    if (Q > 0.0)
+        for (int c = tid; c < S.ncell; c += 64) {
+            const double hh = W - (double)A.z[A.cells[S.cell0 + c]];
+            if (!(hh > 0.0)) continue;
+            const double k = pe * ((double)iq[S.slot0 + c] * dx) / hh;
+            D += k;
+            N += nu_of(c) * k;
+        }
+    D = block_reduce<false>(D, red);
     __syncthreads();
-    // D. gather per tile cell
-    const int tx = threadIdx.x, ty = threadIdx.y;
-    const int i = I0 + tx, j = J0 + ty;
-    if (i >= nx || j >= ny) return;
-    const size_t c = (size_t)j * P + i;
-    const T lu = sL[ty + 1][tx + 1];
-    const T lh = lu + cXr[ty][tx] + cXl[ty][tx + 1] + cYr[ty][tx] + cYl[ty + 1][tx];
-    const T gs = (cXn[ty][tx] + cXn[ty][tx + 1]) + (cYn[ty][tx] + cYn[ty + 1][tx]);
-    A.lh_out[c] = lh;
-    A.gn[c] += (double)gs;
-    if (i == 0 || j == 0 || i == nx - 1 || j == ny - 1) A.lhu[c] = lu;   // read by the inflow pass
+    if (tid == 0) red[31] = D;
+    __syncthreads();
+    D = red[31];
+    __syncthreads();
+    N = block_reduce<false>(N, red);
+    __syncthreads();
+    if (tid == 0) red[30] = N;
+    __syncthreads();
+    N = red[30];
+    for (int c = tid; c < S.ncell; c += 64) {
+        const int64_t idx = A.cells[S.cell0 + c];
+        const double hh = W - (double)A.z[idx];
+        double t = 0.0;
+        if (Q > 0.0 && D > 0.0 && hh > 0.0) t = ((double)iq[S.slot0 + c] * dx / (double)A.n[idx]) * (N / D - nu_of(c));
+        terms[S.slot0 + c] = t;
+    }
+}
+
+// Each section cell's terms, in the order of the sweep.
+__global__ void adj_inflow_sum_kernel(const AdjInflowArgs A)
+{
+    const int c = blockIdx.x * blockDim.x + threadIdx.x;
+    if (c >= A.n_slots) return;
+    double g = A.gn_in[c];
+    for (int e = 0; e < A.n_entries; e++) g += A.terms[(size_t)e * A.n_slots + c];
+    A.gn_in[c] = g;
 }
 
 // ---------------------------------------------------------------- the scheme options
@@ -1128,7 +1348,6 @@ template <typename T>
 cudaError_t launch_adjoint_step(const AdjArgs<T> &A, cudaStream_t st)
 {
     const Geom &G = A.fwd.geo;
-    cudaError_t e0 = cudaSuccess;
     if (G.theta != 1.0 || G.friction != 0) {
         if (!A.scratch) return cudaErrorInvalidValue;
         const dim3 block(BX, 8);
@@ -1141,30 +1360,11 @@ cudaError_t launch_adjoint_step(const AdjArgs<T> &A, cudaStream_t st)
         adj_opt_faces_kernel<T><<<(unsigned)((int64_t)nbx * nby1), block, 0, st>>>(A, 1, nbx);
         adj_opt_gather_kernel<T><<<(unsigned)((int64_t)nbx * nby), block, 0, st>>>(A, nbx);
     } else if constexpr (std::is_same<T, float>::value) {
-        // FP32: the tile's inputs staged by tensor copies (maps of this step's buffers)
-        const int P = G.pitch, nx = G.nx, ny = G.ny;
-        const StepArgs<float> &f = A.fwd;
-        AdjMaps maps;
-        constexpr int TB = kAdjTB;
-        const struct {
-            const float *base;
-            int w, h, bw, bh;
-        } fields[8] = {{f.h, nx, ny, kAW, TB + 4},          {f.z, nx, ny, kAW, TB + 4},
-                       {f.n, nx, ny, kAW, TB + 4},          {f.qx, nx + 1, ny, kAW, TB + 2},
-                       {f.qy, nx, ny + 1, kAW, TB + 3},     {A.lh, nx, ny, kAW, TB + 2},
-                       {A.lqx, nx + 1, ny, kAW, TB},        {A.lqy, nx, ny + 1, BX, TB + 1}};
-        for (int k = 0; k < 8; k++) {
-            const cudaError_t e = encode_map_f32(&maps.m[k], fields[k].base, fields[k].w, fields[k].h, P,
-                                                 fields[k].bw, fields[k].bh);
-            if (e != cudaSuccess) return e;
-        }
-        const int nbx = (nx + BX - 1) / BX, nby = (ny + TB - 1) / TB;
-        const int n_tiles = nbx * nby, n_sec = A.gn_in ? A.fwd.n_inflow_sec : 0;
-        adj_step_tma_kernel<TB><<<(unsigned)(n_tiles + n_sec), dim3(BX, TB), 0, st>>>(A, nbx, n_tiles, maps);
-        e0 = cudaGetLastError();
-        if (e0 != cudaSuccess || n_sec > 0) return e0;   // pass 3 ran in the same launch
-        if (A.fwd.n_inflow_sec > 0) adj_inflow_kernel<T><<<A.fwd.n_inflow_sec, 256, 0, st>>>(A);
-        return cudaGetLastError();
+        int rows = 0, edge = 0;
+        tiled_rows(G.nx, G.ny, 2, 0, &rows, &edge);      // an item repeats four rows, as a two-step item does
+        const int items = tiled_item_count(G.nx, G.ny, out_cols(2), rows, edge);
+        adj_rows_kernel<<<items, 32, 0, st>>>(A, rows, edge);
+        return cudaGetLastError();                       // pass 3: launch_adjoint_inflow, after the sweep's steps
     } else {
         constexpr int BYT = TileRows<T>::v;
         dim3 block(BX, BYT);
@@ -1172,6 +1372,14 @@ cudaError_t launch_adjoint_step(const AdjArgs<T> &A, cudaStream_t st)
         adj_step_kernel<T><<<(unsigned)((int64_t)nbx * nby), block, 0, st>>>(A, nbx);
     }
     if (A.fwd.n_inflow_sec > 0) adj_inflow_kernel<T><<<A.fwd.n_inflow_sec, 256, 0, st>>>(A);
+    return cudaGetLastError();
+}
+
+cudaError_t launch_adjoint_inflow(const AdjInflowArgs &A, cudaStream_t st)
+{
+    if (A.n_entries <= 0 || A.n_sec <= 0) return cudaSuccess;
+    adj_inflow_terms_kernel<<<dim3(A.n_entries, A.n_sec), 64, 0, st>>>(A);
+    adj_inflow_sum_kernel<<<(A.n_slots + 63) / 64, 64, 0, st>>>(A);
     return cudaGetLastError();
 }
 

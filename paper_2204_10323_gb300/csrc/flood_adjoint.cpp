@@ -95,8 +95,16 @@ struct Sweep {
     double *gn = nullptr;
     double *gn_in = nullptr;      // FP32, Eq. 3 as printed, with inflow sections: their dL/dn terms per cell
     int n_in_cells = 0;
+    // what pass 3 needs of each reverse step, kept for up to log_cap steps and then worked off at once: a launch
+    // per step for a section's few hundred cells took as long as the step
+    static constexpr int kLogSteps = 512;
+    float2 *in_log = nullptr;
+    double *in_terms = nullptr;
+    int log_cap = 0, logged_steps = 0;
+    int64_t log_first = 0;        // global step of the log's first entry
     int cur_l = 0;
     const int64_t *cells = nullptr;
+    const int2 *cells_rc = nullptr;
     int G = 0;
     const double *seed = nullptr;    // device, N x G
     int64_t fwd_steps = 0;
@@ -245,6 +253,37 @@ flood_status advance_to(Sweep &S, int64_t step, const Planes *last_dst = nullptr
     return FLOOD_OK;
 }
 
+// Pass 3 for the logged reverse steps.
+flood_status flush_inflow(Sweep &S)
+{
+    flood_handle *h = S.h;
+    if (S.logged_steps == 0) return FLOOD_OK;
+    AdjInflowArgs A;
+    std::memset(&A, 0, sizeof(A));
+    A.geo = h->geo;
+    A.secs = h->secs_dev;
+    A.cells = h->sec_cells;
+    A.z = (const float *)h->z;
+    A.n = (const float *)h->n;
+    A.n_sec = h->n_in;
+    A.n_slots = h->n_slots;
+    A.E = S.E;
+    A.e0 = S.e0;
+    A.first_step = S.log_first;
+    A.n_entries = S.logged_steps;
+    A.inflow_q = (const float *)S.iq_log;
+    A.inflow_Q = S.iQ_log;
+    A.inflow_W = S.iW_log;
+    A.dt = S.dt_log;
+    A.nQ = S.nQ;
+    A.log = S.in_log;
+    A.terms = S.in_terms;
+    A.gn_in = S.gn_in;
+    CKA(launch_adjoint_inflow(A, h->stream));
+    S.logged_steps = 0;
+    return FLOOD_OK;
+}
+
 template <typename T>
 flood_status reverse_step_t(Sweep &S)
 {
@@ -290,10 +329,16 @@ flood_status reverse_step_t(Sweep &S)
     A.sec_cells = h->sec_cells;
     A.inflow_W = h->inflow_W;
     A.gauge_cells = S.cells;
+    A.gauge_rc = S.cells_rc;
     A.n_gauges = S.G;
     A.seed = S.seed + (size_t)k * S.G;      // dL/dh after step k, added to lambda_{k+1}
     A.scratch = (T *)S.scratch;
-    A.gn_in = S.gn_in;
+    if (S.in_log) {
+        if (S.logged_steps == S.log_cap && (st = flush_inflow(S))) return st;
+        if (S.logged_steps == 0) S.log_first = g;
+        A.in_log = S.in_log + (size_t)S.logged_steps * h->n_slots;
+        S.logged_steps++;
+    }
     if (S.profile) {
         flood_status ts = timed(S, S.ev_rev, [&] {
             cudaError_t e = launch_adjoint_step<T>(A, h->stream);
@@ -473,16 +518,23 @@ extern "C" flood_status flood_adjoint(flood_handle *h, int64_t n_steps, const in
     const bool opts = h->geo.theta != 1.0 || h->geo.friction != 0;
     if (opts) S.scratch = alloc(11 * S.plane_y);
     S.gn = (double *)alloc(P * h->geo.ny * sizeof(double));
-    if (h->prec == FLOOD_F32 && !opts && h->n_in > 0) {      // the reverse step computes pass 3 beside its tiles
+    if (h->prec == FLOOD_F32 && !opts && h->n_in > 0) {      // pass 3 runs over many steps at once
         S.n_in_cells = h->n_slots;
+        S.log_cap = (int)std::min<int64_t>(n_steps, Sweep::kLogSteps);
         S.gn_in = (double *)alloc((size_t)S.n_in_cells * sizeof(double));
-        if (!S.gn_in) {
+        S.in_log = (float2 *)alloc((size_t)S.log_cap * h->n_slots * sizeof(float2));
+        S.in_terms = (double *)alloc((size_t)S.log_cap * h->n_slots * sizeof(double));
+        if (!S.gn_in || !S.in_log || !S.in_terms) {
             release();
             return fail(h, FLOOD_ERR_OOM, "adjoint buffer allocation");
         }
     }
     double *seed_dev = (double *)alloc(std::max<size_t>((size_t)n_steps * n_gauges, 1) * sizeof(double));
-    int64_t *cells_dev = (int64_t *)alloc(std::max(n_gauges, 1) * sizeof(int64_t));
+    int64_t *cells_dev = (int64_t *)alloc(std::max(n_gauges, 1) * (sizeof(int64_t) + sizeof(int2)));
+    int2 *rc_dev = (int2 *)(cells_dev + std::max(n_gauges, 1));
+    std::vector<int2> rc(n_gauges);
+    for (int g = 0; g < n_gauges; g++)
+        rc[g] = make_int2((int)(gauge_cells[g] / h->geo.nx), (int)(gauge_cells[g] % h->geo.nx));
     for (void *p : {(void *)S.dt_log, (void *)S.tl_log, S.iq_log, (void *)S.iQ_log, (void *)S.iW_log, S.lh[0],
                     S.lh[1], S.lqx[0], S.lqx[1], S.lqy[0], S.lqy[1], S.lhu, (void *)S.gn, (void *)seed_dev,
                     (void *)cells_dev})
@@ -532,6 +584,7 @@ extern "C" flood_status flood_adjoint(flood_handle *h, int64_t n_steps, const in
         CKF(cudaMemcpyAsync(seed_dev, dLdh, (size_t)n_steps * n_gauges * sizeof(double), cudaMemcpyHostToDevice,
                             h->stream));
         CKF(cudaMemcpyAsync(cells_dev, gauge_cells, n_gauges * sizeof(int64_t), cudaMemcpyHostToDevice, h->stream));
+        CKF(cudaMemcpyAsync(rc_dev, rc.data(), n_gauges * sizeof(int2), cudaMemcpyHostToDevice, h->stream));
     }
     for (int b = 0; b < 2; b++) {
         CKF(cudaMemsetAsync(S.lh[b], 0, S.plane, h->stream));
@@ -542,6 +595,7 @@ extern "C" flood_status flood_adjoint(flood_handle *h, int64_t n_steps, const in
     CKF(cudaMemsetAsync(S.gn, 0, P * h->geo.ny * sizeof(double), h->stream));
     if (S.gn_in) CKF(cudaMemsetAsync(S.gn_in, 0, (size_t)S.n_in_cells * sizeof(double), h->stream));
     S.cells = cells_dev;
+    S.cells_rc = rc_dev;
     S.G = n_gauges;
     S.seed = seed_dev;
     // FP32 forward replays run the arithmetic the adjoint linearises: launches of
@@ -566,6 +620,10 @@ extern "C" flood_status flood_adjoint(flood_handle *h, int64_t n_steps, const in
         if (st) return finish(st);
     }
     h->adj_forward_steps = S.fwd_steps;
+    {
+        flood_status st = flush_inflow(S);
+        if (st) return finish(st);
+    }
     if (S.profile) {
         CKF(cudaStreamSynchronize(h->stream));
         h->adj_prof_rev_steps = (int64_t)S.ev_rev.size() / 2;

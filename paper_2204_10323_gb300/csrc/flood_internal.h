@@ -173,16 +173,36 @@ struct AdjArgs {
     const int64_t *sec_cells;
     const double *inflow_W;       // E x n_sec levels of this epoch
     const int64_t *gauge_cells;   // flat j*nx+i of the loss's gauges
+    const int2 *gauge_rc;         // the same as (row, column)
     int n_gauges;
     const double *seed;           // dL/d(depth at gauge g after this step), n_gauges values (device)
     T *scratch;                   // scheme options only: 11 planes of pitch x (ny + 1) elements (face
                                   // contributions of both axes and the clip mask); null otherwise
-    double *gn_in;                // FP32, Eq. 3 as printed: the inflow sections' dL/dn terms per section cell
-                                  // (index cell0 + c), summed over the sweep, added to gn after it
-                                  // (launch_gn_inflow_add); null: added to gn by each step
+    float2 *in_log;               // FP32, Eq. 3 as printed: per inflow slot, the adjoint of the cell's unclipped
+                                  // depth and lambda_q of the face at this step, for pass 3
+                                  // (launch_adjoint_inflow); null without inflow sections
 };
 template <typename T>
 cudaError_t launch_adjoint_step(const AdjArgs<T> &a, cudaStream_t st);
+// Pass 3 of the FP32 sweep (Eq. 3 as printed): the inflow sections' dL/dn terms of n_entries logged steps,
+// entry e the global step first_step - e, summed per section cell into gn_in (added to gn after the sweep,
+// launch_gn_inflow_add).
+struct AdjInflowArgs {
+    Geom geo;
+    const InflowSec *secs;
+    const int64_t *cells;
+    const float *z, *n;
+    int n_sec, n_slots, E;
+    int64_t e0, first_step;       // epoch of the logs' first slice, step of entry 0
+    int n_entries;
+    const float *inflow_q;        // per epoch: E x n_slots
+    const double *inflow_Q, *inflow_W, *dt;   // per epoch: nQ = E x n_sec values, one dt
+    size_t nQ;
+    const float2 *log;            // n_entries x n_slots
+    double *terms;                // n_entries x n_slots (scratch)
+    double *gn_in;                // n_slots
+};
+cudaError_t launch_adjoint_inflow(const AdjInflowArgs &A, cudaStream_t st);
 // 2D tensor map (a CUtensorMap, 64-byte aligned storage at map) of a pitched FP32
 // field of width x height elements and a row pitch of `pitch` elements, for boxes
 // of box_w x box_h elements; elements outside the field read as zeros.
