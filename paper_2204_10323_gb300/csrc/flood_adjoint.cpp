@@ -598,10 +598,9 @@ extern "C" flood_status flood_adjoint(flood_handle *h, int64_t n_steps, const in
     S.cells_rc = rc_dev;
     S.G = n_gauges;
     S.seed = seed_dev;
-    // FP32 forward replays run the arithmetic the adjoint linearises: launches of
-    // one step the tensor-tile kernel below 2^27 cells, the stream kernel above;
-    // launches of up to four steps (replay_steps) the temporal-blocking kernel (all
-    // bitwise equal)
+    // FP32 forward replays run the arithmetic the adjoint linearises: launches of up to four steps
+    // (replay_steps) by the temporal-blocking kernel; single steps on large grids by the tensor-tile kernel
+    // below 2^27 cells, the stream kernel above (launch_step_planes; all bitwise equal)
     if (h->prec == FLOOD_F32)
         h->kernel = (int64_t)h->geo.nx * h->geo.ny < ((int64_t)1 << 27) ? FLOOD_KERNEL_TMA : FLOOD_KERNEL_STREAM;
     for (int b = 0; b < 2; b++) {

@@ -278,14 +278,7 @@ static cudaError_t launch_f32(flood_handle *h, const StepArgs<float> &a)
 {
     switch (h->kernel) {
     case FLOOD_KERNEL_REFERENCE: return launch_step_reference<float>(a, h->stream);
-    case FLOOD_KERNEL_TILED:
-        // gauge recording needs the depth after every step: single steps there
-        if (a.gauge_out) {
-            StepArgs<float> b = a;
-            b.tile_x = b.tile_y = 0;
-            return launch_step_stream(b, h->stream);
-        }
-        return launch_step_tiled(a, h->stream);
+    case FLOOD_KERNEL_TILED: return launch_step_tiled(a, h->stream);
     case FLOOD_KERNEL_STREAM: return launch_step_stream(a, h->stream);
     case FLOOD_KERNEL_TMA: return launch_step_tma(a, h->stream);
     default: return launch_step_rows(a, h->stream);
@@ -328,7 +321,11 @@ flood_status launch_step_planes(flood_handle *h, int s, int k, const void *const
     } else {
         StepArgs<float> a = make_args<float>(h, s, k, 0, nullptr, 0, nullptr);
         set_planes(a, in, out);
-        if (k > 1) {                       // several steps: the temporal-blocking kernel (bitwise the single steps)
+        // The temporal-blocking kernel for several steps, and for one on grids below 2^25 cells: us a step tiled
+        // K = 1 / TMA / stream 11.7 / 13.9 / 15.9 (1024^2), 28.2 / 31.0 / 36.5 (2048^2), 97 / 99 / 103
+        // (4096^2), but 368 / 343 / 349 (8192^2) and 1430 / 1301 / 1298 (16384^2), where one step is bound by
+        // memory and the tiled strips read their halo columns twice.  All bitwise equal.
+        if (k > 1 || (int64_t)h->geo.nx * h->geo.ny < ((int64_t)1 << 25)) {
             a.tile_x = a.tile_y = 0;
             e = launch_step_tiled(a, h->stream);
         } else {
@@ -358,7 +355,7 @@ flood_status advance(flood_handle *h, int64_t n, const int64_t *gcells, int ng, 
             if (st) return st;
         }
         int k = 1;
-        if (h->prec == FLOOD_F32 && h->kernel == FLOOD_KERNEL_TILED && !gcells) {
+        if (h->prec == FLOOD_F32 && h->kernel == FLOOD_KERNEL_TILED) {
             k = std::min<int64_t>(h->k_per_launch, std::min<int64_t>(E - s, n - done));
         }
         int want = (s + k == E) ? 1 : 0;

@@ -83,7 +83,7 @@ struct StepArgs {
     int want_hmax;                // 1: record max depth after the launch's last step
     const int64_t *gauge_cells;   // flat j*nx+i; h after each step -> gauge_out
     int n_gauges;
-    double *gauge_out;            // (k_steps) x n_gauges rows for this launch, or null
+    double *gauge_out;            // k_steps x n_gauges values of this launch, or null
     int tile_x, tile_y;           // launch shape (stream/TMA: warps, rows; tiled: rows per item of the edge
                                   // strips and of the others; on its way in: cap on pipelines, rows per item)
 };

@@ -188,6 +188,7 @@ struct alignas(16) TiledSmem {
     float qy[kMode ? 4 : kAhead][128];   // and qy (the scheme options read it one row further on)
     float z[kRowsZ][128];
     float c[4][2][128];                  // face_c of a row's west and south faces, for levels 2 .. K
+    int gauge[32][3];                    // gauges in the item's own cells: row, staged column, index
 };
 
 // One work item: strip `strip`, rows [y0, y1) of grid a, steps s0 .. s0 + K - 1 of the epoch.
@@ -197,7 +198,8 @@ struct alignas(16) TiledSmem {
 // (4 more per option and level), the old qy of the row above is the row that level s - 1 has just
 // computed (level 1: the next row in flight).  A lane at the strip's edge takes its missing
 // neighbour column as garbage, like the plain arithmetic's edge lanes: it stays inside the halo.
-template <int K, int kMode>
+// kGauge: the depth of the item's gauges after each of the K steps goes to a.gauge_out.
+template <int K, int kMode, bool kGauge>
 __device__ __forceinline__ void tiled_item(const StepArgs<float> &a, const int s0, const int strip, const int y0,
                                            const int y1, const int want_hmax, TiledSmem<kMode> &sm)
 {
@@ -274,6 +276,31 @@ __device__ __forceinline__ void tiled_item(const StepArgs<float> &a, const int s
     };
     border_fetch(jb - bl);
 
+    // the item's gauges; one with more than 32 scans them all at every tick
+    int ng = 0;
+    auto gauge_at = [&](int g, int &row, int &col) {   // false: not in the item
+        const int64_t flat = a.gauge_cells[g];
+        row = (int)(flat / nx);
+        const int c = (int)(flat - (int64_t)row * nx);
+        col = c - x0;
+        return row >= y0 && row < y1 && c >= own_lo && c < own_hi;
+    };
+    if constexpr (kGauge) {
+        for (int g0 = 0; g0 < a.n_gauges; g0 += 32) {
+            int row = 0, col = 0;
+            const bool mine = g0 + lane < a.n_gauges && gauge_at(g0 + lane, row, col);
+            const unsigned m = __ballot_sync(0xffffffffu, mine);
+            const int slot = ng + __popc(m & ((1u << lane) - 1));
+            if (mine && slot < 32) {
+                sm.gauge[slot][0] = row;
+                sm.gauge[slot][1] = col;
+                sm.gauge[slot][2] = g0 + lane;
+            }
+            ng += __popc(m);
+        }
+        __syncwarp();
+    }
+
     Row4 sh[K], sx[K], sy[K];                          // per level: the previous row's old depth and new faces
     Row4 ox[K], oy[K];                                 // and its old qx (kVec) and qy (kTheta)
     Row4 pn{0, 0};                                     // n of the previous row (level 1)
@@ -286,6 +313,7 @@ __device__ __forceinline__ void tiled_item(const StepArgs<float> &a, const int s
     auto tick = [&](auto steady_t, auto edge_t, const int j) {
         constexpr bool kSteady = decltype(steady_t)::value, kEdge = decltype(edge_t)::value;
         Row4 ch{0, 0}, cx{0, 0}, cy{0, 0}, cyn{0, 0};  // the current level's input row, and the old qy of the row above it
+        Row4 last{0, 0};                               // the row that level K finished (kGauge)
         copy_wait<kAhead - 1>();
 #pragma unroll
         for (int s = 1; s <= K; s++) {
@@ -390,6 +418,7 @@ __device__ __forceinline__ void tiled_item(const StepArgs<float> &a, const int s
                                 }
                             fin = row_pack(v[0], v[1], v[2], v[3]);
                         }
+                        if (kGauge && s == K) last = fin;
                         if (s == K && rr >= y0 && (kSteady || rr < y1)) {
                             const float2 g0 = f2unpack(fin.a), g1 = f2unpack(fin.b);
                             const size_t ro = (size_t)rr * P + lane_off;
@@ -454,6 +483,25 @@ __device__ __forceinline__ void tiled_item(const StepArgs<float> &a, const int s
                 }
             } else if (s == 1) {
                 issue(j + kAhead);
+            }
+        }
+        if constexpr (kGauge) {
+            // level s finished row j - s: the next level's previous row (level K's: last)
+            const int n_scan = ng > 32 ? a.n_gauges : ng;
+            for (int x = 0; x < n_scan; x++) {
+                int row, col, idx = x;
+                if (ng <= 32) {
+                    row = sm.gauge[x][0];
+                    col = sm.gauge[x][1];
+                    idx = sm.gauge[x][2];
+                } else if (!gauge_at(x, row, col)) continue;
+                const int k = col & 3;
+#pragma unroll
+                for (int s = 1; s <= K; s++) {
+                    const Row4 v = s < K ? sh[s < K ? s : 0] : last;
+                    if (row == j - s && lane == col >> 2)
+                        a.gauge_out[(size_t)(s - 1) * a.n_gauges + idx] = (double)row_get(v, k);
+                }
             }
         }
         if (kEdge && (west || east)) {
@@ -526,6 +574,7 @@ __device__ __forceinline__ void tiled_item(const StepArgs<float> &a, const int s
         }
     }
     copy_wait<0>();
+    if constexpr (kGauge) __syncwarp();                // before the next item's list
     if (lane == 0) {
         if (led_q != 0.0) atomicAdd(&a.ctrl->V_out, a.ctrl->dt * led_q * G.dx);
         if (led_c != 0.0) atomicAdd(&a.ctrl->V_clip, led_c * G.dx * G.dx);
@@ -552,7 +601,7 @@ __device__ __forceinline__ void tiled_finish(const StepArgs<float> &a, const int
 }
 
 // Item `item` of grid a (a.tile_y rows per item, a.tile_x in the edge strips).
-template <int K, int kMode>
+template <int K, int kMode, bool kGauge>
 __device__ __forceinline__ void tiled_run(const StepArgs<float> &a, const int s0, const int item, const int want_hmax,
                                           TiledSmem<kMode> &sm)
 {
@@ -569,17 +618,17 @@ __device__ __forceinline__ void tiled_run(const StepArgs<float> &a, const int s0
         rows = a.tile_y;
         y0 = (item - edge_items) / (n_strips - n_edge) * rows;
     }
-    tiled_item<K, kMode>(a, s0, strip, y0, min(y0 + rows, a.geo.ny), want_hmax, sm);
+    tiled_item<K, kMode, kGauge>(a, s0, strip, y0, min(y0 + rows, a.geo.ny), want_hmax, sm);
 }
 
 // One grid: a block per item, or (a caller's cap on the pipelines) gridDim.x blocks that walk the items.
-template <int K, int kMode>
+template <int K, int kMode, bool kGauge>
 __global__ void __launch_bounds__(32, tiled_warps(kMode)) step_tiled_kernel(const __grid_constant__ StepArgs<float> a)
 {
     __shared__ TiledSmem<kMode> sm;
     const int n_items = tiled_item_count(a.geo.nx, a.geo.ny, out_cols(K, kMode), a.tile_y, a.tile_x);
 #pragma unroll 1
-    for (int item = blockIdx.x; item < n_items; item += gridDim.x) tiled_run<K, kMode>(a, a.s, item, a.want_hmax, sm);
+    for (int item = blockIdx.x; item < n_items; item += gridDim.x) tiled_run<K, kMode, kGauge>(a, a.s, item, a.want_hmax, sm);
     if (blockIdx.x == 0 && threadIdx.x == 0) tiled_finish<K>(a, a.s);
 }
 
@@ -607,7 +656,7 @@ __global__ void __launch_bounds__(32, tiled_warps(kMode))
     if (local == 0 && threadIdx.x == 0) tiled_finish<K>(a, s0);
     // (the items are numbered for the ensemble's K; a shorter launch's strips may be wider)
     if (local >= tiled_item_count(a.geo.nx, a.geo.ny, out_cols(K, kMode), a.tile_y, a.tile_x)) return;
-    tiled_run<K, kMode>(a, s0, local, want_hmax, sm);
+    tiled_run<K, kMode, false>(a, s0, local, want_hmax, sm);
 }
 
 template <int K, int kMode>
@@ -625,7 +674,8 @@ cudaError_t launch_k(const StepArgs<float> &a0, cudaStream_t st)
     blocks = a0.tile_x > 0 && a0.tile_x < items ? a0.tile_x : items;    // caller's cap on pipelines
     a.tile_x = edge;
     a.tile_y = rows;
-    step_tiled_kernel<K, kMode><<<blocks, 32, 0, st>>>(a);
+    if (a.gauge_out && a.n_gauges > 0) step_tiled_kernel<K, kMode, true><<<blocks, 32, 0, st>>>(a);
+    else step_tiled_kernel<K, kMode, false><<<blocks, 32, 0, st>>>(a);
     return cudaGetLastError();
 }
 

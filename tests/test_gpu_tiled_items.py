@@ -55,3 +55,27 @@ def test_chunks_shorter_than_the_steps_of_a_launch(nx, ny, rows, theta, friction
 @pytest.mark.parametrize("tile", [(1, 0), (3, 4), (2, 200)])
 def test_few_warps_walk_many_items(tile):
     pair(300, 90, 4, tile, 1.0, 0, 50, 5)
+
+
+@pytest.mark.parametrize("k,theta,friction", [(4, 1.0, 0), (3, 1.0, 0), (1, 1.0, 0), (4, 0.9, 1)])
+@pytest.mark.parametrize("nx,ny,tile", [(7, 5, (0, 0)), (250, 61, (0, 9)), (130, 40, (2, 0))])
+def test_gauges_inside_a_launch(nx, ny, tile, k, theta, friction):
+    """Gauge depths after every step of a launch, in border and seam cells, more of them in one
+    item than its list holds and repeated ones, against the stream kernel (bitwise)."""
+    Fm = F()
+    p = inputs.random_small(nx, ny, 3)
+    p.opts.theta, p.opts.friction, p.opts.epoch_steps = theta, friction, 12
+    for a in ("z", "n", "h0", "qx0", "qy0"):
+        setattr(p, a, getattr(p, a).astype(np.float32).astype(np.float64))
+    rng = np.random.default_rng(nx)
+    some = np.stack([rng.integers(0, nx, 6), rng.integers(0, ny, 6)], 1)
+    many = np.stack([rng.integers(0, min(nx, 40), 70), rng.integers(0, min(ny, 8), 70)], 1)
+    edge = np.array([[0, 0], [nx - 1, ny - 1], [nx - 1, 0], [0, ny - 1], [min(119, nx - 1), ny // 2], [min(120, nx - 1), ny // 2]])
+    for gauges in (some, edge, many):
+        a = Fm.Sim(p, kernel=Fm.KERNEL_STREAM)
+        b = Fm.Sim(p, kernel=Fm.KERNEL_TILED, steps_per_launch=k, tile=tile)
+        assert np.array_equal(a.run_gauges(29, gauges), b.run_gauges(29, gauges))
+        for x, y in zip(a.state(), b.state()):
+            assert np.array_equal(x, y)
+        a.close()
+        b.close()
