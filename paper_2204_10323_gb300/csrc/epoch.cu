@@ -11,6 +11,14 @@ namespace {
 
 // Time-step rule at an epoch start: constant, frozen (adjoint replays), or
 // dt = min(dt_cap, alpha dx / sqrt(g h_max)); h_max = 0 gives dt_cap.
+__device__ double epoch_dt(const Geom &G, double hmax, const double *fixed_dt)
+{
+    if (fixed_dt) return *fixed_dt;
+    if (G.dt_mode == 1) return G.dt_const;
+    if (!(hmax > 0.0)) return G.dt_cap;
+    return fmin(G.dt_cap, G.cfl_alpha * G.dx / sqrt(G.g * hmax));
+}
+
 __device__ void epoch_begin_body(const Geom &G, Ctrl *ctrl, double *t_list, int E, const double *fixed_dt)
 {
     double hmax = __longlong_as_double((long long)ctrl->hmax_bits);
@@ -21,11 +29,7 @@ __device__ void epoch_begin_body(const Geom &G, Ctrl *ctrl, double *t_list, int 
         ctrl->cfl_exceed += 1.0;
         ctrl->status |= kStatusCfl;
     }
-    double dt;
-    if (fixed_dt) dt = *fixed_dt;
-    else if (G.dt_mode == 1) dt = G.dt_const;
-    else if (!(hmax > 0.0)) dt = G.dt_cap;
-    else dt = fmin(G.dt_cap, G.cfl_alpha * G.dx / sqrt(G.g * hmax));
+    const double dt = epoch_dt(G, hmax, fixed_dt);
     ctrl->dt = dt;
     ctrl->h_max = hmax;
     ctrl->hmax_bits = 0ull;
@@ -89,7 +93,7 @@ __device__ __forceinline__ double manning_cell_t(double hh, double sqrtS, double
 
 constexpr int kInflowThreads = 128;
 
-// Sections of at most this many cells are solved by warp 0 alone: a bisection
+// Sections of at most this many cells are solved by warp 0 alone: a search
 // step then costs one warp reduction instead of two block barriers, and the
 // solve is latency-bound (the sections of the workloads hold 12-512 cells).
 // FP64 handles evaluate Eq. 5 with the slow double pow, so only the smallest
@@ -103,26 +107,47 @@ __device__ __forceinline__ bool one_warp(const InflowSec &S)
     return S.ncell <= (sizeof(T) == 4 ? kWarpCells : 32);
 }
 
+// Depth exponent of Eq. 5.
+__device__ __forceinline__ double depth_exponent(int form) { return form == 0 ? 5.0 / 3.0 : 2.0 / 3.0; }
+
 // Sum of a one-warp section's Eq. 5 discharges at level W from its cells' z
-// and n staged in shared memory (every lane of warp 0 gets the sum).
+// and n staged in shared memory, and its slope (every lane of warp 0 gets them).
 template <typename T>
 __device__ double section_total_warp(const InflowSec &S, const T *sz, const T *sn, double W, double dx,
-                                     int form)
+                                     int form, double &slope)
 {
-    double s = 0.0;
+    double s = 0.0, d = 0.0;
     for (int c = threadIdx.x; c < S.ncell; c += 32) {
         double hh = W - (double)sz[c];
-        if (hh > 0.0) s += manning_cell_t(hh, S.sqrtS, sn[c], dx, form);
+        if (hh > 0.0) {
+            const double w = manning_cell_t(hh, S.sqrtS, sn[c], dx, form);
+            s += w;
+            d += depth_exponent(form) * w / hh;
+        }
     }
+    slope = warp_sum(d);
     return warp_sum(s);
 }
 
-// FP32 handles, one-warp sections: Eq. 6 in single precision throughout the
-// search (the level W, Eq. 5 per cell, the warp's butterfly sum), bisecting
-// until the midpoint rounds to an end of the bracket (the double-precision
-// search to 1e-12 m spends about twenty more halvings below the resolution of
-// single-precision Eq. 5, each on the slow FP64 pipe); then each cell's
-// discharge rescaled to Q_in in double.
+// The level search.  The section's discharge is increasing in the level W and, for the cross-section form
+// (h^(5/3)), convex: Newton's method from above falls monotonically to the root in a handful of evaluations,
+// where the halvings took 25 (FP32) or 41 and more (FP64), each a chain of powers and a sum over the section.
+// An iteration that leaves the bracket is replaced by a halving, as are all of them for the literal form
+// (h^(2/3): its slope is infinite where a cell falls dry).
+
+// x moved n floats up (down for n < 0).
+__device__ __forceinline__ float float_step(float x, int n)
+{
+    int i = __float_as_int(x);
+    i = i < 0 ? (int)(0x80000000u - (unsigned)i) : i;  // floats in order as integers
+    i += n;
+    return __int_as_float(i < 0 ? (int)(0x80000000u - (unsigned)i) : i);
+}
+
+// FP32 handles, one-warp sections: Eq. 6 in single precision throughout the search (the level W, Eq. 5
+// per cell, the warp's butterfly sum), to neighbouring floats lo, hi with total(lo) < Q <= total(hi): W = hi;
+// then each cell's discharge rescaled to Q_in in double.  An epoch start of 16 steps of a 13-cell section: 17 us
+// in two launches with the halvings, 10.4 in one with Newton's steps; FP64 179 and 55.5 us.
 __device__ void inflow_solve_warp_f32(const InflowSec &S, const float *sz, const float *sn, float zmin, double Q,
                                       double dx, int form, float *out, double *W_slot)
 {
@@ -130,28 +155,57 @@ __device__ void inflow_solve_warp_f32(const InflowSec &S, const float *sz, const
     const float p = form == 0 ? 5.0f / 3.0f : 2.0f / 3.0f;
     const float a = form == 0 ? (float)dx : (float)(dx * dx);
     const float sq = (float)S.sqrtS;
-    auto total = [&](float W) {
+    // the discharge at level W, and its slope in d
+    auto total = [&](float W, float &d) {
         float s = 0.0f;
+        d = 0.0f;
         for (int c = lane; c < S.ncell; c += 32) {
             const float hh = W - sz[c];
-            if (hh > 0.0f) s += a * powf(hh, p) * sq / sn[c];
+            if (hh > 0.0f) {
+                const float w = a * powf(hh, p) * sq / sn[c];
+                s += w;
+                d += __fdividef(p * w, hh);
+            }
         }
-        for (int o = 16; o > 0; o >>= 1) s += __shfl_xor_sync(0xffffffffu, s, o);
+        for (int o = 16; o > 0; o >>= 1) {
+            s += __shfl_xor_sync(0xffffffffu, s, o);
+            d += __shfl_xor_sync(0xffffffffu, d, o);
+        }
         return s;
     };
     const float Qf = (float)Q;
-    float Hb = 1.0f;
-    while (total(zmin + Hb) < Qf && Hb < 1e12f) Hb *= 2.0f;
-    float lo = zmin, hi = zmin + Hb;
+    float Hb = 1.0f, d, f = total(zmin + Hb, d);
+    while (f < Qf && Hb < 1e12f) {
+        Hb *= 2.0f;
+        f = total(zmin + Hb, d);
+    }
+    float lo = zmin, hi = zmin + Hb;                   // f, d: at hi
+    int step = 1;                                      // floats to move when Newton's step is lost in rounding
     for (int it = 0; it < 200; it++) {
-        const float mid = 0.5f * (lo + hi);
-        if (!(mid > lo && mid < hi)) break;
-        if (total(mid) < Qf) lo = mid;
-        else hi = mid;
+        const float half = 0.5f * (lo + hi);
+        if (!(half > lo && half < hi)) break;          // neighbouring floats
+        float W = half;
+        if (form == 0) {
+            W = hi - __fdividef(f - Qf, d);
+            if (!(W > lo && W < hi)) {
+                // at the root up to rounding: a few floats above lo, or below hi
+                W = W <= lo ? float_step(lo, step) : float_step(hi, -step);
+                step *= 2;
+                if (!(W > lo && W < hi)) W = half;
+            }
+        }
+        float dW;
+        const float fW = total(W, dW);
+        if (fW < Qf) lo = W;
+        else {
+            hi = W;
+            f = fW;
+            d = dW;
+        }
     }
     const float W = hi;
     if (lane == 0 && W_slot) *W_slot = (double)W;
-    const double tot = (double)total(W);
+    const double tot = (double)total(W, d);
     for (int c = lane; c < S.ncell; c += 32) {
         const float hh = W - sz[c];
         const float w = hh > 0.0f ? a * powf(hh, p) * sq / sn[c] : 0.0f;
@@ -159,40 +213,50 @@ __device__ void inflow_solve_warp_f32(const InflowSec &S, const float *sz, const
     }
 }
 
-// Block-wide sum of the section's Eq. 5 discharges at level W (all threads get it).
+// Block-wide sum of the section's Eq. 5 discharges at level W, and its slope (all threads get them).
 template <typename T>
 __device__ double section_total(const InflowSec &S, const int64_t *cells, const T *z, const T *n,
-                                double W, double dx, int form, double *red)
+                                double W, double dx, int form, double *red, double &slope)
 {
-    double s = 0.0;
+    double s = 0.0, d = 0.0;
     for (int c = threadIdx.x; c < S.ncell; c += kInflowThreads) {
         int64_t idx = cells[S.cell0 + c];
         double hh = W - (double)z[idx];
-        if (hh > 0.0) s += manning_cell_t(hh, S.sqrtS, n[idx], dx, form);
+        if (hh > 0.0) {
+            const double w = manning_cell_t(hh, S.sqrtS, n[idx], dx, form);
+            s += w;
+            d += depth_exponent(form) * w / hh;
+        }
     }
     s = warp_sum(s);
+    d = warp_sum(d);
     __syncthreads();
-    if ((threadIdx.x & 31) == 0) red[threadIdx.x >> 5] = s;
+    if ((threadIdx.x & 31) == 0) {
+        red[threadIdx.x >> 5] = s;
+        red[kInflowThreads / 32 + (threadIdx.x >> 5)] = d;
+    }
     __syncthreads();
     double t = 0.0;
-    for (int w = 0; w < kInflowThreads / 32; w++) t += red[w];
+    slope = 0.0;
+    for (int w = 0; w < kInflowThreads / 32; w++) {
+        t += red[w];
+        slope += red[kInflowThreads / 32 + w];
+    }
     return t;
 }
 
 // Eq. 6 for (step s of the epoch, inflow section k), by warp 0 or the whole
-// block (one_warp): bisection for
-// the level W with sum_c Q_c(W) = Q_in(t_s) on [min z, min z + H] (H doubled
-// from 1 m), 200 halvings at most or a bracket below 1e-12 m, W = upper end;
-// then each cell's discharge scaled by Q_in / sum, stored as unit-width flux.
+// block (one_warp): the level W with sum_c Q_c(W) = Q_in(t) bracketed on [min z, min z + H]
+// (H doubled from 1 m), 200 steps at most or a bracket below 1e-12 m, W = upper end; then
+// each cell's discharge scaled by Q_in / sum, stored as unit-width flux.
 template <typename T>
 __device__ void inflow_body(const Geom &G, const InflowSec *secs, int nsec, const int64_t *cells,
                             const double *tab_t, const double *tab_q, const T *z, const T *n,
-                            const double *t_list, T *inflow_q, int n_slots, double *inflow_Q, double *W_out,
+                            const double t, T *inflow_q, int n_slots, double *inflow_Q, double *W_out,
                             const int s, const int k, double *red, T *sz, T *sn)
 {
     const int tid = threadIdx.x;
     const InflowSec S = secs[k];
-    const double t = t_list[s];
     const double Q = hydrograph(tab_t + S.tab0, tab_q + S.tab0, S.ntab, t);
     T *out = inflow_q + (size_t)s * n_slots + S.slot0;
     // a section that covers no cell carries no discharge
@@ -225,20 +289,40 @@ __device__ void inflow_body(const Geom &G, const InflowSec *secs, int nsec, cons
             return;
         }
     }
-    auto total_at = [&](double W) {
-        return warp_only ? section_total_warp(S, sz, sn, W, dx, form) : section_total(S, cells, z, n, W, dx, form, red);
+    auto total_at = [&](double W, double &d) {
+        return warp_only ? section_total_warp(S, sz, sn, W, dx, form, d)
+                         : section_total(S, cells, z, n, W, dx, form, red, d);
     };
-    double Hb = 1.0;
-    while (total_at(zmin + Hb) < Q && Hb < 1e12) Hb *= 2.0;
-    double lo = zmin, hi = zmin + Hb;
+    double Hb = 1.0, d, f = total_at(zmin + Hb, d);
+    while (f < Q && Hb < 1e12) {
+        Hb *= 2.0;
+        f = total_at(zmin + Hb, d);
+    }
+    double lo = zmin, hi = zmin + Hb;                  // f, d: at hi
     for (int it = 0; it < 200 && hi - lo >= 1e-12; it++) {
-        double mid = 0.5 * (lo + hi);
-        if (total_at(mid) < Q) lo = mid;
-        else hi = mid;
+        const double half = 0.5 * (lo + hi);
+        if (!(half > lo && half < hi)) break;          // neighbouring doubles
+        double W = half;
+        if (form == 0 && it < 60) {
+            // Newton's step; once it is below the bracket's width, the end of that width from hi (or, where
+            // rounding has left lo at the root, from lo)
+            W = hi - (f - Q) / d;
+            if (W > hi - 0.45e-12) W = hi - 0.9e-12;
+            else if (W <= lo + 0.45e-12) W = lo + 0.9e-12;
+            if (!(W > lo && W < hi)) W = half;
+        }
+        double dW;
+        const double fW = total_at(W, dW);
+        if (fW < Q) lo = W;
+        else {
+            hi = W;
+            f = fW;
+            d = dW;
+        }
     }
     const double W = hi;
     if (tid == 0 && W_out) W_out[(size_t)s * nsec + k] = W;
-    const double total = total_at(W);
+    const double total = total_at(W, d);
     for (int c = tid; c < S.ncell; c += nthreads) {
         int64_t idx = cells[S.cell0 + c];
         double hh = W - (double)z[idx];
@@ -247,27 +331,60 @@ __device__ void inflow_body(const Geom &G, const InflowSec *secs, int nsec, cons
     }
 }
 
-template <typename T>
-__global__ void inflow_kernel(Geom G, const InflowSec *secs, int nsec, const int64_t *cells,
-                              const double *tab_t, const double *tab_q, const T *z, const T *n,
-                              const double *t_list, T *inflow_q, int n_slots, double *inflow_Q, double *W_out)
+// An epoch start in the blocks of its inflow solve, in place of a launch of its own (one thread's few
+// microseconds and a launch gap): each block derives the time step and its step's start time for itself,
+// and the last of the simulation's `blocks` blocks to have read the control block writes the epoch's into it.
+__device__ double epoch_time(const Geom &G, const Ctrl *ctrl, const double *fixed_dt, int s, double *shared_t)
 {
-    __shared__ double red[kInflowThreads / 32];
-    __shared__ T sz[kWarpCells], sn[kWarpCells];
-    inflow_body<T>(G, secs, nsec, cells, tab_t, tab_q, z, n, t_list, inflow_q, n_slots, inflow_Q, W_out, blockIdx.x,
-                   blockIdx.y, red, sz, sn);
+    if (threadIdx.x == 0) {
+        const double dt = epoch_dt(G, __longlong_as_double((long long)ctrl->hmax_bits), fixed_dt);
+        double t = ctrl->t;
+        for (int k = 0; k < s; k++) t = t + dt;        // the additions of t_list
+        *shared_t = t;
+    }
+    __syncthreads();
+    return *shared_t;
 }
 
-// Eq. 6 for every (step, section) of a batch of simulations: block (s, task).
-template <typename T>
-__global__ void inflow_batched_kernel(const EpochArgs<T> *tab, const int2 *tasks)
+// By the block's last thread, which a one-warp solve leaves free.
+__device__ void epoch_commit(const Geom &G, Ctrl *ctrl, double *t_list, int E, const double *fixed_dt, unsigned blocks)
 {
-    __shared__ double red[kInflowThreads / 32];
+    if (threadIdx.x != kInflowThreads - 1) return;
+    __threadfence();
+    if (atomicAdd(&ctrl->epoch_blocks, 1u) != blocks - 1) return;
+    __threadfence();
+    ctrl->epoch_blocks = 0;
+    epoch_begin_body(G, ctrl, t_list, E, fixed_dt);
+}
+
+// Eq. 6 for (step, section) = block (x, y); kBegin: the epoch starts here (ctrl, fixed_dt), else t_list holds
+// its times.
+template <typename T, bool kBegin>
+__global__ void __launch_bounds__(kInflowThreads)
+    inflow_kernel(Geom G, Ctrl *ctrl, const double *fixed_dt, const InflowSec *secs, int nsec, const int64_t *cells,
+                  const double *tab_t, const double *tab_q, const T *z, const T *n, double *t_list, int E, T *inflow_q,
+                  int n_slots, double *inflow_Q, double *W_out)
+{
+    __shared__ double red[2 * kInflowThreads / 32], st;
     __shared__ T sz[kWarpCells], sn[kWarpCells];
-    const int2 t = tasks[blockIdx.y];
-    const EpochArgs<T> &A = tab[t.x];
-    inflow_body<T>(A.geo, A.secs, A.nsec, A.cells, A.tab_t, A.tab_q, A.z, A.n, A.t_list, A.inflow_q, A.n_slots,
-                   A.inflow_Q, A.inflow_W, blockIdx.x, t.y, red, sz, sn);
+    const double t = kBegin ? epoch_time(G, ctrl, fixed_dt, blockIdx.x, &st) : t_list[blockIdx.x];
+    inflow_body<T>(G, secs, nsec, cells, tab_t, tab_q, z, n, t, inflow_q, n_slots, inflow_Q, W_out, blockIdx.x,
+                   blockIdx.y, red, sz, sn);
+    if (kBegin) epoch_commit(G, ctrl, t_list, E, fixed_dt, gridDim.x * gridDim.y);
+}
+
+// The same for every (step, section) of a batch of simulations: block (s, task).
+template <typename T, bool kBegin>
+__global__ void __launch_bounds__(kInflowThreads) inflow_batched_kernel(const EpochArgs<T> *tab, const int2 *tasks)
+{
+    __shared__ double red[2 * kInflowThreads / 32], st;
+    __shared__ T sz[kWarpCells], sn[kWarpCells];
+    const int2 task = tasks[blockIdx.y];
+    const EpochArgs<T> &A = tab[task.x];
+    const double t = kBegin ? epoch_time(A.geo, A.ctrl, nullptr, blockIdx.x, &st) : A.t_list[blockIdx.x];
+    inflow_body<T>(A.geo, A.secs, A.nsec, A.cells, A.tab_t, A.tab_q, A.z, A.n, t, A.inflow_q, A.n_slots,
+                   A.inflow_Q, A.inflow_W, blockIdx.x, task.y, red, sz, sn);
+    if (kBegin) epoch_commit(A.geo, A.ctrl, A.t_list, gridDim.x, nullptr, gridDim.x * A.nsec);
 }
 
 // Rows over blocks, columns over threads; the maximum is exact in the state's
@@ -368,36 +485,44 @@ cudaError_t launch_hmax_allreduce(Ctrl *const *ctrls, int n, cudaStream_t st)
     return cudaGetLastError();
 }
 
-cudaError_t launch_epoch_begin(const Geom &g, Ctrl *ctrl, double *t_list, int E, const double *fixed_dt,
-                               cudaStream_t st)
+static cudaError_t launch_epoch_begin(const Geom &g, Ctrl *ctrl, double *t_list, int E, const double *fixed_dt,
+                                      cudaStream_t st)
 {
     epoch_begin_kernel<<<1, 32, 0, st>>>(g, ctrl, t_list, E, fixed_dt);
     return cudaGetLastError();
 }
 
 template <typename T>
-cudaError_t launch_epoch_batched(const EpochArgs<T> *tab, int n, const int2 *tasks, int n_tasks, int E,
+cudaError_t launch_epoch_batched(const EpochArgs<T> *tab, int n, const int2 *tasks, int n_tasks, int E, bool all_inflow,
                                  cudaStream_t st)
 {
+    if (all_inflow) {
+        inflow_batched_kernel<T, true><<<dim3(E, n_tasks), kInflowThreads, 0, st>>>(tab, tasks);
+        return cudaGetLastError();
+    }
     epoch_begin_batched_kernel<T><<<(n + 127) / 128, 128, 0, st>>>(tab, n, E);
     cudaError_t e = cudaGetLastError();
     if (e != cudaSuccess || n_tasks == 0) return e;
-    inflow_batched_kernel<T><<<dim3(E, n_tasks), kInflowThreads, 0, st>>>(tab, tasks);
+    inflow_batched_kernel<T, false><<<dim3(E, n_tasks), kInflowThreads, 0, st>>>(tab, tasks);
     return cudaGetLastError();
 }
 
-template cudaError_t launch_epoch_batched<float>(const EpochArgs<float> *, int, const int2 *, int, int, cudaStream_t);
+template cudaError_t launch_epoch_batched<float>(const EpochArgs<float> *, int, const int2 *, int, int, bool,
+                                                 cudaStream_t);
 
 template <typename T>
-cudaError_t launch_inflow(const Geom &g, const InflowSec *secs, int nsec, const int64_t *sec_cells,
-                          const int8_t * /*sec_side*/, const double *tab_t, const double *tab_q,
-                          const T *z, const T *n, const double *t_list, int E, T *inflow_q, int n_slots,
-                          double *inflow_Q, double *W_out, cudaStream_t st)
+cudaError_t launch_inflow(const EpochArgs<T> &A, int E, bool begin, const double *fixed_dt, cudaStream_t st)
 {
-    if (nsec == 0) return cudaSuccess;
-    dim3 grid(E, nsec);
-    inflow_kernel<T><<<grid, kInflowThreads, 0, st>>>(g, secs, nsec, sec_cells, tab_t, tab_q, z, n, t_list, inflow_q,
-                                          n_slots, inflow_Q, W_out);
+    if (A.nsec == 0) return begin ? launch_epoch_begin(A.geo, A.ctrl, A.t_list, E, fixed_dt, st) : cudaSuccess;
+    const dim3 grid(E, A.nsec);
+    if (begin)
+        inflow_kernel<T, true><<<grid, kInflowThreads, 0, st>>>(A.geo, A.ctrl, fixed_dt, A.secs, A.nsec, A.cells, A.tab_t, A.tab_q,
+                                                                A.z, A.n, A.t_list, E, A.inflow_q, A.n_slots, A.inflow_Q,
+                                                                A.inflow_W);
+    else
+        inflow_kernel<T, false><<<grid, kInflowThreads, 0, st>>>(A.geo, A.ctrl, nullptr, A.secs, A.nsec, A.cells, A.tab_t, A.tab_q,
+                                                                 A.z, A.n, A.t_list, E, A.inflow_q, A.n_slots, A.inflow_Q,
+                                                                 A.inflow_W);
     return cudaGetLastError();
 }
 
@@ -479,10 +604,7 @@ cudaError_t launch_gauges(const Geom &g, const T *h, const int64_t *cells, int G
 }
 
 #define FLOOD_INST(T)                                                                                      \
-    template cudaError_t launch_inflow<T>(const Geom &, const InflowSec *, int, const int64_t *,             \
-                                          const int8_t *, const double *, const double *, const T *,       \
-                                          const T *, const double *, int, T *, int, double *, double *,      \
-                                          cudaStream_t);                                                    \
+    template cudaError_t launch_inflow<T>(const EpochArgs<T> &, int, bool, const double *, cudaStream_t);       \
     template cudaError_t launch_hmax<T>(const Geom &, const T *, Ctrl *, cudaStream_t);                     \
     template cudaError_t launch_volume<T>(const Geom &, const T *, double *, int, double *, cudaStream_t);   \
     template cudaError_t launch_gauges<T>(const Geom &, const T *, const int64_t *, int, double *, cudaStream_t); \

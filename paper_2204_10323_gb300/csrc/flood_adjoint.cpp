@@ -178,10 +178,9 @@ flood_status ensure_epoch(Sweep &S, int64_t e)
         CKA(cudaMemsetAsync(&h->ctrl->hmax_bits, 0, sizeof(unsigned long long), h->stream));
         if (h->prec == FLOOD_F32) CKA(launch_hmax<float>(h->geo, (const float *)S.src.h, h->ctrl, h->stream));
         else CKA(launch_hmax<double>(h->geo, (const double *)S.src.h, h->ctrl, h->stream));
-        CKA(launch_epoch_begin(h->geo, h->ctrl, h->t_list, E, nullptr, h->stream));
-        CKA(cudaMemcpyAsync(dtl, &h->ctrl->dt, sizeof(double), cudaMemcpyDeviceToDevice, h->stream));
-        flood_status st = launch_inflow_epoch(h);
+        flood_status st = begin_epoch(h);
         if (st) return st;
+        CKA(cudaMemcpyAsync(dtl, &h->ctrl->dt, sizeof(double), cudaMemcpyDeviceToDevice, h->stream));
         S.logged[ie] = 1;
     } else {
         CKA(cudaMemcpyAsync(&h->ctrl->dt, dtl, sizeof(double), cudaMemcpyDeviceToDevice, h->stream));

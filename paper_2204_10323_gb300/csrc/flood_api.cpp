@@ -217,22 +217,41 @@ flood_status refresh_hmax(flood_handle *h)
     return FLOOD_OK;
 }
 
-flood_status launch_inflow_epoch(flood_handle *h)
+template <typename T>
+static EpochArgs<T> epoch_args(flood_handle *h)
 {
-    if (h->n_in == 0) return FLOOD_OK;
-    int E = h->geo.epoch_steps;
+    EpochArgs<T> A;
+    A.geo = h->geo;
+    A.ctrl = h->ctrl;
+    A.t_list = h->t_list;
+    A.secs = h->secs_dev;
+    A.nsec = h->n_in;
+    A.cells = h->sec_cells;
+    A.tab_t = h->tab_t;
+    A.tab_q = h->tab_q;
     // the section cells' z and n: in the grid's own planes, or a part's copies of them
-    const void *z = h->sec_z ? h->sec_z : h->z, *n = h->sec_z ? h->sec_n : h->n;
-    if (h->prec == FLOOD_F32)
-        CK(launch_inflow<float>(h->geo, h->secs_dev, h->n_in, h->sec_cells, nullptr, h->tab_t, h->tab_q,
-                                (const float *)z, (const float *)n, h->t_list, E, (float *)h->inflow_q,
-                                h->n_slots, h->inflow_Q, h->inflow_W, h->stream));
-    else
-        CK(launch_inflow<double>(h->geo, h->secs_dev, h->n_in, h->sec_cells, nullptr, h->tab_t, h->tab_q,
-                                 (const double *)z, (const double *)n, h->t_list, E, (double *)h->inflow_q,
-                                 h->n_slots, h->inflow_Q, h->inflow_W, h->stream));
+    A.z = (const T *)(h->sec_z ? h->sec_z : h->z);
+    A.n = (const T *)(h->sec_z ? h->sec_n : h->n);
+    A.inflow_q = (T *)h->inflow_q;
+    A.n_slots = h->n_slots;
+    A.inflow_Q = h->inflow_Q;
+    A.inflow_W = h->inflow_W;
+    return A;
+}
+
+EpochArgs<float> epoch_args_f32(flood_handle *h) { return epoch_args<float>(h); }
+
+static flood_status launch_epoch(flood_handle *h, bool begin, const double *fixed_dt)
+{
+    const int E = h->geo.epoch_steps;
+    if (h->prec == FLOOD_F32) CK(launch_inflow<float>(epoch_args<float>(h), E, begin, fixed_dt, h->stream));
+    else CK(launch_inflow<double>(epoch_args<double>(h), E, begin, fixed_dt, h->stream));
     return FLOOD_OK;
 }
+
+flood_status launch_inflow_epoch(flood_handle *h) { return launch_epoch(h, false, nullptr); }
+
+flood_status begin_epoch(flood_handle *h, const double *fixed_dt) { return launch_epoch(h, true, fixed_dt); }
 
 template <typename T>
 StepArgs<T> make_args(flood_handle *h, int s, int k_steps, int want_hmax, const int64_t *gcells,
@@ -350,8 +369,7 @@ flood_status advance(flood_handle *h, int64_t n, const int64_t *gcells, int ng, 
         if (s == 0 && !(epoch_open && done == 0)) {
             NvtxRange epoch("flood: epoch start (dt, Eq. 6 inflow)");
             const double *fdt = fixed_dt_log ? fixed_dt_log + done : nullptr;
-            CK(launch_epoch_begin(h->geo, h->ctrl, h->t_list, E, fdt, h->stream));
-            flood_status st = launch_inflow_epoch(h);
+            flood_status st = begin_epoch(h, fdt);
             if (st) return st;
         }
         int k = 1;
@@ -821,8 +839,7 @@ extern "C" flood_status flood_advance(flood_handle *h, double t_end, int64_t *st
         const int s = (int)(h->step % E);
         const bool begun = s == 0;
         if (begun) {                                   // begin the epoch here: its dt decides the steps
-            CK(launch_epoch_begin(h->geo, h->ctrl, h->t_list, E, nullptr, h->stream));
-            flood_status st = launch_inflow_epoch(h);
+            flood_status st = begin_epoch(h);
             if (st) return st;
         }
         CK(cudaMemcpyAsync(tl.data(), h->t_list, (E + 1) * sizeof(double), cudaMemcpyDeviceToHost, h->stream));

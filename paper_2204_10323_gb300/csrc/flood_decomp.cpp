@@ -276,8 +276,7 @@ extern "C" flood_status flood_decomp_step(flood_decomp *d, int64_t n_steps)
             // epoch start: every part chooses dt from the whole grid's h_max, and solves Eq. 6
             for (int r = 0; r < d->n_parts; r++) {
                 flood_handle *h = d->parts[r];
-                DCK(launch_epoch_begin(h->geo, h->ctrl, h->t_list, E, nullptr, h->stream));
-                flood_status st = launch_inflow_epoch(h);
+                flood_status st = begin_epoch(h);
                 if (st) return part_fail(d, r, st);
             }
         }

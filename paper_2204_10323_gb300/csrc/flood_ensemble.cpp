@@ -46,6 +46,7 @@ struct flood_ensemble {
     EpochArgs<float> *getab[kGroups] = {nullptr, nullptr};   // the group's members' epoch arguments
     int2 *gtasks[kGroups] = {nullptr, nullptr};              // (member in the group, inflow section)
     int gntasks[kGroups] = {0, 0};
+    bool ginflow[kGroups] = {false, false}, inflow = false;  // every member (of the group) has an inflow section
     cudaStream_t lane[kGroups] = {nullptr, nullptr};
     cudaEvent_t lane_ev[kGroups] = {nullptr, nullptr};
     cudaEvent_t fork_ev = nullptr;
@@ -76,27 +77,6 @@ void drop_graphs(flood_ensemble *e)
     for (auto &g : e->graphs)
         if (g) cudaGraphExecDestroy(g);
     e->graphs.assign(2, nullptr);
-}
-
-// Epoch bookkeeping arguments of a member.
-EpochArgs<float> epoch_args(const flood_handle *h)
-{
-    EpochArgs<float> A;
-    A.geo = h->geo;
-    A.ctrl = h->ctrl;
-    A.t_list = h->t_list;
-    A.secs = h->secs_dev;
-    A.nsec = h->n_in;
-    A.cells = h->sec_cells;
-    A.tab_t = h->tab_t;
-    A.tab_q = h->tab_q;
-    A.z = (const float *)h->z;
-    A.n = (const float *)h->n;
-    A.inflow_q = (float *)h->inflow_q;
-    A.n_slots = h->n_slots;
-    A.inflow_Q = h->inflow_Q;
-    A.inflow_W = h->inflow_W;
-    return A;
 }
 
 // Rows per work item of the temporal-blocking kernel for a member grid (an edge
@@ -210,9 +190,11 @@ flood_status build_tables(flood_ensemble *e)
             // the group's own epoch starts (dt, Eq. 6), on its stream
             std::vector<EpochArgs<float>> et(ng);
             std::vector<int2> tk;
+            e->ginflow[g] = ng > 0;
             for (int i = 0; i < ng; i++) {
-                const flood_handle *h = e->members[members[g][i]];
-                et[i] = epoch_args(h);
+                flood_handle *h = e->members[members[g][i]];
+                et[i] = epoch_args_f32(h);
+                e->ginflow[g] = e->ginflow[g] && h->n_in > 0;
                 for (int sct = 0; sct < h->n_in; sct++) tk.push_back(make_int2(i, sct));
             }
             e->gntasks[g] = (int)tk.size();
@@ -268,13 +250,14 @@ flood_status ensemble_step(flood_ensemble *e, int64_t limit, cudaStream_t st, in
         if (fs) return fs;
         for (int g = 0; g < flood_ensemble::kGroups; g++) {
             if (e->gn[g] == 0) continue;
-            cudaError_t c = launch_epoch_batched<float>(e->getab[g], e->gn[g], e->gtasks[g], e->gntasks[g], E, e->lane[g]);
+            cudaError_t c = launch_epoch_batched<float>(e->getab[g], e->gn[g], e->gtasks[g], e->gntasks[g], E, e->ginflow[g],
+                                                        e->lane[g]);
             if (c != cudaSuccess) return efail(e, FLOOD_ERR_CUDA, cudaGetErrorString(c));
         }
     } else if (s == 0) {
         flood_status fs = join_groups(e, st);
         if (fs) return fs;
-        cudaError_t c = launch_epoch_batched<float>(e->etab, (int)e->members.size(), e->tasks, e->n_tasks, E, st);
+        cudaError_t c = launch_epoch_batched<float>(e->etab, (int)e->members.size(), e->tasks, e->n_tasks, E, e->inflow, st);
         if (c != cudaSuccess) return efail(e, FLOOD_ERR_CUDA, cudaGetErrorString(c));
     }
     const int parity = e->members[0]->cur;
@@ -433,23 +416,11 @@ extern "C" flood_status flood_ensemble_create(int32_t n, const flood_grid *grids
     e->etab = (EpochArgs<float> *)dev_alloc(e->owner, n * sizeof(EpochArgs<float>));
     std::vector<EpochArgs<float>> et(n);
     std::vector<int2> tk;
+    e->inflow = true;
     for (int k = 0; k < n; k++) {
         flood_handle *h = e->members[k];
-        EpochArgs<float> &A = et[k];
-        A.geo = h->geo;
-        A.ctrl = h->ctrl;
-        A.t_list = h->t_list;
-        A.secs = h->secs_dev;
-        A.nsec = h->n_in;
-        A.cells = h->sec_cells;
-        A.tab_t = h->tab_t;
-        A.tab_q = h->tab_q;
-        A.z = (const float *)h->z;
-        A.n = (const float *)h->n;
-        A.inflow_q = (float *)h->inflow_q;
-        A.n_slots = h->n_slots;
-        A.inflow_Q = h->inflow_Q;
-        A.inflow_W = h->inflow_W;
+        et[k] = epoch_args_f32(h);
+        e->inflow = e->inflow && h->n_in > 0;
         for (int sct = 0; sct < h->n_in; sct++) tk.push_back(make_int2(k, sct));
     }
     e->n_tasks = (int)tk.size();

@@ -28,7 +28,7 @@ struct Ctrl {
     double cfl_exceed;            // epochs whose dt broke dx / sqrt(g h_max) at their end
     unsigned long long hmax_bits; // running max of h (bits of a non-negative double)
     int status;                   // kStatus* bits
-    int pad;
+    unsigned epoch_blocks;        // blocks of an epoch start that have read the words above (0 between epoch starts)
 };
 
 // One inflow section as seen by the Eq. 6 solver.
@@ -110,23 +110,10 @@ cudaError_t launch_step_tiled_ensemble(const StepArgs<float> *table, const int *
 void stream_launch_shape(const Geom &g, int tile_x, int tile_y, int *warps, int *rows);
 cudaError_t launch_step_tiled(const StepArgs<float> &a, cudaStream_t st);
 
-// Epoch start: choose dt from h_max (or constant, or fixed_dt[0] when given:
-// the adjoint's replay of a logged epoch), fill t_list, reset the running
-// maximum, count CFL exceedances, flag NaN/Inf.
-cudaError_t launch_epoch_begin(const Geom &g, Ctrl *ctrl, double *t_list, int E, const double *fixed_dt,
-                               cudaStream_t st);
 // Decomposed grid: every part's running h_max (ctrls: n device pointers, on
 // the device) set to the largest of them.
 cudaError_t launch_hmax_allreduce(Ctrl *const *ctrls, int n, cudaStream_t st);
-// Eq. 6 for every (step of the epoch, inflow section) pair.
-template <typename T>
-cudaError_t launch_inflow(const Geom &g, const InflowSec *secs, int nsec, const int64_t *sec_cells,
-                          const int8_t *sec_side, const double *tab_t, const double *tab_q,
-                          const T *z, const T *n, const double *t_list, int E, T *inflow_q,
-                          int n_slots, double *inflow_Q, double *W_out, cudaStream_t st);
-// Epoch bookkeeping of a batch of simulations in two launches: the time-step
-// rule for each (one thread each), then Eq. 6 for every (step, section) task
-// (task = {simulation, section}).
+// What an epoch start of one simulation reads and writes.
 template <typename T>
 struct EpochArgs {
     Geom geo;
@@ -141,8 +128,15 @@ struct EpochArgs {
     int n_slots;
     double *inflow_Q, *inflow_W;
 };
+// Eq. 6 for every (step of the epoch, inflow section) pair.  begin: the epoch starts: choose dt from h_max (or
+// constant, or fixed_dt[0] when given: the adjoint's replay of a logged epoch), fill t_list, reset the running
+// maximum, count CFL exceedances, flag NaN/Inf; else Eq. 6 alone, from the t_list there is.
 template <typename T>
-cudaError_t launch_epoch_batched(const EpochArgs<T> *tab, int n, const int2 *tasks, int n_tasks, int E,
+cudaError_t launch_inflow(const EpochArgs<T> &A, int E, bool begin, const double *fixed_dt, cudaStream_t st);
+// Epoch starts of a batch of simulations (task = {simulation, section}); all_inflow: every one has a section
+// (one launch, else two).
+template <typename T>
+cudaError_t launch_epoch_batched(const EpochArgs<T> *tab, int n, const int2 *tasks, int n_tasks, int E, bool all_inflow,
                                  cudaStream_t st);
 // h_max of a state into ctrl->hmax_bits (max with what is there).
 template <typename T>

@@ -125,7 +125,10 @@ flood_status copy_out(flood_handle *h, void *dst, const void *src_pitched, int r
 cudaError_t copy_rows(void *dst, size_t dpitch, const void *src, size_t spitch, size_t width, size_t rows, int on_device,
                       bool to_device, int device, cudaStream_t st);
 flood_status refresh_hmax(flood_handle *h);
+// Eq. 6 for the epoch in progress; begin_epoch: the epoch start (time step, times) with it.
 flood_status launch_inflow_epoch(flood_handle *h);
+flood_status begin_epoch(flood_handle *h, const double *fixed_dt = nullptr);
+EpochArgs<float> epoch_args_f32(flood_handle *h);
 flood_status launch_steps(flood_handle *h, int s, int k, int want_hmax, const int64_t *gcells, int ng,
                           double *gout);
 // One step at step-in-epoch s reading the state planes in[] = {h, qx, qy} and
