@@ -46,6 +46,18 @@ template <> struct R<double> {
 // Operations in the order of the plain definition, each rounded once (no
 // contraction).
 template <typename T>
+__device__ __forceinline__ T face_wet_ieee(T qn, T qmag, T etaL, T etaR, T hf, T nL, T nR, T g, T dt, T dx)
+{
+    using O = R<T>;
+    T nf = O::mul(T(0.5), O::add(nL, nR));
+    T gdt = O::mul(g, dt);
+    T slope_term = O::div(O::mul(O::mul(gdt, hf), O::sub(etaR, etaL)), dx);
+    T hf_m73 = O::div(T(1), O::mul(O::mul(hf, hf), O::cbrt(hf)));
+    T friction = O::mul(O::mul(O::mul(O::mul(gdt, nf), nf), qmag), hf_m73);
+    return O::div(O::sub(qn, slope_term), O::add(T(1), friction));
+}
+
+template <typename T>
 __device__ __forceinline__ T face_update_ieee(T qn, T qmag, T hL, T zL, T nL, T hR, T zR, T nR, T g, T dt,
                                               T dx, T h_dry)
 {
@@ -53,12 +65,7 @@ __device__ __forceinline__ T face_update_ieee(T qn, T qmag, T hL, T zL, T nL, T 
     T etaL = O::add(hL, zL), etaR = O::add(hR, zR);
     T hf = O::sub(O::max(etaL, etaR), O::max(zL, zR));
     if (!(hf > h_dry)) return T(0);
-    T nf = O::mul(T(0.5), O::add(nL, nR));
-    T gdt = O::mul(g, dt);
-    T slope_term = O::div(O::mul(O::mul(gdt, hf), O::sub(etaR, etaL)), dx);
-    T hf_m73 = O::div(T(1), O::mul(O::mul(hf, hf), O::cbrt(hf)));
-    T friction = O::mul(O::mul(O::mul(O::mul(gdt, nf), nf), qmag), hf_m73);
-    return O::div(O::sub(qn, slope_term), O::add(T(1), friction));
+    return face_wet_ieee<T>(qn, qmag, etaL, etaR, hf, nL, nR, g, dt, dx);
 }
 
 // |q| of the friction term of a face: its own |q|, or with vec the vector

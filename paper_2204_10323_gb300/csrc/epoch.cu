@@ -213,6 +213,42 @@ __device__ void inflow_solve_warp_f32(const InflowSec &S, const float *sz, const
     }
 }
 
+// The depth above zmin at which a one-warp section carries about Q, in single precision (form 0).
+template <typename T>
+__device__ float level_guess_f32(const InflowSec &S, const T *sz, const T *sn, double zmin, double Q, double dx)
+{
+    const float a = (float)(dx * S.sqrtS), Qf = (float)Q;
+    auto total = [&](float H, float &d) {
+        float s = 0.0f;
+        d = 0.0f;
+        for (int c = threadIdx.x; c < S.ncell; c += 32) {
+            const float hh = H - (float)((double)sz[c] - zmin);
+            if (hh > 0.0f) {
+                const float w = __fdividef(a * __powf(hh, 5.0f / 3.0f), (float)sn[c]);
+                s += w;
+                d += __fdividef(5.0f / 3.0f * w, hh);
+            }
+        }
+        for (int o = 16; o > 0; o >>= 1) {
+            s += __shfl_xor_sync(0xffffffffu, s, o);
+            d += __shfl_xor_sync(0xffffffffu, d, o);
+        }
+        return s;
+    };
+    float H = 1.0f, d, f = total(H, d);
+    while (f < Qf && H < 1e12f) {
+        H *= 2.0f;
+        f = total(H, d);
+    }
+    for (int it = 0; it < 12; it++) {
+        const float step = __fdividef(f - Qf, d);
+        if (!(step > 1e-6f * H)) break;
+        H -= step;
+        f = total(H, d);
+    }
+    return H;
+}
+
 // Block-wide sum of the section's Eq. 5 discharges at level W, and its slope (all threads get them).
 template <typename T>
 __device__ double section_total(const InflowSec &S, const int64_t *cells, const T *z, const T *n,
@@ -293,12 +329,25 @@ __device__ void inflow_body(const Geom &G, const InflowSec *secs, int nsec, cons
         return warp_only ? section_total_warp(S, sz, sn, W, dx, form, d)
                          : section_total(S, cells, z, n, W, dx, form, red, d);
     };
-    double Hb = 1.0, d, f = total_at(zmin + Hb, d);
-    while (f < Q && Hb < 1e12) {
-        Hb *= 2.0;
-        f = total_at(zmin + Hb, d);
+    // FP64, one warp: the level in single precision first (depths above the lowest bed, so that high ground
+    // costs no digits), and the double search from just above it: three or four evaluations of the slow FP64
+    // powers instead of ten
+    double hi = 0.0, d = 0.0, f = -1.0;
+    if (sizeof(T) == 8 && warp_only && form == 0) {
+        const float H = level_guess_f32(S, sz, sn, zmin, Q, dx);
+        hi = zmin + (double)H * (1.0 + 1e-5);
+        f = total_at(hi, d);
     }
-    double lo = zmin, hi = zmin + Hb;                  // f, d: at hi
+    if (!(f >= Q && f < 1e300)) {
+        double Hb = 1.0;
+        f = total_at(zmin + Hb, d);
+        while (f < Q && Hb < 1e12) {
+            Hb *= 2.0;
+            f = total_at(zmin + Hb, d);
+        }
+        hi = zmin + Hb;
+    }
+    double lo = zmin;                                  // f, d: at hi
     for (int it = 0; it < 200 && hi - lo >= 1e-12; it++) {
         const double half = 0.5 * (lo + hi);
         if (!(half > lo && half < hi)) break;          // neighbouring doubles
@@ -322,7 +371,7 @@ __device__ void inflow_body(const Geom &G, const InflowSec *secs, int nsec, cons
     }
     const double W = hi;
     if (tid == 0 && W_out) W_out[(size_t)s * nsec + k] = W;
-    const double total = total_at(W, d);
+    const double total = f;                            // at W
     for (int c = tid; c < S.ncell; c += nthreads) {
         int64_t idx = cells[S.cell0 + c];
         double hh = W - (double)z[idx];
