@@ -53,7 +53,24 @@ cudaError_t launch(void *dst, size_t dpitch, const void *src, size_t spitch, siz
     return cudaGetLastError();
 }
 
+// Copy blockIdx.y of the list.
+__global__ void __launch_bounds__(kThreads) halo_rows_kernel(const HaloRows *__restrict__ copies)
+{
+    const HaloRows c = copies[blockIdx.y];
+    for (int64_t k = (int64_t)blockIdx.x * kThreads + threadIdx.x; k < c.units; k += (int64_t)gridDim.x * kThreads)
+        reinterpret_cast<float4 *>(c.dst)[k] = reinterpret_cast<const float4 *>(c.src)[k];
+}
+
 }  // namespace
+
+cudaError_t launch_halo_rows(const HaloRows *copies, int n, int64_t max_units, cudaStream_t st)
+{
+    if (n <= 0 || max_units <= 0) return cudaSuccess;
+    const int blocks = (int)std::min<int64_t>((max_units + kThreads - 1) / kThreads, 64);
+    for (int k = 0; k < n; k += 65535)
+        halo_rows_kernel<<<dim3(blocks, std::min(n - k, 65535)), kThreads, 0, st>>>(copies + k);
+    return cudaGetLastError();
+}
 
 cudaError_t launch_copy_rows(void *dst, size_t dpitch, const void *src, size_t spitch, size_t width, size_t rows,
                              cudaStream_t st)

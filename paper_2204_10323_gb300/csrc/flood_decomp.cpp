@@ -8,11 +8,15 @@
 // spoils one more row of the strip per step (the scheme's stencil reaches one
 // cell), so after `halo` steps the strip's own rows -- and the face row on
 // either side of them -- are still bit for bit what the whole grid computes.
-// Then the halo rows are copied in again from the neighbours' own rows.  Here
-// all strips live on one GPU, each stepping on a stream of its own (as each
-// would on its own GPU); the copies are device-to-device copies on the
-// decomposition's stream, between two joins of the strips' streams.  The copy
-// list (flood_decomp_plan) names source and destination rows only, so a
+// Then the halo rows are copied in again from the neighbours' own rows, all
+// copies by one launch.  Here all strips live on one GPU.  With the
+// temporal-blocking kernel one launch covers the items of every strip (the
+// ensemble kernel over the strips' arguments) and one launch their epoch
+// starts; the other kernels step each strip on a stream of its own (as each
+// would on its own GPU), joined for the copies.  A launch per strip, a copy per
+// field and neighbour and two joins per exchange kept the GPU waiting for the
+// host: 4096^2 in 4 strips took 77 us a step against 41 of the whole grid.  The
+// copy list (flood_decomp_plan) names source and destination rows only, so a
 // transport between GPUs would carry the same list (each row into the
 // receiving GPU's own memory).
 //
@@ -48,6 +52,17 @@ struct flood_decomp {
     std::vector<int32_t> rows;               // 4 per part: y0, y1, a, b
     std::vector<flood_halo_copy> copies;
     Ctrl **ctrls_dev = nullptr;              // the parts' control blocks (device array)
+    // device tables per phase: 0 the parts' current buffers as of build_tables, 1 the other halves
+    std::vector<int> cur0;                   // the parts' halves at build_tables
+    HaloRows *halo_dev[2] = {nullptr, nullptr};
+    int64_t halo_units = 0;                  // 16-byte units of the longest copy
+    bool batched = false;                    // one launch for all parts (FP32, temporal blocking, no caller's launch shape)
+    StepArgs<float> *args_dev[2] = {nullptr, nullptr};
+    int *base_dev = nullptr;                 // item prefix, n_parts + 1
+    int total_items = 0, mode = 0;
+    EpochArgs<float> *etab_dev = nullptr;
+    int2 *tasks_dev = nullptr;               // (part, inflow section)
+    int n_tasks = 0;
     int64_t step = 0;
     int since = 0;                           // steps since the halos were last refreshed
     int sticky = 0;
@@ -95,7 +110,7 @@ void *field_plane(flood_handle *h, int field)
 // The decomposition's stream waits for every part's stream.
 flood_status join_lanes(flood_decomp *d)
 {
-    for (int r = 0; r < d->n_parts; r++) {
+    for (size_t r = 0; r < d->lanes.size(); r++) {
         DCK(cudaEventRecord(d->lane_ev[r], d->lanes[r]));
         DCK(cudaStreamWaitEvent(d->stream, d->lane_ev[r], 0));
     }
@@ -105,8 +120,59 @@ flood_status join_lanes(flood_decomp *d)
 // Every part's stream waits for the decomposition's stream.
 flood_status fork_lanes(flood_decomp *d)
 {
+    if (d->lanes.empty()) return FLOOD_OK;
     DCK(cudaEventRecord(d->main_ev, d->stream));
-    for (int r = 0; r < d->n_parts; r++) DCK(cudaStreamWaitEvent(d->lanes[r], d->main_ev, 0));
+    for (size_t r = 0; r < d->lanes.size(); r++) DCK(cudaStreamWaitEvent(d->lanes[r], d->main_ev, 0));
+    return FLOOD_OK;
+}
+
+int phase(const flood_decomp *d) { return d->parts[0]->cur ^ d->cur0[0]; }
+
+// The device tables of both phases, for the halves that the parts hold now (all parts flip theirs with
+// every launch; a state from the host flips them too, and may have failed for some parts before).
+flood_status build_tables(flood_decomp *d)
+{
+    const int n = d->n_parts;
+    d->cur0.resize(n);
+    for (int r = 0; r < n; r++) d->cur0[r] = d->parts[r]->cur;
+    for (int ph = 0; ph < 2; ph++) {
+        for (int r = 0; r < n; r++) d->parts[r]->cur = d->cur0[r] ^ ph;
+        std::vector<HaloRows> halo;
+        for (const flood_halo_copy &c : d->copies) {
+            flood_handle *s = d->parts[c.src_part], *t = d->parts[c.dst_part];
+            const size_t row_bytes = (size_t)s->geo.pitch * d->esz;        // a multiple of 128
+            HaloRows e;
+            e.src = (const char *)field_plane(s, c.field) + (size_t)c.src_row * row_bytes;
+            e.dst = (char *)field_plane(t, c.field) + (size_t)c.dst_row * row_bytes;
+            e.units = (int64_t)((size_t)c.rows * row_bytes / 16);
+            d->halo_units = std::max(d->halo_units, e.units);
+            halo.push_back(e);
+        }
+        std::vector<StepArgs<float>> args(d->batched ? n : 0);
+        std::vector<int> base(1, 0);
+        if (d->batched) {
+            int rows = 0, edge = 0;
+            tiled_rows(d->nx, d->ny, d->parts[0]->k_per_launch, d->mode, &rows, &edge);   // as for the whole grid
+            for (int r = 0; r < n; r++) {
+                args[r] = step_args_f32(d->parts[r], 0);
+                args[r].tile_y = std::min(rows, d->parts[r]->geo.ny);
+                args[r].tile_x = std::min(edge, d->parts[r]->geo.ny);
+                base.push_back(base.back() +
+                               tiled_items(d->parts[r]->geo, args[r].tile_y, args[r].tile_x, d->parts[r]->k_per_launch));
+            }
+            d->total_items = base.back();
+        }
+        cudaError_t e = cudaSuccess;
+        if (!halo.empty())
+            e = cudaMemcpyAsync(d->halo_dev[ph], halo.data(), halo.size() * sizeof(HaloRows), cudaMemcpyHostToDevice, d->stream);
+        if (e == cudaSuccess && d->batched)
+            e = cudaMemcpyAsync(d->args_dev[ph], args.data(), n * sizeof(StepArgs<float>), cudaMemcpyHostToDevice, d->stream);
+        if (e == cudaSuccess && d->batched && ph == 0)
+            e = cudaMemcpyAsync(d->base_dev, base.data(), (n + 1) * sizeof(int), cudaMemcpyHostToDevice, d->stream);
+        if (e == cudaSuccess) e = cudaStreamSynchronize(d->stream);
+        for (int r = 0; r < n; r++) d->parts[r]->cur = d->cur0[r];
+        if (e != cudaSuccess) return dfail(d, FLOOD_ERR_CUDA, std::string("decomposition tables: ") + cudaGetErrorString(e));
+    }
     return FLOOD_OK;
 }
 
@@ -115,14 +181,24 @@ flood_status fork_lanes(flood_decomp *d)
 flood_status exchange(flood_decomp *d)
 {
     NvtxRange range("flood: halo exchange");
-    for (const flood_halo_copy &c : d->copies) {
-        flood_handle *s = d->parts[c.src_part], *t = d->parts[c.dst_part];
-        const size_t row_bytes = (size_t)s->geo.pitch * d->esz;
-        const char *src = (const char *)field_plane(s, c.field) + (size_t)c.src_row * row_bytes;
-        char *dst = (char *)field_plane(t, c.field) + (size_t)c.dst_row * row_bytes;
-        DCK(cudaMemcpyAsync(dst, src, (size_t)c.rows * row_bytes, cudaMemcpyDeviceToDevice, d->stream));
-    }
+    if (!d->copies.empty()) DCK(launch_halo_rows(d->halo_dev[phase(d)], (int)d->copies.size(), d->halo_units, d->stream));
     d->since = 0;
+    return FLOOD_OK;
+}
+
+// m steps of every part from step s of the epoch, one launch per up to four steps for all of them.
+flood_status step_batched(flood_decomp *d, int s, int m)
+{
+    for (int done = 0; done < m;) {
+        const int k = std::min(d->parts[0]->k_per_launch, m - done);
+        DCK(launch_step_tiled_ensemble(d->args_dev[phase(d)], d->base_dev, d->n_parts, d->total_items, k, s + done,
+                                       s + done + k == d->E ? 1 : 0, d->mode, d->stream));
+        for (flood_handle *h : d->parts) {
+            h->cur = 1 - h->cur;
+            h->step += k;
+        }
+        done += k;
+    }
     return FLOOD_OK;
 }
 
@@ -224,19 +300,52 @@ extern "C" flood_status flood_decomp_create(const flood_grid *grid, const void *
         d->parts.push_back(h);
     }
     d->stream = d->parts[0]->stream;
-    // a stream per part: the parts step side by side, as on separate GPUs
-    d->lanes.assign(n_parts, nullptr);
-    d->lane_ev.assign(n_parts, nullptr);
-    if (cudaEventCreateWithFlags(&d->main_ev, cudaEventDisableTiming) != cudaSuccess)
-        return bail(FLOOD_ERR_CUDA, "event creation");
-    for (int r = 0; r < n_parts; r++) {
-        if (cudaStreamCreateWithFlags(&d->lanes[r], cudaStreamNonBlocking) != cudaSuccess ||
-            cudaEventCreateWithFlags(&d->lane_ev[r], cudaEventDisableTiming) != cudaSuccess)
-            return bail(FLOOD_ERR_CUDA, "stream creation");
+    d->batched = d->prec == FLOOD_F32 && d->parts[0]->kernel == FLOOD_KERNEL_TILED && o.tile_x == 0 && o.tile_y == 0;
+    d->mode = (o.theta != 1.0 ? 1 : 0) | (o.friction != 0 ? 2 : 0);
+    if (!d->batched) {
+        // a stream per part: the parts step side by side, as on separate GPUs
+        d->lanes.assign(n_parts, nullptr);
+        d->lane_ev.assign(n_parts, nullptr);
+        if (cudaEventCreateWithFlags(&d->main_ev, cudaEventDisableTiming) != cudaSuccess)
+            return bail(FLOOD_ERR_CUDA, "event creation");
+        for (int r = 0; r < n_parts; r++) {
+            if (cudaStreamCreateWithFlags(&d->lanes[r], cudaStreamNonBlocking) != cudaSuccess ||
+                cudaEventCreateWithFlags(&d->lane_ev[r], cudaEventDisableTiming) != cudaSuccess)
+                return bail(FLOOD_ERR_CUDA, "stream creation");
+        }
     }
     // the parts' set-up on the caller's stream is done before their own streams start
     if (cudaStreamSynchronize(d->stream) != cudaSuccess) return bail(FLOOD_ERR_CUDA, "part set-up");
-    for (int r = 0; r < n_parts; r++) d->parts[r]->stream = d->lanes[r];
+    for (size_t r = 0; r < d->lanes.size(); r++) d->parts[r]->stream = d->lanes[r];
+    for (int ph = 0; ph < 2; ph++) {
+        d->halo_dev[ph] = (HaloRows *)raw_device_alloc(std::max<size_t>(ncopy, 1) * sizeof(HaloRows), d->stream);
+        if (!d->halo_dev[ph]) return bail(FLOOD_ERR_OOM, "device allocation failed");
+        if (!d->batched) continue;
+        d->args_dev[ph] = (StepArgs<float> *)raw_device_alloc(n_parts * sizeof(StepArgs<float>), d->stream);
+        if (!d->args_dev[ph]) return bail(FLOOD_ERR_OOM, "device allocation failed");
+    }
+    if (d->batched) {
+        std::vector<EpochArgs<float>> et(n_parts);
+        std::vector<int2> tk;
+        for (int r = 0; r < n_parts; r++) {
+            et[r] = epoch_args_f32(d->parts[r]);
+            for (int k = 0; k < d->parts[r]->n_in; k++) tk.push_back(make_int2(r, k));
+        }
+        d->n_tasks = (int)tk.size();
+        d->base_dev = (int *)raw_device_alloc((n_parts + 1) * sizeof(int), d->stream);
+        d->etab_dev = (EpochArgs<float> *)raw_device_alloc(n_parts * sizeof(EpochArgs<float>), d->stream);
+        d->tasks_dev = (int2 *)raw_device_alloc(std::max<size_t>(tk.size(), 1) * sizeof(int2), d->stream);
+        if (!d->base_dev || !d->etab_dev || !d->tasks_dev) return bail(FLOOD_ERR_OOM, "device allocation failed");
+        if (cudaMemcpyAsync(d->etab_dev, et.data(), n_parts * sizeof(EpochArgs<float>), cudaMemcpyHostToDevice, d->stream) ||
+            (!tk.empty() &&
+             cudaMemcpyAsync(d->tasks_dev, tk.data(), tk.size() * sizeof(int2), cudaMemcpyHostToDevice, d->stream)) ||
+            cudaStreamSynchronize(d->stream))
+            return bail(FLOOD_ERR_CUDA, "epoch table upload");
+    }
+    if (build_tables(d)) {
+        const std::string m = d->err;
+        return bail(FLOOD_ERR_CUDA, m);
+    }
     d->ctrls_dev = (Ctrl **)raw_device_alloc(n_parts * sizeof(Ctrl *), d->stream);
     if (!d->ctrls_dev) return bail(FLOOD_ERR_OOM, "device allocation failed");
     std::vector<Ctrl *> ctrls(n_parts);
@@ -272,6 +381,17 @@ extern "C" flood_status flood_decomp_step(flood_decomp *d, int64_t n_steps)
             if (due && (st = exchange(d))) return st;
             if ((st = fork_lanes(d))) return st;
         }
+        const int m = (int)std::min<int64_t>(std::min(d->halo - d->since, E - s), n_steps - done);
+        if (d->batched) {
+            if (s == 0)
+                DCK(launch_epoch_batched<float>(d->etab_dev, d->n_parts, d->tasks_dev, d->n_tasks, E, d->n_tasks > 0, d->stream));
+            flood_status st = step_batched(d, s, m);     // (the kernel measures the own rows' maximum)
+            if (st) return st;
+            d->step += m;
+            d->since += m;
+            done += m;
+            continue;
+        }
         if (s == 0) {
             // epoch start: every part chooses dt from the whole grid's h_max, and solves Eq. 6
             for (int r = 0; r < d->n_parts; r++) {
@@ -280,7 +400,6 @@ extern "C" flood_status flood_decomp_step(flood_decomp *d, int64_t n_steps)
                 if (st) return part_fail(d, r, st);
             }
         }
-        const int m = (int)std::min<int64_t>(std::min(d->halo - d->since, E - s), n_steps - done);
         for (int r = 0; r < d->n_parts; r++) {
             flood_handle *h = d->parts[r];
             for (int k_done = 0; k_done < m;) {
@@ -380,6 +499,10 @@ extern "C" flood_status flood_decomp_write_state(flood_decomp *d, const void *de
             return dfail(d, st, std::string("part ") + std::to_string(r) + ": " + flood_last_error(d->parts[r]));
         }
     }
+    {
+        flood_status st = build_tables(d);     // a state from the host has swapped the parts' halves
+        if (st) return st;
+    }
     d->since = 0;
     d->sticky = FLOOD_OK;
     d->err.clear();
@@ -403,7 +526,9 @@ extern "C" flood_status flood_decomp_destroy(flood_decomp *d)
         if (r < d->lanes.size() && d->lanes[r] && h->stream == d->lanes[r]) h->stream = d->stream;
         flood_destroy(h);
     }
-    if (d->ctrls_dev) c10::cuda::CUDACachingAllocator::raw_delete(d->ctrls_dev);
+    for (void *p : {(void *)d->ctrls_dev, (void *)d->halo_dev[0], (void *)d->halo_dev[1], (void *)d->args_dev[0], (void *)d->args_dev[1],
+                    (void *)d->base_dev, (void *)d->etab_dev, (void *)d->tasks_dev})
+        if (p) c10::cuda::CUDACachingAllocator::raw_delete(p);
     for (cudaEvent_t e : d->lane_ev)
         if (e) cudaEventDestroy(e);
     if (d->main_ev) cudaEventDestroy(d->main_ev);

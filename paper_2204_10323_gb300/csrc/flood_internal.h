@@ -105,6 +105,9 @@ cudaError_t launch_step_tma(const StepArgs<float> &a, cudaStream_t st);
 // Temporal blocking over many grids: the items of grid k are base[k] .. base[k+1] - 1 (tiled_items per
 // grid, table[k].tile_y rows per item, tile_x in the edge strips), k_steps steps from s0.
 int tiled_items(const Geom &g, int rows, int rows_edge, int k_steps);
+// Rows per work item (inner strips, and the one or two strips with the borders x = 0 and x = nx) for a grid
+// alone on the GPU.
+void tiled_rows(int nx, int ny, int K, int mode, int *rows, int *rows_edge);
 cudaError_t launch_step_tiled_ensemble(const StepArgs<float> *table, const int *base, int n, int total_items,
                                        int k_steps, int s0, int want_hmax, int mode, cudaStream_t st);
 void stream_launch_shape(const Geom &g, int tile_x, int tile_y, int *warps, int *rows);
@@ -144,6 +147,13 @@ cudaError_t launch_hmax(const Geom &g, const T *h, Ctrl *ctrl, cudaStream_t st);
 // rows of `width` bytes from src to dst (device memory of the current device), pitches in bytes.
 cudaError_t launch_copy_rows(void *dst, size_t dpitch, const void *src, size_t spitch, size_t width, size_t rows,
                              cudaStream_t st);
+// n copies of `units` 16-byte units each (device memory, 16-byte aligned), max_units the longest.
+struct HaloRows {
+    const void *src;
+    void *dst;
+    int64_t units;
+};
+cudaError_t launch_halo_rows(const HaloRows *copies, int n, int64_t max_units, cudaStream_t st);
 // Block mean (f x f, partial blocks at the far edges) of a ny x nx field into ceil(ny/f) x ceil(nx/f).
 template <typename T>
 cudaError_t launch_coarsen(const T *src, int nx, int ny, int f, T *dst, cudaStream_t st);

@@ -37,9 +37,6 @@
 
 namespace flood {
 
-// Rows per work item (inner strips, and the one or two strips with the borders x = 0
-// and x = nx) that the launcher chooses for a grid (step_tiled.cu).
-void tiled_rows(int nx, int ny, int K, int mode, int *rows, int *rows_edge);
 // Rows per work item and pipelines for `resident` pipelines that walk the items in turn.
 void tiled_split_dynamic(int n_strips, int ny, int resident, int K, int *chunk_rows, int *blocks);
 
@@ -423,8 +420,9 @@ __device__ __forceinline__ void tiled_item(const StepArgs<float> &a, const int s
                             const float2 g0 = f2unpack(fin.a), g1 = f2unpack(fin.b);
                             const size_t ro = (size_t)rr * P + lane_off;
                             const bool north = !kSteady && rr == ny - 1;   // the grid's north face row too
+                            const bool maximum = want_hmax && rr >= G.led_j0 && rr < G.led_j1;   // a part's own rows
                             if (kEdge ? full : lane >= 1 && lane <= kOut / 4) {
-                                if (want_hmax) hmax = max_nan(max_nan(hmax, max_nan(g0.x, g0.y)), max_nan(g1.x, g1.y));
+                                if (maximum) hmax = max_nan(max_nan(hmax, max_nan(g0.x, g0.y)), max_nan(g1.x, g1.y));
                                 row_store(a.h_out + ro, fin);
                                 row_store(a.qx_out + ro, x0r);
                                 row_store(a.qy_out + ro, y0r);
@@ -435,7 +433,7 @@ __device__ __forceinline__ void tiled_item(const StepArgs<float> &a, const int s
                                 for (int k = 0; k < 4; k++) {
                                     const int c = c0 + k;
                                     if (c < own_hi) {
-                                        if (want_hmax) hmax = max_nan(hmax, f[k]);
+                                        if (maximum) hmax = max_nan(hmax, f[k]);
                                         a.h_out[ro + k] = f[k];
                                         a.qy_out[ro + k] = row_get(y0r, k);
                                         if (north) a.qy_out[ro + P + k] = row_get(qs, k);
