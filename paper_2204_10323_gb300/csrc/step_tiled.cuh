@@ -184,7 +184,7 @@ struct alignas(16) TiledSmem {
     float raw[kAhead][3][128];           // level 1's rows in flight: h, qx, n
     float qy[kMode ? 4 : kAhead][128];   // and qy (the scheme options read it one row further on)
     float z[kRowsZ][128];
-    float c[4][2][128];                  // face_c of a row's west and south faces, for levels 2 .. K
+    float c[4][4][128];                  // face_c and the higher bed of a row's west and south faces, for levels 2 .. K
     int gauge[32][3];                    // gauges in the item's own cells: row, staged column, index
 };
 
@@ -318,7 +318,7 @@ __device__ __forceinline__ void tiled_item(const StepArgs<float> &a, const int s
             const int rstart = jb == 0 ? 0 : jb + (s - 1);
             if (kSteady || (r >= rstart && r <= ny && r <= y1 + K - s)) {
                 const bool row = kSteady || r < ny;    // r == ny: only the north border faces
-                Row4 z{0, 0}, pz{0, 0}, fcx{0, 0}, fcy{0, 0};
+                Row4 z{0, 0}, pz{0, 0}, fcx{0, 0}, fcy{0, 0}, zx{0, 0}, zy{0, 0};
                 if (row) z = row_load(&sm.z[r & (kRowsZ - 1)][4 * lane]);
                 if (kSteady || r > 0) pz = row_load(&sm.z[(r - 1) & (kRowsZ - 1)][4 * lane]);
                 if (s == 1) {
@@ -336,15 +336,22 @@ __device__ __forceinline__ void tiled_item(const StepArgs<float> &a, const int s
                         fcy.a = face_c(f2add(pn.a, n.a), Kc);
                         fcy.b = face_c(f2add(pn.b, n.b), Kc);
                         pn = n;
+                        const Row4 zl = row_left(z, from_left(z));
+                        zx = Row4{f2max(zl.a, z.a), f2max(zl.b, z.b)};
+                        zy = Row4{f2max(pz.a, z.a), f2max(pz.b, z.b)};
                         if (K > 1) {
                             row_store(&sm.c[r & 3][0][4 * lane], fcx);
                             row_store(&sm.c[r & 3][1][4 * lane], fcy);
+                            row_store(&sm.c[r & 3][2][4 * lane], zx);
+                            row_store(&sm.c[r & 3][3][4 * lane], zy);
                         }
                     }
                     issue(j + kAhead);                 // into the slots just read
                 } else if (row) {
                     fcx = row_load(&sm.c[r & 3][0][4 * lane]);
                     fcy = row_load(&sm.c[r & 3][1][4 * lane]);
+                    zx = row_load(&sm.c[r & 3][2][4 * lane]);
+                    zy = row_load(&sm.c[r & 3][3][4 * lane]);
                 }
                 if (!kSteady && r == rstart && jb > 0) {
                     sh[s - 1] = ch;                    // halo row: only becomes the previous row
@@ -369,8 +376,8 @@ __device__ __forceinline__ void tiled_item(const StepArgs<float> &a, const int s
                         } else {
                             cq = Row4{face_cq(fcy.a, cy.a), face_cq(fcy.b, cy.b)};
                         }
-                        qs.a = faces2(f2sub(f2max(ep.a, e.a), f2max(pz.a, z.a)), f2sub(e.a, ep.a), qn.a, cq.a, Kc);
-                        qs.b = faces2(f2sub(f2max(ep.b, e.b), f2max(pz.b, z.b)), f2sub(e.b, ep.b), qn.b, cq.b, Kc);
+                        qs.a = faces2(f2sub(f2max(ep.a, e.a), zy.a), f2sub(e.a, ep.a), qn.a, cq.a, Kc);
+                        qs.b = faces2(f2sub(f2max(ep.b, e.b), zy.b), f2sub(e.b, ep.b), qn.b, cq.b, Kc);
                     } else {
                         // rows 0 and ny: Eq. 5-6
                         float v[4] = {0.0f, 0.0f, 0.0f, 0.0f};
@@ -404,7 +411,7 @@ __device__ __forceinline__ void tiled_item(const StepArgs<float> &a, const int s
                         fin.a = f2fma(f2dup(Kc.dtdx), f2add(dx0, f2sub(y0r.a, qs.a)), h0.a);
                         fin.b = f2fma(f2dup(Kc.dtdx), f2add(dx1, f2sub(y0r.b, qs.b)), h0.b);
                         const float2 f0 = f2unpack(fin.a), f1 = f2unpack(fin.b);
-                        if (fminf(fminf(f0.x, f0.y), fminf(f1.x, f1.y)) < 0.0f) {   // rare: clip, book the removed volume
+                        if ((__float_as_int(f0.x) | __float_as_int(f0.y) | __float_as_int(f1.x) | __float_as_int(f1.y)) < 0) {   // a sign bit (rare): clip, book the removed volume
                             const bool book = rr >= y0 && rr < y1 && rr >= G.led_j0 && rr < G.led_j1;
                             float v[4] = {f0.x, f0.y, f1.x, f1.y};
 #pragma unroll
@@ -447,7 +454,7 @@ __device__ __forceinline__ void tiled_item(const StepArgs<float> &a, const int s
                     // finished one the next level's input
                     Row4 qx{0, 0};
                     if (row) {
-                        const Row4 el = row_left(e, from_left(e)), zl = row_left(z, from_left(z));
+                        const Row4 el = row_left(e, from_left(e));
                         Row4 qn = cx, cq;
                         if constexpr (kTheta) {
                             const Row4 l = row_left(cx, from_left(cx)), n = row_right(cx, from_right(cx));
@@ -465,8 +472,8 @@ __device__ __forceinline__ void tiled_item(const StepArgs<float> &a, const int s
                         const float2 e0 = f2unpack(e.a), e1 = f2unpack(e.b), l0 = f2unpack(el.a);
                         const unsigned long long s0_ = f2pack(__fsub_rn(e0.x, l0.x), __fsub_rn(e0.y, e0.x));
                         const unsigned long long s1_ = f2pack(__fsub_rn(e1.x, e0.y), __fsub_rn(e1.y, e1.x));
-                        qx.a = faces2(f2sub(f2max(el.a, e.a), f2max(zl.a, z.a)), s0_, qn.a, cq.a, Kc);
-                        qx.b = faces2(f2sub(f2max(el.b, e.b), f2max(zl.b, z.b)), s1_, qn.b, cq.b, Kc);
+                        qx.a = faces2(f2sub(f2max(el.a, e.a), zx.a), s0_, qn.a, cq.a, Kc);
+                        qx.b = faces2(f2sub(f2max(el.b, e.b), zx.b), s1_, qn.b, cq.b, Kc);
                     }
                     const Row4 hx = x0r, hy = y0r;
                     h0 = ch;
