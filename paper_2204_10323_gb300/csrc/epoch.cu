@@ -436,20 +436,46 @@ __global__ void __launch_bounds__(kInflowThreads) inflow_batched_kernel(const Ep
     if (kBegin) epoch_commit(A.geo, A.ctrl, A.t_list, gridDim.x, nullptr, gridDim.x * A.nsec);
 }
 
-// Rows over blocks, columns over threads; the maximum is exact in the state's
-// own precision, and a NaN, once seen, is kept.
+// A thread's share of the depths, in 16-byte vectors along the rows (they start on 128-byte boundaries), two rows
+// in flight: fn(value) per depth.  Rows over the blocks' warps, vectors over lanes.  One element at a time, a row
+// per block, the depth maximum of 1024^2 took 11.8 us.
+template <typename T, typename Fn>
+__device__ __forceinline__ void for_depths(const Geom &G, const T *h, Fn fn)
+{
+    constexpr int V = 16 / sizeof(T);
+    struct alignas(16) Vec {
+        T v[V];
+    };
+    const int lane = threadIdx.x & 31, warps = gridDim.x * (blockDim.x >> 5);
+    const int whole = G.nx / V;                        // whole vectors of a row
+    for (int j = blockIdx.x * (blockDim.x >> 5) + (threadIdx.x >> 5); j < G.ny; j += warps) {
+        const T *row = h + (size_t)j * G.pitch;
+        int i = lane;
+        for (; i + 96 < whole; i += 128) {
+            Vec x[4];
+#pragma unroll
+            for (int u = 0; u < 4; u++) x[u] = reinterpret_cast<const Vec *>(row)[i + 32 * u];
+#pragma unroll
+            for (int u = 0; u < 4; u++)
+#pragma unroll
+                for (int k = 0; k < V; k++) fn(x[u].v[k]);
+        }
+        for (; i < whole; i += 32) {
+            const Vec x = reinterpret_cast<const Vec *>(row)[i];
+#pragma unroll
+            for (int k = 0; k < V; k++) fn(x.v[k]);
+        }
+        for (i = whole * V + lane; i < G.nx; i += 32) fn(row[i]);
+    }
+}
+
+// The maximum is exact in the state's own precision, and a NaN, once seen, is kept.
 template <typename T>
-__global__ void hmax_kernel(Geom G, const T *h, Ctrl *ctrl)
+__global__ void __launch_bounds__(256) hmax_kernel(Geom G, const T *h, Ctrl *ctrl)
 {
     __shared__ double red[32];
     T m = T(0);
-    for (int j = blockIdx.x; j < G.ny; j += gridDim.x) {
-        const T *row = h + (size_t)j * G.pitch;
-        for (int i = threadIdx.x; i < G.nx; i += blockDim.x) {
-            const T v = row[i];
-            m = (v > m || v != v) ? v : m;
-        }
-    }
+    for_depths(G, h, [&](T v) { m = (v > m || v != v) ? v : m; });
     const double bm = block_reduce<true>((double)m, red);
     if (threadIdx.x == 0) atomic_max_nonneg(&ctrl->hmax_bits, bm);
 }
@@ -483,16 +509,13 @@ struct ThreadSum<float> {
     __device__ double value() const { return (double)s + (double)c; }
 };
 
-// Pass 1: block b sums rows b, b + nb, ... (fixed order for a fixed launch shape).
+// Pass 1: a fixed share of the rows per block (fixed order for a fixed launch shape).
 template <typename T>
-__global__ void volume_partial_kernel(Geom G, const T *h, double *partials)
+__global__ void __launch_bounds__(256) volume_partial_kernel(Geom G, const T *h, double *partials)
 {
     __shared__ double red[32];
     ThreadSum<T> acc;
-    for (int j = blockIdx.x; j < G.ny; j += gridDim.x) {
-        const T *row = h + (size_t)j * G.pitch;
-        for (int i = threadIdx.x; i < G.nx; i += blockDim.x) acc.add(row[i]);
-    }
+    for_depths(G, h, [&](T v) { acc.add(v); });
     const double s = block_reduce<false>(acc.value(), red);
     if (threadIdx.x == 0) partials[blockIdx.x] = s;
 }
@@ -578,7 +601,7 @@ cudaError_t launch_inflow(const EpochArgs<T> &A, int E, bool begin, const double
 template <typename T>
 cudaError_t launch_hmax(const Geom &g, const T *h, Ctrl *ctrl, cudaStream_t st)
 {
-    const int blocks = g.ny < 152 * 8 ? g.ny : 152 * 8;
+    const int rows = (g.ny + 7) / 8, blocks = rows < 152 * 8 ? rows : 152 * 8;   // a row per warp
     hmax_kernel<T><<<blocks, 256, 0, st>>>(g, h, ctrl);
     return cudaGetLastError();
 }
@@ -587,8 +610,9 @@ template <typename T>
 cudaError_t launch_volume(const Geom &g, const T *h, double *partials, int n_partials, double *out,
                           cudaStream_t st)
 {
-    volume_partial_kernel<T><<<n_partials, 256, 0, st>>>(g, h, partials);
-    volume_final_kernel<<<1, 256, 0, st>>>(partials, n_partials, g.dx * g.dx, out);
+    const int rows = (g.ny + 7) / 8, blocks = rows < 1 ? 1 : rows < n_partials ? rows : n_partials;   // a row per warp
+    volume_partial_kernel<T><<<blocks, 256, 0, st>>>(g, h, partials);
+    volume_final_kernel<<<1, 256, 0, st>>>(partials, blocks, g.dx * g.dx, out);
     return cudaGetLastError();
 }
 

@@ -178,14 +178,19 @@ __device__ __forceinline__ unsigned long long theta_q_x2(unsigned long long q, u
     return f2fma(f2pack(k.theta, k.theta), q, f2mul(f2pack(k.w, k.w), f2add(q_prev, q_next)));
 }
 
-// q_norm for two faces (packed q and the four orthogonal neighbours a, b, c, d).
+// q_norm for two faces: packed q, and the sums a + b and c + d of the orthogonal neighbours.
+__device__ __forceinline__ unsigned long long q_norm_sums_x2(unsigned long long q, unsigned long long ab, unsigned long long cd)
+{
+    const unsigned long long qo = f2mul(f2pack(0.25f, 0.25f), f2add(ab, cd));
+    const float2 s = f2unpack(f2fma(q, q, f2mul(qo, qo)));
+    return f2pack(sqrt_fast(s.x), sqrt_fast(s.y));
+}
+
 __device__ __forceinline__ unsigned long long q_norm_x2(unsigned long long q, unsigned long long a,
                                                         unsigned long long b, unsigned long long c,
                                                         unsigned long long d)
 {
-    const unsigned long long qo = f2mul(f2pack(0.25f, 0.25f), f2add(f2add(a, b), f2add(c, d)));
-    const float2 s = f2unpack(f2fma(q, q, f2mul(qo, qo)));
-    return f2pack(sqrt_fast(s.x), sqrt_fast(s.y));
+    return q_norm_sums_x2(q, f2add(a, b), f2add(c, d));
 }
 
 // Eq. 3 at one face: eta_L, eta_R water levels, zmax = max(z_L, z_R),

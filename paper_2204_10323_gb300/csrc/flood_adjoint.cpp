@@ -176,8 +176,10 @@ flood_status ensure_epoch(Sweep &S, int64_t e)
     double *dtl = S.dt_log + ie;
     if (!S.logged[ie]) {
         CKA(cudaMemsetAsync(&h->ctrl->hmax_bits, 0, sizeof(unsigned long long), h->stream));
-        if (h->prec == FLOOD_F32) CKA(launch_hmax<float>(h->geo, (const float *)S.src.h, h->ctrl, h->stream));
-        else CKA(launch_hmax<double>(h->geo, (const double *)S.src.h, h->ctrl, h->stream));
+        if (h->geo.dt_mode != 1) {         // a constant step does not ask for the depth maximum
+            if (h->prec == FLOOD_F32) CKA(launch_hmax<float>(h->geo, (const float *)S.src.h, h->ctrl, h->stream));
+            else CKA(launch_hmax<double>(h->geo, (const double *)S.src.h, h->ctrl, h->stream));
+        }
         flood_status st = begin_epoch(h);
         if (st) return st;
         CKA(cudaMemcpyAsync(dtl, &h->ctrl->dt, sizeof(double), cudaMemcpyDeviceToDevice, h->stream));
@@ -585,12 +587,10 @@ extern "C" flood_status flood_adjoint(flood_handle *h, int64_t n_steps, const in
         CKF(cudaMemcpyAsync(cells_dev, gauge_cells, n_gauges * sizeof(int64_t), cudaMemcpyHostToDevice, h->stream));
         CKF(cudaMemcpyAsync(rc_dev, rc.data(), n_gauges * sizeof(int2), cudaMemcpyHostToDevice, h->stream));
     }
-    for (int b = 0; b < 2; b++) {
-        CKF(cudaMemsetAsync(S.lh[b], 0, S.plane, h->stream));
-        CKF(cudaMemsetAsync(S.lqx[b], 0, S.plane, h->stream));
-        CKF(cudaMemsetAsync(S.lqy[b], 0, S.plane_y, h->stream));
-    }
-    CKF(cudaMemsetAsync(S.lhu, 0, S.plane, h->stream));
+    // the adjoint after the last step; every reverse step writes the other half whole (and lhu before it is read)
+    CKF(cudaMemsetAsync(S.lh[0], 0, S.plane, h->stream));
+    CKF(cudaMemsetAsync(S.lqx[0], 0, S.plane, h->stream));
+    CKF(cudaMemsetAsync(S.lqy[0], 0, S.plane_y, h->stream));
     CKF(cudaMemsetAsync(S.gn, 0, P * h->geo.ny * sizeof(double), h->stream));
     if (S.gn_in) CKF(cudaMemsetAsync(S.gn_in, 0, (size_t)S.n_in_cells * sizeof(double), h->stream));
     S.cells = cells_dev;

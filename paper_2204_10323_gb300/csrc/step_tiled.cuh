@@ -299,7 +299,7 @@ __device__ __forceinline__ void tiled_item(const StepArgs<float> &a, const int s
     }
 
     Row4 sh[K], sx[K], sy[K];                          // per level: the previous row's old depth and new faces
-    Row4 ox[K], oy[K];                                 // and its old qx (kVec) and qy (kTheta)
+    Row4 ox[K], oy[K];                                 // the sums of its neighbouring old qx (kVec), its old qy (kTheta)
     Row4 pn{0, 0};                                     // n of the previous row (level 1)
 #pragma unroll
     for (int s = 0; s < K; s++) sh[s] = sx[s] = sy[s] = ox[s] = oy[s] = Row4{0, 0};
@@ -356,10 +356,18 @@ __device__ __forceinline__ void tiled_item(const StepArgs<float> &a, const int s
                 if (!kSteady && r == rstart && jb > 0) {
                     sh[s - 1] = ch;                    // halo row: only becomes the previous row
                     if constexpr (kTheta) oy[s - 1] = cy;
-                    if constexpr (kVec) ox[s - 1] = cx;
+                    if constexpr (kVec) {
+                        const Row4 c1 = row_right(cx, from_right(cx));
+                        ox[s - 1] = Row4{f2add(cx.a, c1.a), f2add(cx.b, c1.b)};
+                    }
                 } else {
                     Row4 &h0 = sh[s - 1], &x0r = sx[s - 1], &y0r = sy[s - 1];
                     const Row4 e{f2add(ch.a, z.a), f2add(ch.b, z.b)};
+                    Row4 px{0, 0};                     // qx of the row's cells, west + east (kVec)
+                    if constexpr (kVec) {
+                        const Row4 c1 = row_right(cx, from_right(cx));
+                        px = Row4{f2add(cx.a, c1.a), f2add(cx.b, c1.b)};
+                    }
                     // ---- new south faces of row r
                     Row4 qs;
                     if (kSteady || (r > 0 && r < ny)) {
@@ -370,9 +378,8 @@ __device__ __forceinline__ void tiled_item(const StepArgs<float> &a, const int s
                             qn.b = theta_q_x2(cy.b, oy[s - 1].b, cyn.b, Kc);
                         }
                         if constexpr (kVec) {          // the mean of the old qx of rows r - 1 and r around the face
-                            const Row4 o1 = row_right(ox[s - 1], from_right(ox[s - 1])), c1 = row_right(cx, from_right(cx));
-                            cq.a = f2mul(fcy.a, q_norm_x2(cy.a, ox[s - 1].a, o1.a, cx.a, c1.a));
-                            cq.b = f2mul(fcy.b, q_norm_x2(cy.b, ox[s - 1].b, o1.b, cx.b, c1.b));
+                            cq.a = f2mul(fcy.a, q_norm_sums_x2(cy.a, ox[s - 1].a, px.a));
+                            cq.b = f2mul(fcy.b, q_norm_sums_x2(cy.b, ox[s - 1].b, px.b));
                         } else {
                             cq = Row4{face_cq(fcy.a, cy.a), face_cq(fcy.b, cy.b)};
                         }
@@ -478,7 +485,7 @@ __device__ __forceinline__ void tiled_item(const StepArgs<float> &a, const int s
                     const Row4 hx = x0r, hy = y0r;
                     h0 = ch;
                     if constexpr (kTheta) oy[s - 1] = cy;
-                    if constexpr (kVec) ox[s - 1] = cx;
+                    if constexpr (kVec) ox[s - 1] = px;
                     x0r = qx;
                     y0r = qs;
                     ch = fin;
