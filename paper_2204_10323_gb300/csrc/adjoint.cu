@@ -921,6 +921,8 @@ __device__ __forceinline__ void adj_rows_item(const AdjArgs<float> &A, const int
 __global__ void __launch_bounds__(32, 12) adj_rows_kernel(const __grid_constant__ AdjArgs<float> A, const int rows, const int rows_edge)
 {
     __shared__ AdjSmem sm;
+    pdl_wait();
+    pdl_launch();
     constexpr int kOut = out_cols(2);
     const int n_strips = (A.fwd.geo.nx + kOut - 1) / kOut, n_edge = min(n_strips, 2);
     const int edge_items = n_edge * ((A.fwd.geo.ny + rows_edge - 1) / rows_edge), item = blockIdx.x;
@@ -1363,8 +1365,7 @@ cudaError_t launch_adjoint_step(const AdjArgs<T> &A, cudaStream_t st)
         int rows = 0, edge = 0;
         tiled_rows(G.nx, G.ny, 2, 0, &rows, &edge);      // an item repeats four rows, as a two-step item does
         const int items = tiled_item_count(G.nx, G.ny, out_cols(2), rows, edge);
-        adj_rows_kernel<<<items, 32, 0, st>>>(A, rows, edge);
-        return cudaGetLastError();                       // pass 3: launch_adjoint_inflow, after the sweep's steps
+        return launch_pdl(adj_rows_kernel, items, 32, st, A, rows, edge);   // pass 3: launch_adjoint_inflow, after the steps
     } else {
         constexpr int BYT = TileRows<T>::v;
         dim3 block(BX, BYT);

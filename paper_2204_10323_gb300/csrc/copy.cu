@@ -12,6 +12,7 @@
 #include <cstdint>
 
 #include "flood_internal.h"
+#include "pdl.cuh"
 
 namespace flood {
 
@@ -24,6 +25,8 @@ template <typename U>
 __global__ void __launch_bounds__(kThreads)
     copy_rows_kernel(U *__restrict__ dst, size_t dpitch, const U *__restrict__ src, size_t spitch, size_t cols, size_t rows)
 {
+    pdl_wait();
+    pdl_launch();
     const size_t tx = blockDim.x;
     for (size_t r = (size_t)blockIdx.x * blockDim.y + threadIdx.y; r < rows; r += (size_t)gridDim.x * blockDim.y) {
         const U *s = src + r * spitch;
@@ -48,9 +51,8 @@ cudaError_t launch(void *dst, size_t dpitch, const void *src, size_t spitch, siz
     while (tx < kThreads && (size_t)tx * kUnroll < cols) tx *= 2;
     const int ty = kThreads / tx;
     const size_t blocks = (rows + ty - 1) / ty;
-    copy_rows_kernel<U><<<(unsigned)std::min<size_t>(blocks, 1u << 20), dim3(tx, ty), 0, st>>>(
-        (U *)dst, dpitch / sizeof(U), (const U *)src, spitch / sizeof(U), cols, rows);
-    return cudaGetLastError();
+    return launch_pdl(copy_rows_kernel<U>, (unsigned)std::min<size_t>(blocks, 1u << 20), dim3(tx, ty), st, (U *)dst,
+                      dpitch / sizeof(U), (const U *)src, spitch / sizeof(U), cols, rows);
 }
 
 // Copy blockIdx.y of the list.

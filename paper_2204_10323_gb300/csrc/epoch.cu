@@ -4,6 +4,7 @@
 #include <cfloat>
 
 #include "device_common.cuh"
+#include "pdl.cuh"
 
 namespace flood {
 
@@ -416,6 +417,8 @@ __global__ void __launch_bounds__(kInflowThreads)
 {
     __shared__ double red[2 * kInflowThreads / 32], st;
     __shared__ T sz[kWarpCells], sn[kWarpCells];
+    pdl_wait();
+    pdl_launch();
     const double t = kBegin ? epoch_time(G, ctrl, fixed_dt, blockIdx.x, &st) : t_list[blockIdx.x];
     inflow_body<T>(G, secs, nsec, cells, tab_t, tab_q, z, n, t, inflow_q, n_slots, inflow_Q, W_out, blockIdx.x,
                    blockIdx.y, red, sz, sn);
@@ -587,15 +590,9 @@ cudaError_t launch_inflow(const EpochArgs<T> &A, int E, bool begin, const double
 {
     if (A.nsec == 0) return begin ? launch_epoch_begin(A.geo, A.ctrl, A.t_list, E, fixed_dt, st) : cudaSuccess;
     const dim3 grid(E, A.nsec);
-    if (begin)
-        inflow_kernel<T, true><<<grid, kInflowThreads, 0, st>>>(A.geo, A.ctrl, fixed_dt, A.secs, A.nsec, A.cells, A.tab_t, A.tab_q,
-                                                                A.z, A.n, A.t_list, E, A.inflow_q, A.n_slots, A.inflow_Q,
-                                                                A.inflow_W);
-    else
-        inflow_kernel<T, false><<<grid, kInflowThreads, 0, st>>>(A.geo, A.ctrl, nullptr, A.secs, A.nsec, A.cells, A.tab_t, A.tab_q,
-                                                                 A.z, A.n, A.t_list, E, A.inflow_q, A.n_slots, A.inflow_Q,
-                                                                 A.inflow_W);
-    return cudaGetLastError();
+    return launch_pdl(begin ? inflow_kernel<T, true> : inflow_kernel<T, false>, grid, kInflowThreads, st, A.geo, A.ctrl,
+                      fixed_dt, A.secs, A.nsec, A.cells, A.tab_t, A.tab_q, A.z, A.n, A.t_list, E, A.inflow_q, A.n_slots,
+                      A.inflow_Q, A.inflow_W);
 }
 
 template <typename T>

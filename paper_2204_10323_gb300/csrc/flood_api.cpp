@@ -341,9 +341,9 @@ flood_status launch_step_planes(flood_handle *h, int s, int k, const void *const
         StepArgs<float> a = make_args<float>(h, s, k, 0, nullptr, 0, nullptr);
         set_planes(a, in, out);
         // The temporal-blocking kernel for several steps, and for one on grids below 2^25 cells: us a step tiled
-        // K = 1 / TMA / stream 11.7 / 13.9 / 15.9 (1024^2), 28.2 / 31.0 / 36.5 (2048^2), 97 / 99 / 103
-        // (4096^2), but 368 / 343 / 349 (8192^2) and 1430 / 1301 / 1298 (16384^2), where one step is bound by
-        // memory and the tiled strips read their halo columns twice.  All bitwise equal.
+        // K = 1 / TMA / stream 9.7 / 13.9 / 15.9 (1024^2), 28 / 31 / 36 (2048^2), 97 / 99 / 103 (4096^2), but
+        // 368 / 343 / 349 (8192^2) and 1430 / 1301 / 1298 (16384^2), where one step is bound by memory and
+        // the tiled strips read their halo columns twice.  All bitwise equal.
         if (k > 1 || (int64_t)h->geo.nx * h->geo.ny < ((int64_t)1 << 25)) {
             a.tile_x = a.tile_y = 0;
             e = launch_step_tiled(a, h->stream);

@@ -15,6 +15,7 @@
 // operations a cell.  A thread per cell computing its four faces itself took 274 us a step
 // at 1001 x 777 (30 % wet; now 130), 36 at 128^2 (now 15).
 #include "device_common.cuh"
+#include "pdl.cuh"
 
 namespace flood {
 
@@ -77,6 +78,8 @@ template <typename T>
 __global__ void __launch_bounds__(32) step_reference_kernel(const __grid_constant__ StepArgs<T> a, const int n_strips, const int rows)
 {
     using O = R<T>;
+    pdl_wait();
+    pdl_launch();
     const Geom &G = a.geo;
     const int nx = G.nx, ny = G.ny, lane = threadIdx.x;
     const int x0 = (int)(blockIdx.x % (unsigned)n_strips) * kCols, c = x0 + lane;
@@ -213,8 +216,7 @@ cudaError_t launch_step_reference(const StepArgs<T> &a, cudaStream_t st)
     const int n_strips = (a.geo.nx + kCols - 1) / kCols;
     const int rows = reference_rows(a.geo.nx, a.geo.ny);
     const int64_t items = (int64_t)n_strips * ((a.geo.ny + rows - 1) / rows);
-    step_reference_kernel<T><<<(unsigned)items, 32, 0, st>>>(a, n_strips, rows);
-    const cudaError_t e = cudaGetLastError();
+    const cudaError_t e = launch_pdl(step_reference_kernel<T>, (unsigned)items, 32, st, a, n_strips, rows);
     if (e != cudaSuccess || !a.gauge_out) return e;
     return launch_gauges<T>(a.geo, a.h_out, a.gauge_cells, a.n_gauges, a.gauge_out, st);
 }

@@ -34,6 +34,7 @@
 #include <type_traits>
 
 #include "fast_face.cuh"
+#include "pdl.cuh"
 
 namespace flood {
 
@@ -638,6 +639,8 @@ template <int K, int kMode, bool kGauge>
 __global__ void __launch_bounds__(32, tiled_warps(kMode)) step_tiled_kernel(const __grid_constant__ StepArgs<float> a)
 {
     __shared__ TiledSmem<kMode> sm;
+    pdl_wait();
+    pdl_launch();
     const int n_items = tiled_item_count(a.geo.nx, a.geo.ny, out_cols(K, kMode), a.tile_y, a.tile_x);
 #pragma unroll 1
     for (int item = blockIdx.x; item < n_items; item += gridDim.x) tiled_run<K, kMode, kGauge>(a, a.s, item, a.want_hmax, sm);
@@ -686,9 +689,8 @@ cudaError_t launch_k(const StepArgs<float> &a0, cudaStream_t st)
     blocks = a0.tile_x > 0 && a0.tile_x < items ? a0.tile_x : items;    // caller's cap on pipelines
     a.tile_x = edge;
     a.tile_y = rows;
-    if (a.gauge_out && a.n_gauges > 0) step_tiled_kernel<K, kMode, true><<<blocks, 32, 0, st>>>(a);
-    else step_tiled_kernel<K, kMode, false><<<blocks, 32, 0, st>>>(a);
-    return cudaGetLastError();
+    return launch_pdl(a.gauge_out && a.n_gauges > 0 ? step_tiled_kernel<K, kMode, true> : step_tiled_kernel<K, kMode, false>,
+                      blocks, 32, st, a);
 }
 
 // Launchers of one scheme mode for every steps-per-launch K.
