@@ -466,8 +466,8 @@ __global__ void adj_inflow_kernel(const AdjArgs<T> A)
 }
 
 // ---------------------------------------------------------------- FP32, Eq. 3 as printed
-// The FP32 reverse step: one warp walks the rows of a strip of 120 output columns (128 staged,
-// four per lane) south to north, as the temporal-blocking kernel does, in one pass.  At tick j:
+// The FP32 reverse step: one warp walks the rows of a strip of 60 output columns (64 staged, a
+// pair per lane) south to north, as the temporal-blocking kernel does, in one pass.  At tick j:
 //  A. row j's new faces (the forward arithmetic) and, from the same intermediates, each face's
 //     derivatives with respect to its old discharge, its two depths and n; kept one tick;
 //  B. the adjoint lu of row j-1's unclipped depth: its update needs the south faces of row j;
@@ -479,21 +479,47 @@ __global__ void adj_inflow_kernel(const AdjArgs<T> A)
 // asynchronous copies, every lane's shared memory is its own: no barrier, no index arithmetic per
 // element.
 //
-// At 1024^2 (20.2 us, 11 warps per SM) a lone warp's chain bounds it: a tick of 550 instructions takes
-// some 2300 cycles by itself, 3000 beside two others, and an item of six rows runs nine.  Eight warps per
-// SM without spills: 22.2 us; the derivatives kept in shared memory: 20.7.  A tile kernel (32 x 8 cells staged
-// by tensor copies, flat loops over the staged arrays between block barriers) executed 647 thread
-// instructions per cell, 285 of them integer, and took 28.8 us.
+// A lone warp's chain bounds it (powers, reciprocals, shuffles, FP64 adds in series: six cycles an
+// instruction), so a strip takes two columns per lane where the forward kernel takes four: half the instructions
+// a tick and twice the warps.  A sweep of 64 steps with its states kept, two / four columns: 2.07 / 2.23 ms
+// (1024^2), 1.27 / 1.59 (512^2), 1.08 / 1.56 (256^2), 5.74 / 6.08 (2048^2).  A step of 1024^2 takes 20 us; a tile
+// kernel (32 x 8 cells staged by tensor copies, flat loops over the staged arrays between block barriers)
+// executed 647 thread instructions per cell, 285 of them integer, and took 28.8.
+constexpr int kAdjOut = 60;              // output columns of a strip
 
 struct alignas(16) AdjSmem {
-    float raw[kAhead][8][128];           // rows in flight: h, z, n, qx, qy of row j; lambda_h, lambda_qx, lambda_qy of row j - 1
-    double gn[kAhead][128];              // dL/dn of row j - 2
+    float raw[kAhead][8][64];            // rows in flight: h, z, n, qx, qy of row j; lambda_h, lambda_qx, lambda_qy of row j - 1
+    double gn[kAhead][64];               // dL/dn of row j - 2
     int gauge[32][3];                    // gauges in the staged cells, in gauge order: row, column, index
 };
 
+// Two columns of a row.
+using Pair = unsigned long long;
+
+__device__ __forceinline__ Pair pair_load(const float *p) { return *reinterpret_cast<const Pair *>(p); }
+__device__ __forceinline__ void pair_store(float *p, Pair v) { *reinterpret_cast<Pair *>(p) = v; }
+__device__ __forceinline__ float pair_get(Pair v, int k) { return k ? f2unpack(v).y : f2unpack(v).x; }
+__device__ __forceinline__ void pair_set(Pair &v, int k, float x)
+{
+    const float2 p = f2unpack(v);
+    v = f2pack(k ? p.x : x, k ? x : p.y);
+}
+// The lane to the left's second column, the lane to the right's first; the pair one column to the left or right.
+__device__ __forceinline__ float pair_from_left(Pair v) { return __shfl_up_sync(0xffffffffu, f2unpack(v).y, 1); }
+__device__ __forceinline__ float pair_from_right(Pair v) { return __shfl_down_sync(0xffffffffu, f2unpack(v).x, 1); }
+__device__ __forceinline__ Pair pair_right(Pair v) { return f2pack(f2unpack(v).y, pair_from_right(v)); }
+
+// 8 bytes global -> shared, asynchronously (in the thread's current group); in == false: zeros.
+__device__ __forceinline__ void copy8(float *dst, const float *src, bool in)
+{
+    asm volatile("cp.async.ca.shared.global [%0], [%1], 8, %2;" ::"r"((unsigned)__cvta_generic_to_shared(dst)), "l"(src),
+                 "r"(in ? 8 : 0)
+                 : "memory");
+}
+
 // The derivatives of a row's faces.
 struct FaceRow {
-    Row4 q, L, R, n;                     // with respect to the old discharge, the depths of the two cells, n of either
+    Pair q, L, R, n;                     // with respect to the old discharge, the depths of the two cells, n of either
 };
 
 __device__ __forceinline__ unsigned long long f2sel(bool x, bool y, unsigned long long a, unsigned long long b)
@@ -575,18 +601,9 @@ __device__ __forceinline__ float border_lin(int type, float inward, float h, flo
     return -inward * q;
 }
 
-__device__ __forceinline__ void row_set(Row4 &v, int k, float x)
-{
-    const float2 a = f2unpack(v.a), b = f2unpack(v.b);
-    v = row_pack(k == 0 ? x : a.x, k == 1 ? x : a.y, k == 2 ? x : b.x, k == 3 ? x : b.y);
-}
-
-__device__ __forceinline__ Row4 row_add(const Row4 &x, const Row4 &y) { return Row4{f2add(x.a, y.a), f2add(x.b, y.b)}; }
-__device__ __forceinline__ Row4 row_mul(const Row4 &x, const Row4 &y) { return Row4{f2mul(x.a, y.a), f2mul(x.b, y.b)}; }
-
 __device__ __forceinline__ void adj_rows_item(const AdjArgs<float> &A, const int strip, const int y0, const int y1, AdjSmem &sm)
 {
-    constexpr int kOut = out_cols(2);
+    constexpr int kOut = kAdjOut;
     const StepArgs<float> &a = A.fwd;
     const Geom &G = a.geo;
     const int lane = threadIdx.x;
@@ -594,20 +611,20 @@ __device__ __forceinline__ void adj_rows_item(const AdjArgs<float> &A, const int
     const size_t P = (size_t)G.pitch;
     const Fwd<float> FW(G, a.ctrl->dt);
     const FastConst Kc = FW.K;
-    const int x0 = strip * kOut - 4;
-    const int c0 = x0 + 4 * lane;
+    const int x0 = strip * kOut - 2;
+    const int c0 = x0 + 2 * lane;
     const int own_lo = strip * kOut, own_hi = min(own_lo + kOut, nx);
-    const bool west = x0 < 0, east = x0 + 127 >= nx;
+    const bool west = x0 < 0, east = x0 + 63 >= nx;
     const bool in = c0 >= 0 && c0 < (int)P;
     const int jb = max(y0 - 2, 0);
     const int jhi = min(y1 + 1, ny - 1);               // last row of the state
     const int jlast = y1 + 1;                          // last tick: row y1 - 1 is completed
-    const int steady_lo = jb > 0 ? jb : 2, steady_hi = nx >= 4 ? jhi : -1;
-    const bool full = c0 >= own_lo && c0 + 3 < own_hi;
+    const int steady_lo = jb > 0 ? jb : 2, steady_hi = nx >= 2 ? jhi : -1;
+    const bool full = c0 >= own_lo && c0 + 1 < own_hi;
     const bool part = !full && c0 >= own_lo && (c0 < own_hi || (c0 == nx && own_hi == nx));
-    // the border face at x = 0 or x = nx in this lane's columns (with nx < 4 a lane can hold both, and every
+    // the border face at x = 0 or x = nx in this lane's columns (with nx < 2 a lane can hold both, and every
     // tick takes the general form); its type, inflow slot and sqrt(S) are read a tick ahead
-    const bool lane_w = west && c0 == 0, lane_e = east && nx - c0 >= 0 && nx - c0 < 4;
+    const bool lane_w = west && c0 == 0, lane_e = east && nx - c0 >= 0 && nx - c0 < 2;
     const int side = lane_e ? 1 : 0, kb = lane_e ? nx - c0 : lane_w ? 0 : -1;
     int nb_t = kBcWall, nb_s = 0, pb_t = kBcWall, pb_s = 0;
     float nb_q = 0.0f;
@@ -622,27 +639,26 @@ __device__ __forceinline__ void adj_rows_item(const AdjArgs<float> &A, const int
     const size_t lane_off = in ? (size_t)c0 : 0;
 
     auto issue = [&](int j) {
-        float *d = &sm.raw[j & (kAhead - 1)][0][4 * lane];
+        float *d = &sm.raw[j & (kAhead - 1)][0][2 * lane];
         if (j <= jhi) {
             const size_t o = (size_t)j * P + lane_off;
-            copy16(d, a.h + o, in);
-            copy16(d + 128, a.z + o, in);
-            copy16(d + 256, a.n + o, in);
-            copy16(d + 384, a.qx + o, in);
-            copy16(d + 512, a.qy + o, in);
+            copy8(d, a.h + o, in);
+            copy8(d + 64, a.z + o, in);
+            copy8(d + 128, a.n + o, in);
+            copy8(d + 192, a.qx + o, in);
+            copy8(d + 256, a.qy + o, in);
         }
         if (j >= 1 && j <= jlast) {                    // face row ny has lambda_qy only
             const size_t o = (size_t)(j - 1) * P + lane_off;
             if (j - 1 < ny) {
-                copy16(d + 640, A.lh + o, in);
-                copy16(d + 768, A.lqx + o, in);
+                copy8(d + 320, A.lh + o, in);
+                copy8(d + 384, A.lqx + o, in);
             }
-            copy16(d + 896, A.lqy + o, in);
+            copy8(d + 448, A.lqy + o, in);
         }
         if (j - 2 >= y0 && j - 2 < y1) {
             const double *g = A.gn + (size_t)(j - 2) * P + lane_off;
-            copy16(reinterpret_cast<float *>(&sm.gn[j & (kAhead - 1)][4 * lane]), reinterpret_cast<const float *>(g), in);
-            copy16(reinterpret_cast<float *>(&sm.gn[j & (kAhead - 1)][4 * lane + 2]), reinterpret_cast<const float *>(g + 2), in);
+            copy16(reinterpret_cast<float *>(&sm.gn[j & (kAhead - 1)][2 * lane]), reinterpret_cast<const float *>(g), in);
         }
         copy_commit();
     };
@@ -658,7 +674,7 @@ __device__ __forceinline__ void adj_rows_item(const AdjArgs<float> &A, const int
             gj = rc.x;
             gi = rc.y;
         }
-        const bool mine = gj >= jb && gj <= jhi && gi >= x0 && gi < x0 + 128;
+        const bool mine = gj >= jb && gj <= jhi && gi >= x0 && gi < x0 + 64;
         const unsigned m = __ballot_sync(0xffffffffu, mine);
         const int slot = ng + __popc(m & ((1u << lane) - 1));
         if (mine && slot < 32) {
@@ -670,69 +686,64 @@ __device__ __forceinline__ void adj_rows_item(const AdjArgs<float> &A, const int
     }
     __syncwarp();
 
-    Row4 hp{0, 0}, zp{0, 0}, np_{0, 0};                // row j - 1: depth, bed, n
-    Row4 xp{0, 0}, yp{0, 0};                           // its new faces
+    Pair hp = 0, zp = 0, np_ = 0;                // row j - 1: depth, bed, n
+    Pair xp = 0, yp = 0;                           // its new faces
     FaceRow dx{}, dy{};                                // and their derivatives
-    Row4 lu2{0, 0}, acc2{0, 0}, gx2{0, 0}, gy2{0, 0};  // row j - 2: lu, and its sums so far
+    Pair lu2 = 0, acc2 = 0, gx2 = 0, gy2 = 0;  // row j - 2: lu, and its sums so far
 
     auto tick = [&](auto steady_t, auto edge_t, const int j) {
         constexpr bool kSteady = decltype(steady_t)::value, kEdge = decltype(edge_t)::value;
         const bool row = kSteady || j < ny, rowp = kSteady || (j >= 1 && j <= ny);   // rows j and j - 1 are cells
         copy_wait<kAhead - 1>();
-        const float *d = &sm.raw[j & (kAhead - 1)][0][4 * lane];
-        const Row4 lq = row_load(d + 768), lqy = row_load(d + 896);
-        Row4 lu = row_load(d + 640);
-        double2 g01 = *reinterpret_cast<const double2 *>(&sm.gn[j & (kAhead - 1)][4 * lane]);
-        double2 g23 = *reinterpret_cast<const double2 *>(&sm.gn[j & (kAhead - 1)][4 * lane + 2]);
-        Row4 ch{0, 0}, cz{0, 0}, cn{0, 0}, cx{0, 0}, cy{0, 0};
+        const float *d = &sm.raw[j & (kAhead - 1)][0][2 * lane];
+        const Pair lq = pair_load(d + 384), lqy = pair_load(d + 448);
+        Pair lu = pair_load(d + 320);
+        double2 gn = *reinterpret_cast<const double2 *>(&sm.gn[j & (kAhead - 1)][2 * lane]);
+        Pair ch = 0, cz = 0, cn = 0, cx = 0, cy = 0;
         if (row) {
-            ch = row_load(d);
-            cz = row_load(d + 128);
-            cn = row_load(d + 256);
-            cx = row_load(d + 384);
-            cy = row_load(d + 512);
+            ch = pair_load(d);
+            cz = pair_load(d + 64);
+            cn = pair_load(d + 128);
+            cx = pair_load(d + 192);
+            cy = pair_load(d + 256);
         }
         issue(j + kAhead);
         // ---- A. the new south faces of row j (their derivatives, and the west faces, after C has used
         // those of row j - 1: they take the same registers)
-        const Row4 e = row_add(ch, cz);
+        const Pair e = f2add(ch, cz);
         const bool inner = kSteady || (j > 0 && j < ny);
-        Row4 qy{0, 0}, bR{0, 0}, bL{0, 0}, bn{0, 0};
-        Faces2 ya, yb;
+        Pair qy = 0, bR = 0, bL = 0, bn = 0;
+        Faces2 ya;
         if (inner) {
-            const Row4 ep = row_add(hp, zp);
-            ya = faces2_value(f2sub(f2max(ep.a, e.a), f2max(zp.a, cz.a)), f2sub(e.a, ep.a), cy.a, f2add(np_.a, cn.a), Kc);
-            yb = faces2_value(f2sub(f2max(ep.b, e.b), f2max(zp.b, cz.b)), f2sub(e.b, ep.b), cy.b, f2add(np_.b, cn.b), Kc);
-            qy = Row4{ya.F, yb.F};
+            const Pair ep = f2add(hp, zp);
+            ya = faces2_value(f2sub(f2max(ep, e), f2max(zp, cz)), f2sub(e, ep), cy, f2add(np_, cn), Kc);
+            qy = ya.F;
         } else if (j == 0 || j == ny) {
             const int off = j == 0 ? 2 * ny : 2 * ny + nx;
-            const Row4 hb = j == 0 ? ch : hp, nb = j == 0 ? cn : np_;
+            const Pair hb = j == 0 ? ch : hp, nb = j == 0 ? cn : np_;
 #pragma unroll 1
-            for (int k = 0; k < 4; k++) {
+            for (int k = 0; k < 2; k++) {
                 const int c = c0 + k;
                 if (c < 0 || c >= nx) continue;
                 const int t = a.bc.type[off + c];
                 float dh, dn;
-                const float v = border_lin(t, j == 0 ? 1.0f : -1.0f, row_get(hb, k), a.bc.sqrtS_f[off + c], row_get(nb, k), G,
+                const float v = border_lin(t, j == 0 ? 1.0f : -1.0f, pair_get(hb, k), a.bc.sqrtS_f[off + c], pair_get(nb, k), G,
                                            t == kBcInflow ? a.inflow_q[(size_t)a.s * a.n_slots + a.bc.slot[off + c]] : 0.0f,
                                            dh, dn);
-                row_set(qy, k, v);
-                if (j == 0) row_set(bR, k, dh);
-                else row_set(bL, k, dh);
-                row_set(bn, k, dn);
+                pair_set(qy, k, v);
+                if (j == 0) pair_set(bR, k, dh);
+                else pair_set(bL, k, dh);
+                pair_set(bn, k, dn);
             }
         }
-        // ---- B. the adjoint of row j - 1's unclipped depth (tick y0 - 1 only readies row y0 - 1's faces)
-        const bool sums = !kSteady || j >= y0;
-        if (sums) {
+        // ---- B. the adjoint of row j - 1's unclipped depth
         if (rowp) {
-            const float2 x01 = f2unpack(xp.a), x23 = f2unpack(xp.b);
-            const float xe = from_right(xp);
-            const unsigned long long d0 = f2add(f2pack(__fsub_rn(x01.x, x01.y), __fsub_rn(x01.y, x23.x)), f2sub(yp.a, qy.a));
-            const unsigned long long d1 = f2add(f2pack(__fsub_rn(x23.x, x23.y), __fsub_rn(x23.y, xe)), f2sub(yp.b, qy.b));
-            const float2 u0 = f2unpack(f2fma(f2dup(Kc.dtdx), d0, hp.a)), u1 = f2unpack(f2fma(f2dup(Kc.dtdx), d1, hp.b));
-            const float u[4] = {u0.x, u0.y, u1.x, u1.y};
-            float v[4] = {row_get(lu, 0), row_get(lu, 1), row_get(lu, 2), row_get(lu, 3)};
+            const float2 x01 = f2unpack(xp);
+            const float xe = pair_from_right(xp);
+            const Pair dv = f2add(f2pack(__fsub_rn(x01.x, x01.y), __fsub_rn(x01.y, xe)), f2sub(yp, qy));
+            const float2 u0 = f2unpack(f2fma(f2dup(Kc.dtdx), dv, hp));
+            const float u[2] = {u0.x, u0.y};
+            float v[2] = {f2unpack(lu).x, f2unpack(lu).y};
             if (ng > 0) {
                 const int n_scan = ng <= 32 ? ng : A.n_gauges;
                 for (int x = 0; x < n_scan; x++) {
@@ -748,130 +759,61 @@ __device__ __forceinline__ void adj_rows_item(const AdjArgs<float> &A, const int
                     if (gj != j - 1) continue;
                     const float sd = (float)A.seed[gk];
 #pragma unroll
-                    for (int k = 0; k < 4; k++)
-                        if (gc == 4 * lane + k) v[k] = v[k] + sd;
+                    for (int k = 0; k < 2; k++)
+                        if (gc == 2 * lane + k) v[k] = v[k] + sd;
                 }
             }
 #pragma unroll
-            for (int k = 0; k < 4; k++) {
+            for (int k = 0; k < 2; k++) {
                 if (u[k] < 0.0f) v[k] = 0.0f;
                 if (kEdge && (c0 + k < 0 || c0 + k >= nx)) v[k] = 0.0f;
             }
-            lu = row_pack(v[0], v[1], v[2], v[3]);
+            lu = f2pack(v[0], v[1]);
         } else {
-            lu = Row4{0, 0};
+            lu = 0;
         }
         // ---- C. the x-faces of row j - 1 and the y-faces below it
-        const float lul = from_left(lu);
-        const float2 a0 = f2unpack(lu.a), a1 = f2unpack(lu.b);
-        const unsigned long long dl0 = f2pack(__fsub_rn(a0.x, lul), __fsub_rn(a0.y, a0.x));
-        const unsigned long long dl1 = f2pack(__fsub_rn(a1.x, a0.y), __fsub_rn(a1.y, a1.x));
-        const Row4 mux{f2fma(f2dup(Kc.dtdx), dl0, lq.a), f2fma(f2dup(Kc.dtdx), dl1, lq.b)};
-        const Row4 muy{f2fma(f2dup(Kc.dtdx), f2sub(lu.a, lu2.a), lqy.a), f2fma(f2dup(Kc.dtdx), f2sub(lu.b, lu2.b), lqy.b)};
-        const Row4 xL = row_mul(mux, dx.L), xR = row_mul(mux, dx.R), xn = row_mul(mux, dx.n), xq = row_mul(mux, dx.q);
-        const Row4 yL = row_mul(muy, dy.L), yR = row_mul(muy, dy.R), yn = row_mul(muy, dy.n), yq = row_mul(muy, dy.q);
-        // ---- D. row j - 2 is complete
-        if (j - 2 >= y0 && j - 2 < y1) {
-            const Row4 out = row_add(acc2, yL), gs = row_add(gx2, row_add(gy2, yn));
-            const float2 s0 = f2unpack(gs.a), s1 = f2unpack(gs.b);
-            const size_t o = (size_t)(j - 2) * P + lane_off;
-            g01.x += (double)s0.x;
-            g01.y += (double)s0.y;
-            g23.x += (double)s1.x;
-            g23.y += (double)s1.y;
-            if (kEdge ? full : lane >= 1 && lane <= kOut / 4) {
-                row_store(A.lh_out + o, out);
-                *reinterpret_cast<double2 *>(A.gn + o) = g01;
-                *reinterpret_cast<double2 *>(A.gn + o + 2) = g23;
-            } else if (kEdge && part) {
-                const double g[4] = {g01.x, g01.y, g23.x, g23.y};
-#pragma unroll
-                for (int k = 0; k < 4; k++)
-                    if (c0 + k < own_hi) {
-                        A.lh_out[o + k] = row_get(out, k);
-                        A.gn[o + k] = g[k];
-                    }
-            }
-        }
-        // the adjoint of the old faces of row j - 1 (and of the grid's north faces, face row ny)
-        const int r = j - 1;
-        if (r >= y0 && (r < y1 || (r == ny && y1 == ny))) {
-            const size_t o = (size_t)r * P + lane_off;
-            const bool cells = r < ny;
-            if (kEdge ? full : lane >= 1 && lane <= kOut / 4) {
-                if (cells) row_store(A.lqx_out + o, xq);
-                row_store(A.lqy_out + o, yq);
-            } else if (kEdge && part) {
-#pragma unroll
-                for (int k = 0; k < 4; k++) {
-                    const int c = c0 + k;
-                    if (cells && (c < own_hi || c == nx)) A.lqx_out[o + k] = row_get(xq, k);
-                    if (c < own_hi) A.lqy_out[o + k] = row_get(yq, k);
-                }
-            }
-            // inflow faces: lu of the cell and lambda_q of the face, for pass 3
-            if (A.in_log) {
-                if (kEdge && cells && (west || east)) {
-                    const int kf = side ? nx - c0 : 0;
-                    if (kb >= 0 && pb_t == kBcInflow && (side ? own_hi == nx : own_lo == 0))
-                        A.in_log[pb_s] = make_float2(side ? (kf == 0 ? lul : row_get(lu, kf - 1)) : a0.x, row_get(lq, kf));
-                    if (!kSteady && lane_w && lane_e && a.bc.type[r] == kBcInflow)     // nx < 4: the west face too
-                        A.in_log[a.bc.slot[r]] = make_float2(a0.x, row_get(lq, 0));
-                }
-                if (!kSteady && (r == 0 || r == ny)) {
-                    const int off = r == 0 ? 2 * ny : 2 * ny + nx;
-                    const Row4 lb = r == 0 ? lu : lu2;
-#pragma unroll
-                    for (int k = 0; k < 4; k++) {
-                        const int c = c0 + k;
-                        if (c >= own_lo && c < own_hi && a.bc.type[off + c] == kBcInflow)
-                            A.in_log[a.bc.slot[off + c]] = make_float2(row_get(lb, k), row_get(lqy, k));
-                    }
-                }
-            }
-        }
+        const float lul = pair_from_left(lu);
+        const float2 a0 = f2unpack(lu);
+        const Pair mux = f2fma(f2dup(Kc.dtdx), f2pack(__fsub_rn(a0.x, lul), __fsub_rn(a0.y, a0.x)), lq);
+        const Pair muy = f2fma(f2dup(Kc.dtdx), f2sub(lu, lu2), lqy);
+        const Pair xL = f2mul(mux, dx.L), xR = f2mul(mux, dx.R), xn = f2mul(mux, dx.n), xq = f2mul(mux, dx.q);
+        const Pair yL = f2mul(muy, dy.L), yR = f2mul(muy, dy.R), yn = f2mul(muy, dy.n), yq = f2mul(muy, dy.q);
+        const Pair out2 = f2add(acc2, yL), gs2 = f2add(gx2, f2add(gy2, yn));   // row j - 2's sums, complete
+        const Pair lu_below = lu2;
         // ---- the rows move on
-        acc2 = row_add(row_add(row_add(lu, xR), row_right(xL, from_right(xL))), yR);
-        gx2 = row_add(xn, row_right(xn, from_right(xn)));
+        acc2 = f2add(f2add(f2add(lu, xR), pair_right(xL)), yR);
+        gx2 = f2add(xn, pair_right(xn));
         gy2 = yn;
         lu2 = lu;
-        }
-        if (j == jlast) return;                        // row y1 + 1 only gave its south faces
         yp = qy;
-        if (inner) {
-            faces2_lin(ya, Kc, dy.q.a, dy.L.a, dy.R.a, dy.n.a);
-            faces2_lin(yb, Kc, dy.q.b, dy.L.b, dy.R.b, dy.n.b);
-        } else {
-            dy = FaceRow{Row4{0, 0}, bL, bR, bn};
-        }
+        const int qb_t = pb_t, qb_s = pb_s;
+
+        if (inner) faces2_lin(ya, Kc, dy.q, dy.L, dy.R, dy.n);
+        else dy = FaceRow{0, bL, bR, bn};
         if (row) {
-            const Row4 el = row_left(e, from_left(e)), zl = row_left(cz, from_left(cz));
-            const float nl = from_left(cn);
-            const float2 e0 = f2unpack(e.a), e1 = f2unpack(e.b), l0 = f2unpack(el.a), n0 = f2unpack(cn.a), n1 = f2unpack(cn.b);
-            const Faces2 xa = faces2_value(f2sub(f2max(el.a, e.a), f2max(zl.a, cz.a)),
-                                           f2pack(__fsub_rn(e0.x, l0.x), __fsub_rn(e0.y, e0.x)), cx.a,
+            const float el = pair_from_left(e), zl = pair_from_left(cz), nl = pair_from_left(cn);
+            const float2 e0 = f2unpack(e), z0 = f2unpack(cz), n0 = f2unpack(cn);
+            const Faces2 xa = faces2_value(f2sub(f2max(f2pack(el, e0.x), e), f2max(f2pack(zl, z0.x), cz)),
+                                           f2pack(__fsub_rn(e0.x, el), __fsub_rn(e0.y, e0.x)), cx,
                                            f2pack(__fadd_rn(nl, n0.x), __fadd_rn(n0.x, n0.y)), Kc);
-            const Faces2 xb = faces2_value(f2sub(f2max(el.b, e.b), f2max(zl.b, cz.b)),
-                                           f2pack(__fsub_rn(e1.x, e0.y), __fsub_rn(e1.y, e1.x)), cx.b,
-                                           f2pack(__fadd_rn(n0.y, n1.x), __fadd_rn(n1.x, n1.y)), Kc);
-            xp = Row4{xa.F, xb.F};
-            faces2_lin(xa, Kc, dx.q.a, dx.L.a, dx.R.a, dx.n.a);
-            faces2_lin(xb, Kc, dx.q.b, dx.L.b, dx.R.b, dx.n.b);
+            xp = xa.F;
+            faces2_lin(xa, Kc, dx.q, dx.L, dx.R, dx.n);
             if (kEdge && (west || east)) {
-                const float hl = from_left(ch);
+                const float hl = pair_from_left(ch);
                 // the border face of side sd in this lane's column kf
                 auto border = [&](int sd, int t, int slot, float sqrtS) {
                     const int kf = sd ? nx - c0 : 0;
-                    const float h = sd ? (kf == 0 ? hl : row_get(ch, kf - 1)) : row_get(ch, 0);
-                    const float n = sd ? (kf == 0 ? nl : row_get(cn, kf - 1)) : n0.x;
+                    const float h = sd && kf == 0 ? hl : f2unpack(ch).x;   // (kf = 1: the cell is the first column)
+                    const float n = sd && kf == 0 ? nl : n0.x;
                     float dh, dn;
                     const float v = border_lin(t, sd ? -1.0f : 1.0f, h, sqrtS, n, G,
                                                t == kBcInflow ? a.inflow_q[(size_t)a.s * a.n_slots + slot] : 0.0f, dh, dn);
-                    row_set(xp, kf, v);
-                    row_set(dx.q, kf, 0.0f);
-                    row_set(dx.L, kf, sd ? dh : 0.0f);
-                    row_set(dx.R, kf, sd ? 0.0f : dh);
-                    row_set(dx.n, kf, dn);
+                    pair_set(xp, kf, v);
+                    pair_set(dx.q, kf, 0.0f);
+                    pair_set(dx.L, kf, sd ? dh : 0.0f);
+                    pair_set(dx.R, kf, sd ? 0.0f : dh);
+                    pair_set(dx.n, kf, dn);
                 };
                 if (kb >= 0) border(side, nb_t, nb_s, nb_q);
                 if (!kSteady && lane_w && lane_e) border(0, a.bc.type[j], a.bc.slot[j], a.bc.sqrtS_f[j]);
@@ -880,22 +822,73 @@ __device__ __forceinline__ void adj_rows_item(const AdjArgs<float> &A, const int
                 border_fetch(j + 1);
             }
         } else {
-            xp = Row4{0, 0};
+            xp = 0;
             dx = FaceRow{};
             pb_t = kBcWall;
         }
         hp = ch;
         zp = cz;
         np_ = cn;
+        // ---- D. row j - 2 is complete
+        if (j - 2 >= y0 && j - 2 < y1) {
+            const float2 gs = f2unpack(gs2);
+            const size_t o = (size_t)(j - 2) * P + lane_off;
+            gn.x += (double)gs.x;
+            gn.y += (double)gs.y;
+            if (kEdge ? full : lane >= 1 && lane <= kOut / 2) {
+                pair_store(A.lh_out + o, out2);
+                *reinterpret_cast<double2 *>(A.gn + o) = gn;
+            } else if (kEdge && part && c0 < own_hi) {
+                A.lh_out[o] = f2unpack(out2).x;
+                A.gn[o] = gn.x;
+            }
+        }
+        // the adjoint of the old faces of row j - 1 (and of the grid's north faces, face row ny)
+        const int r = j - 1;
+        if (r >= y0 && (r < y1 || (r == ny && y1 == ny))) {
+            const size_t o = (size_t)r * P + lane_off;
+            const bool cells = r < ny;
+            if (kEdge ? full : lane >= 1 && lane <= kOut / 2) {
+                if (cells) pair_store(A.lqx_out + o, xq);
+                pair_store(A.lqy_out + o, yq);
+            } else if (kEdge && part) {
+#pragma unroll
+                for (int k = 0; k < 2; k++) {
+                    const int c = c0 + k;
+                    if (cells && (c < own_hi || c == nx)) A.lqx_out[o + k] = pair_get(xq, k);
+                    if (c < own_hi) A.lqy_out[o + k] = pair_get(yq, k);
+                }
+            }
+            // inflow faces: lu of the cell and lambda_q of the face, for pass 3
+            if (A.in_log) {
+                if (kEdge && cells && (west || east)) {
+                    const int kf = side ? nx - c0 : 0;
+                    if (kb >= 0 && qb_t == kBcInflow && (side ? own_hi == nx : own_lo == 0))
+                        A.in_log[qb_s] = make_float2(side ? (kf == 0 ? lul : a0.x) : a0.x, pair_get(lq, kf));
+                    if (!kSteady && lane_w && lane_e && a.bc.type[r] == kBcInflow)     // nx = 1: the west face too
+                        A.in_log[a.bc.slot[r]] = make_float2(a0.x, pair_get(lq, 0));
+                }
+                if (!kSteady && (r == 0 || r == ny)) {
+                    const int off = r == 0 ? 2 * ny : 2 * ny + nx;
+                    const Pair lb = r == 0 ? lu : lu_below;
+#pragma unroll
+                    for (int k = 0; k < 2; k++) {
+                        const int c = c0 + k;
+                        if (c >= own_lo && c < own_hi && a.bc.type[off + c] == kBcInflow)
+                            A.in_log[a.bc.slot[off + c]] = make_float2(pair_get(lb, k), pair_get(lqy, k));
+                    }
+                }
+            }
+        }
     };
 
     int j = jb;
     if (jb > 0) {                                      // row y0 - 2 is only the row below
         copy_wait<kAhead - 1>();
-        const float *d = &sm.raw[jb & (kAhead - 1)][0][4 * lane];
-        hp = row_load(d);
-        zp = row_load(d + 128);
-        np_ = row_load(d + 256);
+        const float *d = &sm.raw[jb & (kAhead - 1)][0][2 * lane];
+        hp = pair_load(d);
+        zp = pair_load(d + 64);
+        np_ = pair_load(d + 128);
         border_fetch(jb + 1);
         issue(jb + kAhead);
         j++;
@@ -923,7 +916,7 @@ __global__ void __launch_bounds__(32, 12) adj_rows_kernel(const __grid_constant_
     __shared__ AdjSmem sm;
     pdl_wait();
     pdl_launch();
-    constexpr int kOut = out_cols(2);
+    constexpr int kOut = kAdjOut;
     const int n_strips = (A.fwd.geo.nx + kOut - 1) / kOut, n_edge = min(n_strips, 2);
     const int edge_items = n_edge * ((A.fwd.geo.ny + rows_edge - 1) / rows_edge), item = blockIdx.x;
     int strip, y0, r;
@@ -1363,8 +1356,9 @@ cudaError_t launch_adjoint_step(const AdjArgs<T> &A, cudaStream_t st)
         adj_opt_gather_kernel<T><<<(unsigned)((int64_t)nbx * nby), block, 0, st>>>(A, nbx);
     } else if constexpr (std::is_same<T, float>::value) {
         int rows = 0, edge = 0;
-        tiled_rows(G.nx, G.ny, 2, 0, &rows, &edge);      // an item repeats four rows, as a two-step item does
-        const int items = tiled_item_count(G.nx, G.ny, out_cols(2), rows, edge);
+        // (an item runs three ticks more than it has rows)
+        tiled_rows_for((G.nx + kAdjOut - 1) / kAdjOut, G.ny, 3, 12, 900.0, 350.0, 500.0, &rows, &edge);
+        const int items = tiled_item_count(G.nx, G.ny, kAdjOut, rows, edge);
         return launch_pdl(adj_rows_kernel, items, 32, st, A, rows, edge);   // pass 3: launch_adjoint_inflow, after the steps
     } else {
         constexpr int BYT = TileRows<T>::v;

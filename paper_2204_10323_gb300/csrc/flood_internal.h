@@ -108,6 +108,8 @@ int tiled_items(const Geom &g, int rows, int rows_edge, int k_steps);
 // Rows per work item (inner strips, and the one or two strips with the borders x = 0 and x = nx) for a grid
 // alone on the GPU.
 void tiled_rows(int nx, int ny, int K, int mode, int *rows, int *rows_edge);
+void tiled_rows_for(int n_strips, int ny, int repeat, int warps, double base, double slope, double edge_more, int *rows,
+                    int *rows_edge);
 cudaError_t launch_step_tiled_ensemble(const StepArgs<float> *table, const int *base, int n, int total_items,
                                        int k_steps, int s0, int want_hmax, int mode, cudaStream_t st);
 void stream_launch_shape(const Geom &g, int tile_x, int tile_y, int *warps, int *rows);

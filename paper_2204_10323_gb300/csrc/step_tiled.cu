@@ -13,19 +13,28 @@ namespace flood {
 // (2048^2), 39 / 50 (4096^2), 131 / 131 (8192^2), 465 / 477 (16384^2).
 void tiled_rows(int nx, int ny, int K, int mode, int *rows, int *rows_edge)
 {
-    static constexpr int kTry[] = {4,  6,  8,  10, 12, 14, 16,  18,  20,  22,  24,  28,  32, 36,
+    const int out = out_cols(K, mode);
+    tiled_rows_for((nx + out - 1) / out, ny, 2 * K, tiled_warps(mode), 1150.0, 490.0, 1000.0, rows, rows_edge);
+}
+
+// The rule for items of r + `repeat` ticks, `warps` of them per SM, a tick taking base + slope * (warps on a
+// quarter of an SM), and `edge` more in an edge strip.
+void tiled_rows_for(int n_strips, int ny, int repeat, int warps, double base, double slope, double edge_more, int *rows,
+                    int *rows_edge)
+{
+    static constexpr int kTry[] = {2,  3,  4,  6,  8,  10, 12, 14, 16,  18,  20,  22,  24,  28,  32, 36,
                                    40, 44, 48, 56, 64, 80, 96, 112, 128, 144, 160, 192, 256};
-    const int sms = 152, resident = sms * tiled_warps(mode);
-    const int out = out_cols(K, mode), n_strips = (nx + out - 1) / out, n_edge = n_strips < 2 ? n_strips : 2;
-    const auto tick = [](double warps) { return 1150.0 + 490.0 * (warps > 1.0 ? warps : 1.0); };
+    const int sms = 152, resident = sms * warps, n_edge = n_strips < 2 ? n_strips : 2;
+    const auto tick = [&](double w) { return base + slope * (w > 1.0 ? w : 1.0); };
     const auto even = [&](int r) { return (ny + (ny + r - 1) / r - 1) / ((ny + r - 1) / r); };   // equal chunks of at most r
     double best = -1.0;
     for (int t : kTry) {
+        if (t < repeat / 2 && t < ny) continue;        // rows that an item mostly repeats
         const int r = even(t), re = even((5 * t + 7) / 8);
         const long long n = (long long)n_edge * ((ny + re - 1) / re) + (long long)(n_strips - n_edge) * ((ny + r - 1) / r);
         const long long full = n / resident, rest = n % resident;
-        double cost = (r + 2 * K) * (full * tick(tiled_warps(mode) / 4.0) + (rest ? tick(rest / (4.0 * sms)) : 0.0));
-        const double edge = (re + 2 * K) * (tick(full ? tiled_warps(mode) / 4.0 : rest / (4.0 * sms)) + 1000.0);
+        double cost = (r + repeat) * (full * tick(warps / 4.0) + (rest ? tick(rest / (4.0 * sms)) : 0.0));
+        const double edge = (re + repeat) * (tick(full ? warps / 4.0 : rest / (4.0 * sms)) + edge_more);
         if (edge > cost) cost = edge;
         if (best < 0.0 || cost < best) {
             best = cost;

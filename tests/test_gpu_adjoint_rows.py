@@ -52,7 +52,7 @@ def compare(p, gauges, steps, checkpoints):
     b.close()
 
 
-@pytest.mark.parametrize("nx,ny", [(2, 9), (3, 5), (4, 4), (5, 33), (119, 6), (120, 7), (121, 8), (123, 9), (124, 30), (125, 3),
+@pytest.mark.parametrize("nx,ny", [(1, 7), (59, 5), (60, 7), (61, 6), (62, 9), (63, 4), (2, 9), (3, 5), (4, 4), (5, 33), (119, 6), (120, 7), (121, 8), (123, 9), (124, 30), (125, 3),
                                    (240, 17), (241, 2), (244, 1), (400, 61)])
 def test_item_edges(nx, ny):
     gauges = np.array([[0, 0], [nx - 1, ny - 1], [nx // 2, ny // 2], [min(119, nx - 1), ny - 1], [min(120, nx - 1), 0]])
