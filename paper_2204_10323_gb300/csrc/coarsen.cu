@@ -27,6 +27,13 @@ namespace {
 // Where s overflows (or the block holds Inf or NaN) the block is summed in double.
 constexpr int kSmall = 16;
 
+// sum / count, the division of the slow FP64 pipe left out where the quotient is a scaling by a power of two.
+__device__ __forceinline__ double mean_of(double sum, int count)
+{
+    if ((count & (count - 1)) == 0) return sum * __hiloint2double((1023 - (31 - __clz(count))) << 20, 0);
+    return sum / (double)count;
+}
+
 template <typename T, int V> struct alignas(sizeof(T) * V) Vec {
     T v[V];
 };
@@ -67,15 +74,13 @@ __global__ void __launch_bounds__(128) coarsen_small_kernel(const T *__restrict_
         if (!std::is_same<T, float>::value || !whole) {
             for (int j = j0; j < j1; j++) {
                 const T *row = src + (size_t)j * nx;
-                double e = 0.0;                         // row by row: the rounding of 2 f additions, not f^2
                 for (int i = i0; i < i1; i += V) {
                     const Vec<T, V> x = *reinterpret_cast<const Vec<T, V> *>(row + i);
 #pragma unroll
-                    for (int k = 0; k < V; k++) e += (double)x.v[k];
+                    for (int k = 0; k < V; k++) d += (double)x.v[k];
                 }
-                d += e;
             }
-            out = (T)(d / (double)count);
+            out = (T)mean_of(d, count);
         }
         dst[(size_t)J * mx + I] = out;
     }
@@ -93,11 +98,11 @@ __global__ void coarsen_kernel(const T *src, int nx, int ny, int f, T *dst, int 
         double s = 0.0;
         for (int j = j0; j < j1; j++) {
             const T *row = src + (size_t)j * nx;
-            double e = 0.0;
-            for (int i = i0; i < i1; i++) e += (double)row[i];
-            s += e;
+            double e = (double)row[i0];                     // row by row: the rounding of 2 f additions, not f^2
+            for (int i = i0 + 1; i < i1; i++) e += (double)row[i];
+            s = j == j0 ? e : s + e;
         }
-        dst[(size_t)J * mx + I] = (T)(s / (double)((j1 - j0) * (i1 - i0)));
+        dst[(size_t)J * mx + I] = (T)mean_of(s, (j1 - j0) * (i1 - i0));
     }
 }
 
