@@ -31,7 +31,7 @@ namespace flood {
 
 namespace {
 
-constexpr int BX = 32, BY = 8;
+constexpr int BX = 32;
 
 // ---------------------------------------------------------------- forward faces per precision
 template <typename T> struct Fwd;
@@ -454,7 +454,7 @@ __device__ void inflow_adjoint(const AdjArgs<T> &A, const int k, double *red)
         if (!(hh > 0.0)) continue;
         const double w = (double)a.inflow_q[(size_t)a.s * a.n_slots + S.slot0 + c] * dx;
         const double nu = c == tid ? nu0 : inward * (lq_of(idx) + inward * dtdx * lhu_of(idx)) / dx;
-        A.gn[idx] += (w / (double)a.n[idx]) * (Nn / D - nu);
+        A.gn_in[S.slot0 + c] += (w / (double)a.n[idx]) * (Nn / D - nu);   // (sections may share a corner cell)
     }
 }
 
@@ -1323,18 +1323,23 @@ cudaError_t launch_gn_out(const Geom &g, const double *gn, T *dst, cudaStream_t 
 template cudaError_t launch_gn_out<float>(const Geom &, const double *, float *, cudaStream_t);
 
 namespace {
-__global__ void gn_inflow_add_kernel(double *gn, const double *gn_in, const int64_t *cells, int n)
+// One block, section by section: a corner cell may belong to several, a cell to a section only once.
+__global__ void __launch_bounds__(256) gn_inflow_add_kernel(double *gn, const double *gn_in, const InflowSec *secs, const int64_t *cells,
+                                                            int n_sec)
 {
-    if (blockIdx.x != 0 || threadIdx.x != 0) return;
-    for (int c = 0; c < n; c++) gn[cells[c]] += gn_in[c];     // in section-cell order (a corner cell may repeat)
+    for (int k = 0; k < n_sec; k++) {
+        const InflowSec S = secs[k];
+        for (int c = threadIdx.x; c < S.ncell; c += 256) gn[cells[S.cell0 + c]] += gn_in[S.slot0 + c];
+        __syncthreads();
+    }
 }
 }  // namespace
 
-cudaError_t launch_gn_inflow_add(double *gn, const double *gn_in, const int64_t *sec_cells, int n_cells,
+cudaError_t launch_gn_inflow_add(double *gn, const double *gn_in, const InflowSec *secs, const int64_t *sec_cells, int n_sec,
                                  cudaStream_t st)
 {
-    if (n_cells <= 0) return cudaSuccess;
-    gn_inflow_add_kernel<<<1, 32, 0, st>>>(gn, gn_in, sec_cells, n_cells);
+    if (n_sec <= 0) return cudaSuccess;
+    gn_inflow_add_kernel<<<1, 256, 0, st>>>(gn, gn_in, secs, sec_cells, n_sec);
     return cudaGetLastError();
 }
 template cudaError_t launch_gn_out<double>(const Geom &, const double *, double *, cudaStream_t);

@@ -93,11 +93,12 @@ struct Sweep {
     void *lhu = nullptr;
     void *scratch = nullptr;      // the scheme options' reverse step: 11 planes of pitch x (ny + 1)
     double *gn = nullptr;
-    double *gn_in = nullptr;      // FP32, Eq. 3 as printed, with inflow sections: their dL/dn terms per cell
+    double *gn_in = nullptr;      // with inflow sections: their dL/dn terms by slot
     int n_in_cells = 0;
     // what pass 3 needs of each reverse step, kept for up to log_cap steps and then worked off at once: a launch
     // per step for a section's few hundred cells took as long as the step
     static constexpr int kLogSteps = 512;
+    static constexpr int64_t kLogBytes = 32 << 20;       // long sections keep fewer steps
     float2 *in_log = nullptr;
     double *in_terms = nullptr;
     int log_cap = 0, logged_steps = 0;
@@ -334,6 +335,7 @@ flood_status reverse_step_t(Sweep &S)
     A.n_gauges = S.G;
     A.seed = S.seed + (size_t)k * S.G;      // dL/dh after step k, added to lambda_{k+1}
     A.scratch = (T *)S.scratch;
+    A.gn_in = S.gn_in;
     if (S.in_log) {
         if (S.logged_steps == S.log_cap && (st = flush_inflow(S))) return st;
         if (S.logged_steps == 0) S.log_first = g;
@@ -519,13 +521,18 @@ extern "C" flood_status flood_adjoint(flood_handle *h, int64_t n_steps, const in
     const bool opts = h->geo.theta != 1.0 || h->geo.friction != 0;
     if (opts) S.scratch = alloc(11 * S.plane_y);
     S.gn = (double *)alloc(P * h->geo.ny * sizeof(double));
-    if (h->prec == FLOOD_F32 && !opts && h->n_in > 0) {      // pass 3 runs over many steps at once
-        S.n_in_cells = h->n_slots;
-        S.log_cap = (int)std::min<int64_t>(n_steps, Sweep::kLogSteps);
+    if (h->n_in > 0) {
+        S.n_in_cells = std::max(h->n_slots, 1);
         S.gn_in = (double *)alloc((size_t)S.n_in_cells * sizeof(double));
-        S.in_log = (float2 *)alloc((size_t)S.log_cap * h->n_slots * sizeof(float2));
-        S.in_terms = (double *)alloc((size_t)S.log_cap * h->n_slots * sizeof(double));
-        if (!S.gn_in || !S.in_log || !S.in_terms) {
+        bool ok = S.gn_in != nullptr;
+        if (h->prec == FLOOD_F32 && !opts) {             // pass 3 runs over many steps at once
+            const int64_t entry = (int64_t)S.n_in_cells * (sizeof(float2) + sizeof(double));
+            S.log_cap = (int)std::max<int64_t>(std::min({n_steps, (int64_t)Sweep::kLogSteps, Sweep::kLogBytes / entry}), 1);
+            S.in_log = (float2 *)alloc((size_t)S.log_cap * S.n_in_cells * sizeof(float2));
+            S.in_terms = (double *)alloc((size_t)S.log_cap * S.n_in_cells * sizeof(double));
+            ok = ok && S.in_log && S.in_terms;
+        }
+        if (!ok) {
             release();
             return fail(h, FLOOD_ERR_OOM, "adjoint buffer allocation");
         }
@@ -630,7 +637,7 @@ extern "C" flood_status flood_adjoint(flood_handle *h, int64_t n_steps, const in
         h->adj_prof_fwd_ms = sum_pairs(S.ev_fwd);
     }
     // outputs
-    if (S.gn_in) CKF(launch_gn_inflow_add(S.gn, S.gn_in, h->sec_cells, S.n_in_cells, h->stream));
+    if (S.gn_in) CKF(launch_gn_inflow_add(S.gn, S.gn_in, h->secs_dev, h->sec_cells, h->n_in, h->stream));
     {
         flood_status st = FLOOD_OK;
         if (h->prec == FLOOD_F32) st = (flood_status)(launch_gn_out<float>(h->geo, S.gn, (float *)S.lhu, h->stream) ? FLOOD_ERR_CUDA : FLOOD_OK);

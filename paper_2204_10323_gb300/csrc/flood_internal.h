@@ -188,6 +188,7 @@ struct AdjArgs {
                                   // depth and lambda_q of the face at this step, for pass 3
                                   // (launch_adjoint_inflow); null without inflow sections
 };
+    double *gn_in;                // FP64 and scheme options: the sections' dL/dn terms by slot (launch_gn_inflow_add)
 template <typename T>
 cudaError_t launch_adjoint_step(const AdjArgs<T> &a, cudaStream_t st);
 // Pass 3 of the FP32 sweep (Eq. 3 as printed): the inflow sections' dL/dn terms of n_entries logged steps,
@@ -216,8 +217,8 @@ cudaError_t encode_map_f32(void *map, const float *base, int width, int height, 
 // dst (pitched, precision T) = gn (pitched doubles).
 template <typename T>
 cudaError_t launch_gn_out(const Geom &g, const double *gn, T *dst, cudaStream_t st);
-// gn[sec_cells[c]] += gn_in[c] for c = 0 .. n_cells - 1, in that order.
-cudaError_t launch_gn_inflow_add(double *gn, const double *gn_in, const int64_t *sec_cells, int n_cells,
+// The sections' terms gn_in (by slot) into gn, section by section.
+cudaError_t launch_gn_inflow_add(double *gn, const double *gn_in, const InflowSec *secs, const int64_t *sec_cells, int n_sec,
                                  cudaStream_t st);
 
 // Pitch padding (columns [cols, pitch) of rows x pitch elements of esz bytes):

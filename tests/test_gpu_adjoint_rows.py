@@ -69,3 +69,20 @@ def test_more_steps_than_the_inflow_log_holds():
     # 600 steps against a log of 512; the errors of 600 steps stay below the bound of 40 deep-water steps
     # because the perturbations leave through the outflow sections
     compare(case(40, 12, 2), np.array([[5, 5], [30, 2]]), 600, 40)
+
+
+@pytest.mark.parametrize("theta,friction", [(1.0, 0), (0.9, 1)])
+@pytest.mark.parametrize("precision", [0, 1])
+def test_sections_that_share_a_corner_cell(precision, theta, friction):
+    """Three inflow sections hold cell (0, 0), two the last one: their terms all reach dL/dn, in one order."""
+    Fm = F()
+    p = case(1, 7, 8)
+    p.opts.theta, p.opts.friction = theta, friction
+    w = np.random.default_rng(1).standard_normal((12, 2))
+    out = []
+    for _ in range(40):
+        sim = Fm.Sim(p, precision=precision)
+        out.append(sim.adjoint(12, np.array([[0, 0], [0, 6]]), w, n_checkpoints=12))
+        sim.close()
+    for g in out[1:]:
+        assert np.array_equal(g, out[0])
