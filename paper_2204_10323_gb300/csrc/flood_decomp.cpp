@@ -365,6 +365,13 @@ extern "C" flood_status flood_decomp_step(flood_decomp *d, int64_t n_steps)
     NvtxRange range("flood: decomposed steps");
     const int E = d->E;
     int64_t done = 0;
+    // a state written through one part's own handle has swapped that part's halves alone
+    for (int r = 0; r < d->n_parts; r++)
+        if (d->parts[r]->cur != (d->cur0[r] ^ phase(d))) {
+            flood_status st = build_tables(d);
+            if (st) return st;
+            break;
+        }
     {
         flood_status st = fork_lanes(d);      // whatever the caller queued comes first
         if (st) return st;
