@@ -187,8 +187,8 @@ struct AdjArgs {
     float2 *in_log;               // FP32, Eq. 3 as printed: per inflow slot, the adjoint of the cell's unclipped
                                   // depth and lambda_q of the face at this step, for pass 3
                                   // (launch_adjoint_inflow); null without inflow sections
-};
     double *gn_in;                // FP64 and scheme options: the sections' dL/dn terms by slot (launch_gn_inflow_add)
+};
 template <typename T>
 cudaError_t launch_adjoint_step(const AdjArgs<T> &a, cudaStream_t st);
 // Pass 3 of the FP32 sweep (Eq. 3 as printed): the inflow sections' dL/dn terms of n_entries logged steps,
