@@ -38,10 +38,11 @@ template <typename T> struct Fwd;
 
 template <> struct Fwd<double> {
     double g, dt, dx, hd;
-    __device__ Fwd(const Geom &G, double dt_) : g(G.g), dt(dt_), dx(G.dx), hd(G.h_dry) {}
+    Divisor<double> over_dx;
+    __device__ Fwd(const Geom &G, double dt_) : g(G.g), dt(dt_), dx(G.dx), hd(G.h_dry), over_dx(G.dx) {}
     __device__ double face(double q, double hL, double zL, double nL, double hR, double zR, double nR) const
     {
-        return face_update_ieee<double>(q, fabs(q), hL, zL, nL, hR, zR, nR, g, dt, dx, hd);
+        return face_update_ieee<double>(q, fabs(q), hL, zL, nL, hR, zR, nR, g, dt, over_dx, hd);
     }
     __device__ double hf(double hL, double zL, double hR, double zR) const
     {
@@ -56,7 +57,7 @@ template <> struct Fwd<double> {
     {
         using O = R<double>;
         double dv = O::add(O::sub(qW, qE), O::sub(qS, qN));
-        return O::add(h, O::div(O::mul(dt, dv), dx));
+        return O::add(h, over_dx.under(O::mul(dt, dv)));
     }
     __device__ static double rcp_(double x) { return 1.0 / x; }
     __device__ static double pow_m73_(double x) { const double m = ::rcbrt(x), r = 1.0 / x; return m * r * r; }
@@ -534,7 +535,7 @@ __device__ __forceinline__ unsigned long long f2rcp(unsigned long long a)
     return f2pack(rcp_fast(v.x), rcp_fast(v.y));
 }
 
-// Eq. 3 for two faces (the operations of face_fast_sel_x2, in its order), with what its derivatives
+// Eq. 3 for two faces (the operations of face_fast_sel, in its order), with what its derivatives
 // need.  A dry face is evaluated at depth 1 with a zero reciprocal of its denominator, which makes
 // its value and its derivatives zero.
 struct Faces2 {
@@ -1040,9 +1041,10 @@ template <> struct OptFace<float> {
 };
 
 template <> struct OptFace<double> {
-    double g, dt, dx, hd, th, w;
+    double g, dt, hd, th, w;
+    Divisor<double> over_dx;
     __device__ OptFace(const Geom &G, double dt_)
-        : g(G.g), dt(dt_), dx(G.dx), hd(G.h_dry), th(G.theta), w(0.5 * (1.0 - G.theta)) {}
+        : g(G.g), dt(dt_), hd(G.h_dry), th(G.theta), w(0.5 * (1.0 - G.theta)), over_dx(G.dx) {}
     __device__ double qn(double q, double qp, double qx, bool t) const { return theta_q_ieee<double>(q, qp, qx, th, w, t); }
     __device__ double qm(double q, double a, double b, double c, double d, bool vec) const
     {
@@ -1056,7 +1058,7 @@ template <> struct OptFace<double> {
     __device__ double face(double qmag, double qnum, double hL, double zL, double nL, double hR, double zR,
                            double nR) const
     {
-        return face_update_ieee<double>(qnum, qmag, hL, zL, nL, hR, zR, nR, g, dt, dx, hd);
+        return face_update_ieee<double>(qnum, qmag, hL, zL, nL, hR, zR, nR, g, dt, over_dx, hd);
     }
 };
 

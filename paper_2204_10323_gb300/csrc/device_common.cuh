@@ -39,6 +39,40 @@ template <> struct R<double> {
     static __device__ __forceinline__ double abs(double a) { return fabs(a); }
 };
 
+// Correctly rounded a / b for one positive divisor and many dividends (a step divides by dx three times a cell).
+// FP64: q0 = RN(a y) with y = RN(1 / b), r = a - q0 b (exact by fma), RN(q0 + r y), which is RN(a / b) by Markstein's
+// theorem (IBM J. Res. Dev. 34, 1990: a faithful q0 and a correctly rounded y suffice, nothing under- or
+// overflowing).  q0 is faithful where |y b - 1| <= 2^-54: then a y lies less than half a unit in the last place of a / b
+// from it (a quarter just above a power of two).  That holds for 1, 3, 5 and their multiples by powers of two;
+// elsewhere, and for tiny or huge dividends, the ordinary division, which takes about eight operations
+// of the FP64 pipe (two a cycle and SM) for the three here.
+template <typename T> struct Divisor {
+    T b;
+    __device__ explicit Divisor(T b_) : b(b_) {}
+    __device__ T under(T a) const { return R<T>::div(a, b); }
+};
+
+template <> struct Divisor<double> {
+    double b, y;
+    bool quick;
+    __device__ explicit Divisor(double b_)
+    {
+        b = b_;
+        y = __ddiv_rn(1.0, b_);
+        quick = b >= 0x1p-20 && b <= 0x1p20 && fabs(__fma_rn(y, b, -1.0)) <= 0x1p-54;
+    }
+    __device__ double under(double a) const
+    {
+        const int hi = __double2hiint(a), e = (hi >> 20) & 0x7ff;
+        if (quick && (unsigned)(e - 323) < 1300u) {    // 2^-700 <= |a| < 2^600
+            const double q = __dmul_rn(a, y);
+            return __fma_rn(__fma_rn(-q, b, a), y, q);
+        }
+        if (((hi << 1) | __double2loint(a)) == 0) return a;   // a zero keeps its sign
+        return __ddiv_rn(a, b);
+    }
+};
+
 // Eq. 3 at one interior face between cell L (lower index) and R, with the
 // time step in the numerator and h_f = max(eta_L, eta_R) - max(z_L, z_R);
 // 0 when h_f <= h_dry.  qn is the discharge in the numerator (q itself unless
@@ -46,12 +80,12 @@ template <> struct R<double> {
 // Operations in the order of the plain definition, each rounded once (no
 // contraction).
 template <typename T>
-__device__ __forceinline__ T face_wet_ieee(T qn, T qmag, T etaL, T etaR, T hf, T nL, T nR, T g, T dt, T dx)
+__device__ __forceinline__ T face_wet_ieee(T qn, T qmag, T etaL, T etaR, T hf, T nL, T nR, T g, T dt, const Divisor<T> &dx)
 {
     using O = R<T>;
     T nf = O::mul(T(0.5), O::add(nL, nR));
     T gdt = O::mul(g, dt);
-    T slope_term = O::div(O::mul(O::mul(gdt, hf), O::sub(etaR, etaL)), dx);
+    T slope_term = dx.under(O::mul(O::mul(gdt, hf), O::sub(etaR, etaL)));
     T hf_m73 = O::div(T(1), O::mul(O::mul(hf, hf), O::cbrt(hf)));
     T friction = O::mul(O::mul(O::mul(O::mul(gdt, nf), nf), qmag), hf_m73);
     return O::div(O::sub(qn, slope_term), O::add(T(1), friction));
@@ -59,7 +93,7 @@ __device__ __forceinline__ T face_wet_ieee(T qn, T qmag, T etaL, T etaR, T hf, T
 
 template <typename T>
 __device__ __forceinline__ T face_update_ieee(T qn, T qmag, T hL, T zL, T nL, T hR, T zR, T nR, T g, T dt,
-                                              T dx, T h_dry)
+                                              const Divisor<T> &dx, T h_dry)
 {
     using O = R<T>;
     T etaL = O::add(hL, zL), etaR = O::add(hR, zR);

@@ -9,11 +9,11 @@
 // the x-faces' lanes and rows/(rows + 1) of the y-faces are new), and both cells take
 // the same bits, so the update conserves mass exactly like the face-by-face definition.
 //
-// FP64 is bound by its pipe: two operations a cycle and SM, about 60 per wet face
-// (three divisions and a cube root).  A dry face takes its maxima and its test on the
-// integer units, and a cell between four dry faces keeps its depth, so dry land costs four
-// operations a cell.  A thread per cell computing its four faces itself took 274 us a step
-// at 1001 x 777 (30 % wet; now 130), 36 at 128^2 (now 15).
+// FP64 is bound by its pipe: two operations a cycle and SM, about 55 per wet face
+// (two divisions and a cube root; the division by dx takes three, Divisor).  A dry face takes its
+// maxima and its test on the integer units, and a cell between four dry faces keeps its depth, so dry
+// land costs four operations a cell.  A thread per cell computing its four faces itself took 274 us a step
+// at 1001 x 777 (30 % wet; now 114, 130 with the ordinary division by dx), 36 at 128^2 (now 14.5).
 #include "device_common.cuh"
 #include "pdl.cuh"
 
@@ -85,7 +85,8 @@ __global__ void __launch_bounds__(32) step_reference_kernel(const __grid_constan
     const int x0 = (int)(blockIdx.x % (unsigned)n_strips) * kCols, c = x0 + lane;
     const int y0 = (int)(blockIdx.x / (unsigned)n_strips) * rows, y1 = min(y0 + rows, ny);
     const size_t P = (size_t)G.pitch;
-    const T dt = T(a.ctrl->dt), dx = T(G.dx), g = T(G.g), hd = T(G.h_dry);
+    const T dt = T(a.ctrl->dt), g = T(G.g), hd = T(G.h_dry);
+    const Divisor<T> dx(T(G.dx));
     const bool wt = G.theta != 1.0;                   // theta-weighted numerator discharges
     const bool vec = G.friction != 0;                 // vector-norm |q| in the friction term
     const T th = T(G.theta), w = T(0.5 * (1.0 - G.theta));
@@ -132,7 +133,7 @@ __global__ void __launch_bounds__(32) step_reference_kernel(const __grid_constan
                 T hn = hp;                              // four dry faces: hp + dt 0 / dx
                 if (!all_zero(xp, xe, yp, ys)) {
                     const T dv = O::add(O::sub(xp, xe), O::sub(yp, ys));
-                    hn = O::add(hp, O::div(O::mul(dt, dv), dx));
+                    hn = O::add(hp, dx.under(O::mul(dt, dv)));
                 }
                 if (hn < T(0)) {
                     if (j - 1 >= G.led_j0 && j - 1 < G.led_j1) vclip += -(double)hn * G.dx * G.dx;
@@ -199,7 +200,7 @@ __global__ void __launch_bounds__(32) step_reference_kernel(const __grid_constan
 }
 
 // Rows per item: an item of r rows computes 2 r + 1 rows of faces, but the FP64 pipes even out over many
-// short items, whose wet ones cluster.  us a step at 1 / 2 / 3 / 4 / 8 rows: 15.3 / 21.5 / 25.8 / 31.8 / 53.1
+// short items, whose wet ones cluster.  us a step (with the ordinary division by dx) at 1 / 2 / 3 / 4 / 8 rows: 15.3 / 21.5 / 25.8 / 31.8 / 53.1
 // (128^2), 59 / 68 / 66 / 67 / 85 (512^2), 142 / 130 / 142 / 134 / 139 (1001 x 777), 117 / 107 / 105 / 109 /
 // 112 (1200^2, 10 % wet), 298 / 261 / 251 / 255 / 255 (1001 x 777, 90 % wet).
 int reference_rows(int nx, int ny)
