@@ -6,8 +6,9 @@ fastest, and caches the choice in a JSON file keyed by the device name and the
 scenario shapes (``$FLOOD_AUTOTUNE_CACHE`` or
 ``~/.cache/paper_2204_10323_gb300/autotune.json``).  K = 0 is the single-step
 stream kernel (warps and rows shape its blocks); K >= 1 the temporal-blocking
-kernel with K steps per launch (rows per (chunk, strip) item of a 2^20-cell
-grid, scaled by the square root of each grid's cells).  Every
+kernel with K steps per launch (the most rows per (chunk, strip) item of a
+2^20-cell grid, scaled by the square root of each grid's cells; the library
+takes fewer where the items would not fill the GPU evenly).  Every
 candidate computes bit-identical depths and discharges, so tuning on the live
 run does not change its trajectory; it only advances it.
 """

@@ -87,8 +87,8 @@ __device__ __forceinline__ float face_wet(float qmag, float qn, float etaL, floa
 // ---- two faces at once on the paired single-precision instructions
 // (add/sub/mul .f32x2: one instruction for two lanes of a 64-bit register
 // pair, each rounded as the scalar instruction), for the issue-bound
-// temporal-blocking kernel.  face_fast_sel_x2 returns exactly the two values
-// face_fast_sel returns for (x, y): the same operations in the same order.
+// temporal-blocking and reverse-step kernels: faces written with them in
+// face_fast_sel's order return exactly its values.
 __device__ __forceinline__ unsigned long long f2pack(float a, float b)
 {
     unsigned long long r;
@@ -143,32 +143,6 @@ __device__ __forceinline__ float ex2_fast(float x)
     float r;
     asm("ex2.approx.ftz.f32 %0, %1;" : "=f"(r) : "f"(x));
     return r;
-}
-
-// face_fast_sel_gen for two faces: qmag and qn packed (|q| of the friction term,
-// numerator discharge), etaL, etaR, nsum packed, zmax the two faces' max(z_L, z_R).
-__device__ __forceinline__ float2 face_fast_sel_x2_gen(unsigned long long qmag, unsigned long long qn,
-                                                       unsigned long long etaL, unsigned long long etaR, float2 zmax,
-                                                       unsigned long long nsum, const FastConst &k)
-{
-    const float2 eL = f2unpack(etaL), eR = f2unpack(etaR);
-    const unsigned long long hf = f2sub(f2pack(fmaxf(eL.x, eR.x), fmaxf(eL.y, eR.y)), f2pack(zmax.x, zmax.y));
-    const float2 h = f2unpack(hf);
-    const unsigned long long l = f2mul(f2pack(lg2_fast(h.x), lg2_fast(h.y)), f2pack(-7.0f / 3.0f, -7.0f / 3.0f));
-    const float2 lv = f2unpack(l);
-    const unsigned long long r7 = f2pack(ex2_fast(lv.x), ex2_fast(lv.y));
-    const unsigned long long aq = f2mul(f2mul(f2pack(k.gdt4, k.gdt4), f2mul(nsum, nsum)), qmag);
-    const unsigned long long num = f2fma(f2mul(f2pack(-k.a1, -k.a1), hf), f2sub(etaR, etaL), qn);
-    const float2 den = f2unpack(f2fma(aq, r7, f2pack(1.0f, 1.0f)));
-    const float2 v = f2unpack(f2mul(num, f2pack(rcp_fast(den.x), rcp_fast(den.y))));
-    return make_float2(h.x > k.h_dry ? v.x : 0.0f, h.y > k.h_dry ? v.y : 0.0f);
-}
-
-// etaL, etaR, zmax, nsum, q: the two faces' arguments of face_fast_sel.
-__device__ __forceinline__ float2 face_fast_sel_x2(float2 q, unsigned long long etaL, unsigned long long etaR,
-                                                   float2 zmax, unsigned long long nsum, const FastConst &k)
-{
-    return face_fast_sel_x2_gen(f2pack(fabsf(q.x), fabsf(q.y)), f2pack(q.x, q.y), etaL, etaR, zmax, nsum, k);
 }
 
 // theta_q for two faces (packed q, previous and next neighbours).

@@ -477,11 +477,11 @@ namespace flood {
 // of 4, no explicit launch shape), for Eq. 3 as printed and for the scheme
 // options alike, else the tensor-tile kernel below 2^27 cells, else the
 // row-staged stream kernel.  Measured on the fractal workload (us per step,
-// epoch starts included): tiled K = 4 / TMA / stream 15.2 / 16.4 / 18.2 at
-// 1024^2, 29.9 / 33.9 / 39.3 at 2048^2, 89.2 / 102.0 / 105.9 at 4096^2,
-// 296 / 349 / 354 at 8192^2, 1059 / 1305 / 1302 at 16384^2; with vector-norm
-// friction tiled / TMA 16.6 / 18.3, 36.1 / 41.0, 116.4 / 119.2, 385 / 381 and
-// 1396 / 1425.  All of them are bitwise equal.
+// epoch starts included): tiled K = 4 / TMA / stream 8.2 / 13.1 / 15.1 at
+// 1024^2, 13.4 / 30.3 / 35.6 at 2048^2, 39 / 99 / 102 at 4096^2, 120 / 345 /
+// 349 at 8192^2, 463 / 1301 / 1299 at 16384^2; with vector-norm friction tiled /
+// TMA 10.7 / 15.1, 18.1 / 37.6, 54 / 115, 164 / 378 and 626 / 1423.  All of them
+// are bitwise equal.
 int auto_kernel(const flood_opts &o, int nx, int ny)
 {
     const bool tiled = o.epoch_steps % 4 == 0 && o.tile_x == 0 && o.tile_y == 0;

@@ -10,7 +10,8 @@ namespace flood {
 // register at 1024^2 .. 4096^2), and 1000 more in an edge strip, whose items are therefore shorter.  The
 // rows minimise the waves of items, the last one with the warps it has: few rows fill the GPU evenly but
 // repeat 2K rows each.  us per step with rows chosen so / fixed at 96: 11.0 / 36.8 (1024^2), 15.9 / 37.3
-// (2048^2), 39 / 50 (4096^2), 131 / 131 (8192^2), 465 / 477 (16384^2).
+// (2048^2), 39 / 50 (4096^2), 131 / 131 (8192^2), 465 / 477 (16384^2); with the higher beds kept and
+// dependent launches since then 8.2, 13.4, 39, 120 and 463.
 void tiled_rows(int nx, int ny, int K, int mode, int *rows, int *rows_edge)
 {
     const int out = out_cols(K, mode);

@@ -19,7 +19,7 @@
 // each end of a chunk: an item runs 2K ticks more than it has rows.
 //
 // What bounds it: instruction issue.  At 16384^2 a launch of 4 steps executes
-// 1.6 warp instructions per cell-update and moves 8.3 B of DRAM traffic per
+// 1.44 warp instructions per cell-update and moves 8.1 B of DRAM traffic per
 // cell-update.  A pipeline of K warps per strip with the rows handed over through
 // shared memory and a barrier per tick, two z and n loads and a Manning factor
 // per level, executed 3.4.
@@ -146,7 +146,7 @@ __device__ __forceinline__ unsigned long long face_cq(unsigned long long c, unsi
 }
 
 // Eq. 3 for two faces given the flow depth, eta_R - eta_L, the numerator discharge and
-// cq = c |q|: the operations of face_fast_sel_x2_gen, in its order.
+// cq = c |q|: the operations of face_fast_sel_gen, in its order.
 __device__ __forceinline__ unsigned long long faces2(unsigned long long hf, unsigned long long slope,
                                                      unsigned long long qn, unsigned long long cq, const FastConst &k)
 {
