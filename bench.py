@@ -38,18 +38,18 @@ BYTES_PER_CELL = 32          # read h, qx, qy, z, n (20 B) + write h, qx, qy (12
 # smaller case of the same workload (state > L2) in the same launch shape, scaled by
 # the cell count; key (kernel, steps per launch).  Stream kernel: the 4096^2 case in
 # the 4 warps x 32-row chunks of the 16384^2 launch.  Temporal-blocking kernel: the
-# 8192^2 case with the 304-row (chunk, strip) items the 16384^2 launch takes from its
-# counter (--tile 0,304).  Only kernels whose code has not changed since their capture
+# 8192^2 case with the 256-row (chunk, strip) items of the 16384^2 launch
+# (--tile 0,256).  Only kernels whose code has not changed since their capture
 # are listed; the others report traffic null.
-TRAFFIC_B_PER_CELL = {("stream", 1): 31.32, ("tiled", 4): 32.29}
+TRAFFIC_B_PER_CELL = {("stream", 1): 31.32, ("tiled", 4): 32.47}
 # Warp instructions per cell-update of the temporal-blocking kernel (issue-bound), from the same
 # capture (smsp__inst_executed.sum): the "alu" roofline beside the one-step HBM one.  The issue peak is
 # 152 SMs x 4 warp-instructions per cycle x the sampled SM clock.
-INST_PER_CELL_UPDATE = {("tiled", 4): 907034250 / (8192 * 8192 * 4)}
+INST_PER_CELL_UPDATE = {("tiled", 4): 386225911 / (8192 * 8192 * 4)}
 SMS, ISSUE_PER_SM_CYCLE = 152, 4
 # the same two for the vector-norm friction option (theta = 1)
-TRAFFIC_VEC_B_PER_CELL = {("tiled", 4): 32.27}
-INST_VEC_PER_CELL_UPDATE = {("tiled", 4): 1117140607 / (8192 * 8192 * 4)}
+TRAFFIC_VEC_B_PER_CELL = {("tiled", 4): 32.50}
+INST_VEC_PER_CELL_UPDATE = {("tiled", 4): 509070602 / (8192 * 8192 * 4)}
 METRIC = "Gcell-updates/s and % of HBM roofline (FP32, 1 GB300); adjoint/forward time ratio"
 UNIT = "Gcell-updates/s"
 
@@ -281,7 +281,7 @@ def timed_run(F, torch, prob, kernel_name, k, tile, graph, steps_req, warmup, lo
         # launches that neither start an epoch nor are cut short run the step kernel alone
         kern += [ev[j].elapsed_time(ev[j + 1]) for j, (begin, kk) in enumerate(plan) if not begin and kk == per_launch]
         n_epochs = sum(1 for begin, _ in plan if begin)
-        launches += len(plan) + n_epochs * (1 + (1 if sim_inflows(prob) else 0))
+        launches += len(plan) + n_epochs       # an epoch starts in one launch
     clk = clocks.stop()
     sim.sync()
     total_ms = max_over_ranks(statistics.median(runs_ms), dist)
@@ -570,9 +570,9 @@ def ensemble_throughput(F, torch, single_value: float, n: int = 96, steps: int =
 
 def decomposition_leg(F, torch, prob, single_value: float, steps: int, parts=(2, 4), halo: int = 4):
     """The same workload split into 1 x N row strips with `halo`-row halos,
-    exchanged every `halo` steps (all parts on this GPU, each on a stream of its own): whole-job
+    exchanged every `halo` steps (all parts on this GPU, stepped by one launch): whole-job
     Gcell-updates/s and the ratio to the single grid, the cost of the halo rows'
-    redundant steps, the exchanges and the per-part launches."""
+    redundant steps and the exchanges."""
     out = []
     E = prob.opts.epoch_steps
     n = max(steps, 2 * E)
@@ -594,10 +594,6 @@ def decomposition_leg(F, torch, prob, single_value: float, steps: int, parts=(2,
                     "ratio_to_single_grid": value / single_value})
         d.close()
     return {"what": "1 x N row strips with halo exchange on one GPU (the paper's subgrids)", "runs": out}
-
-
-def sim_inflows(prob):
-    return any(s.kind == 0 for s in prob.sections)
 
 
 def main():
