@@ -59,7 +59,9 @@ struct flood_decomp {
     bool batched = false;                    // one launch for all parts (FP32, temporal blocking, no caller's launch shape)
     StepArgs<float> *args_dev[2] = {nullptr, nullptr};
     int *base_dev = nullptr;                 // item prefix, n_parts + 1
-    int total_items = 0, mode = 0;
+    std::vector<StepArgs<float>> args[2];    // the same on the host
+    std::vector<int> base;
+    int mode = 0;
     EpochArgs<float> *etab_dev = nullptr;
     int2 *tasks_dev = nullptr;               // (part, inflow section)
     int n_tasks = 0;
@@ -148,9 +150,11 @@ flood_status build_tables(flood_decomp *d)
             d->halo_units = std::max(d->halo_units, e.units);
             halo.push_back(e);
         }
-        std::vector<StepArgs<float>> args(d->batched ? n : 0);
-        std::vector<int> base(1, 0);
+        std::vector<StepArgs<float>> &args = d->args[ph];
+        std::vector<int> &base = d->base;
         if (d->batched) {
+            args.resize(n);
+            base.assign(1, 0);
             int rows = 0, edge = 0;
             tiled_rows(d->nx, d->ny, d->parts[0]->k_per_launch, d->mode, &rows, &edge);   // as for the whole grid
             for (int r = 0; r < n; r++) {
@@ -160,7 +164,6 @@ flood_status build_tables(flood_decomp *d)
                 base.push_back(base.back() +
                                tiled_items(d->parts[r]->geo, args[r].tile_y, args[r].tile_x, d->parts[r]->k_per_launch));
             }
-            d->total_items = base.back();
         }
         cudaError_t e = cudaSuccess;
         if (!halo.empty())
@@ -191,8 +194,9 @@ flood_status step_batched(flood_decomp *d, int s, int m)
 {
     for (int done = 0; done < m;) {
         const int k = std::min(d->parts[0]->k_per_launch, m - done);
-        DCK(launch_step_tiled_ensemble(d->args_dev[phase(d)], d->base_dev, d->n_parts, d->total_items, k, s + done,
-                                       s + done + k == d->E ? 1 : 0, d->mode, d->stream));
+        const int ph = phase(d);
+        const GridTable t = {d->args_dev[ph], d->args[ph].data(), d->base_dev, d->base.data(), d->n_parts};
+        DCK(launch_step_tiled_ensemble(t, k, s + done, s + done + k == d->E ? 1 : 0, d->mode, d->stream));
         for (flood_handle *h : d->parts) {
             h->cur = 1 - h->cur;
             h->step += k;

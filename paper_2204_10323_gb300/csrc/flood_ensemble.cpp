@@ -42,7 +42,9 @@ struct flood_ensemble {
     std::vector<int> group_of;             // per member
     StepArgs<float> *gtable[kGroups][2] = {{nullptr, nullptr}, {nullptr, nullptr}};   // [group][parity]
     int *gtbase[kGroups] = {nullptr, nullptr};
-    int gn[kGroups] = {0, 0}, gtotal[kGroups] = {0, 0};
+    std::vector<StepArgs<float>> gargs[kGroups][2];          // the same on the host
+    std::vector<int> gitems[kGroups];
+    int gn[kGroups] = {0, 0};
     EpochArgs<float> *getab[kGroups] = {nullptr, nullptr};   // the group's members' epoch arguments
     int2 *gtasks[kGroups] = {nullptr, nullptr};              // (member in the group, inflow section)
     int gntasks[kGroups] = {0, 0};
@@ -97,7 +99,8 @@ int edge_rows(int rows) { return (5 * rows + 7) / 8; }
 // with its longest items' last rows, so few rows cost work and many leave warps idle.  The cost is
 // the items' ticks over the warps that the GPU holds, or the longest item if that is more, and a tenth of the
 // longest item for the tail (two groups fill each other's).  20 scenarios of 256^2 .. 2048^2, us a step at 32 / 48 /
-// 64 / 96 / 128 / 256 rows: 72.4 / 68.0 / 66.4 / 79.9 / 94.6 / 157.
+// 64 / 96 / 128 / 256 rows: 72.4 / 68.0 / 66.4 / 79.9 / 94.6 / 157.  (With the arguments in the launch 61.2 at the
+// 64 chosen.)
 void choose_rows(flood_ensemble *e)
 {
     const double resident = 152.0 * 12.0;      // one-warp items the GPU holds at once
@@ -165,15 +168,16 @@ flood_status build_tables(flood_ensemble *e)
         }
         for (int g = 0; g < flood_ensemble::kGroups; g++) {
             const int ng = (int)members[g].size();
-            std::vector<int> gb(ng + 1, 0);
+            std::vector<int> &gb = e->gitems[g];
+            gb.assign(ng + 1, 0);
             for (int i = 0; i < ng; i++) {
                 const Geom &G = e->members[members[g][i]]->geo;
                 gb[i + 1] = gb[i] + tiled_items(G, item_rows(e, G), edge_rows(item_rows(e, G)), e->k_steps);
             }
             e->gn[g] = ng;
-            e->gtotal[g] = gb[ng];
             for (int p = 0; p < 2; p++) {
-                std::vector<StepArgs<float>> t(ng);
+                std::vector<StepArgs<float>> &t = e->gargs[g][p];
+                t.resize(ng);
                 for (int i = 0; i < ng; i++) {
                     flood_handle *h = e->members[members[g][i]];
                     const int cur = h->cur;
@@ -275,8 +279,8 @@ flood_status ensemble_step(flood_ensemble *e, int64_t limit, cudaStream_t st, in
         c = cudaSuccess;
         for (int g = 0; g < flood_ensemble::kGroups && c == cudaSuccess; g++) {
             if (e->gn[g] == 0) continue;
-            c = launch_step_tiled_ensemble(e->gtable[g][parity], e->gtbase[g], e->gn[g], e->gtotal[g], steps, s,
-                                           s + steps == E ? 1 : 0, e->mode, e->lane[g]);
+            const GridTable t = {e->gtable[g][parity], e->gargs[g][parity].data(), e->gtbase[g], e->gitems[g].data(), e->gn[g]};
+            c = launch_step_tiled_ensemble(t, steps, s, s + steps == E ? 1 : 0, e->mode, e->lane[g]);
         }
     } else {
         flood_status fs = join_groups(e, st);

@@ -102,16 +102,20 @@ cudaError_t launch_step_stream_ensemble(const StepArgs<float> *table, const int 
 // Blocks of one grid for the stream kernel, and the (warps, rows) a tile pair selects.
 int stream_blocks(const Geom &g, int warps, int rows);
 cudaError_t launch_step_tma(const StepArgs<float> &a, cudaStream_t st);
-// Temporal blocking over many grids: the items of grid k are base[k] .. base[k+1] - 1 (tiled_items per
-// grid, table[k].tile_y rows per item, tile_x in the edge strips), k_steps steps from s0.
+// Temporal blocking over many grids, k_steps steps from s0: the items of grid k are base[k] .. base[k+1] - 1
+// (tiled_items per grid, table[k].tile_y rows per item, tile_x in the edge strips).
 int tiled_items(const Geom &g, int rows, int rows_edge, int k_steps);
 // Rows per work item (inner strips, and the one or two strips with the borders x = 0 and x = nx) for a grid
 // alone on the GPU.
 void tiled_rows(int nx, int ny, int K, int mode, int *rows, int *rows_edge);
 void tiled_rows_for(int n_strips, int ny, int repeat, int warps, double base, double slope, double edge_more, int *rows,
                     int *rows_edge);
-cudaError_t launch_step_tiled_ensemble(const StepArgs<float> *table, const int *base, int n, int total_items,
-                                       int k_steps, int s0, int want_hmax, int mode, cudaStream_t st);
+struct GridTable {
+    const StepArgs<float> *table, *host_table;    // n grids: on the device, and the same on the host
+    const int *base, *host_base;                  // n + 1
+    int n;
+};
+cudaError_t launch_step_tiled_ensemble(const GridTable &t, int k_steps, int s0, int want_hmax, int mode, cudaStream_t st);
 void stream_launch_shape(const Geom &g, int tile_x, int tile_y, int *warps, int *rows);
 cudaError_t launch_step_tiled(const StepArgs<float> &a, cudaStream_t st);
 

@@ -647,31 +647,64 @@ __global__ void __launch_bounds__(32, tiled_warps(kMode)) step_tiled_kernel(cons
     if (blockIdx.x == 0 && threadIdx.x == 0) tiled_finish<K>(a, a.s);
 }
 
-// Many grids: the items of grid k (table[k].tile_x and tile_y rows per item) are numbered
-// base[k] .. base[k+1] - 1, grids ordered largest first; a block per item.  The block keeps its grid's
-// arguments in shared memory.  The grid's first item books its inflow volume and clock.
-template <int K, int kMode>
-__global__ void __launch_bounds__(32, tiled_warps(kMode))
-    step_tiled_ensemble_kernel(const StepArgs<float> *table, const int *base, const int n, const int s0, const int want_hmax)
+// The grid whose items base[k] .. base[k+1] - 1 hold `item`.
+__device__ __forceinline__ int grid_of_item(const int *base, const int n, const int item)
 {
-    __shared__ TiledSmem<kMode> sm;
-    __shared__ StepArgs<float> a;
-    const int item = blockIdx.x;
     int lo = 0, hi = n - 1;
     while (lo < hi) {
         const int mid = (lo + hi + 1) >> 1;
         if (base[mid] <= item) lo = mid;
         else hi = mid - 1;
     }
+    return lo;
+}
+
+// An item of one of many grids.  The grid's first item books its inflow volume and clock.  (The items are
+// numbered for the table's K; a shorter launch's strips may be wider.)
+template <int K, int kMode>
+__device__ __forceinline__ void tiled_run_of_many(const StepArgs<float> &a, const int s0, const int local, const int want_hmax,
+                                                  TiledSmem<kMode> &sm)
+{
+    if (local == 0 && threadIdx.x == 0) tiled_finish<K>(a, s0);
+    if (local >= tiled_item_count(a.geo.nx, a.geo.ny, out_cols(K, kMode), a.tile_y, a.tile_x)) return;
+    tiled_run<K, kMode, false>(a, s0, local, want_hmax, sm);
+}
+
+// Many grids: the items of grid k (table[k].tile_x and tile_y rows per item) are numbered
+// base[k] .. base[k+1] - 1, grids ordered largest first; a block per item.  With the grids' arguments in
+// the launch's own (step_tiled_grids_kernel) they are read from constant memory as a single grid's are;
+// more than fit there come from a table on the device, and the block keeps its grid's in shared memory
+// (12 more registers, and an item starts with two round trips to memory).  One strip of 16384^2 / 4096^2, us a step: 473 / 40.4
+// and 508 / 43.0 (the single grid's kernel 463 / 39.1).
+template <int N>
+struct GridArgs {
+    StepArgs<float> grid[N];
+    int base[N + 1];
+};
+constexpr int kFewGrids = 12, kManyGrids = 104;    // arguments of 4 and 32 KB, the sizes a launch may have
+static_assert(sizeof(GridArgs<kFewGrids>) + 16 <= 4096 && sizeof(GridArgs<kManyGrids>) + 16 <= 32764, "kernel arguments");
+
+template <int K, int kMode, int N>
+__global__ void __launch_bounds__(32, tiled_warps(kMode))
+    step_tiled_grids_kernel(const __grid_constant__ GridArgs<N> g, const int n, const int s0, const int want_hmax)
+{
+    __shared__ TiledSmem<kMode> sm;
+    const int k = grid_of_item(g.base, n, blockIdx.x);
+    tiled_run_of_many<K, kMode>(g.grid[k], s0, (int)blockIdx.x - g.base[k], want_hmax, sm);
+}
+
+template <int K, int kMode>
+__global__ void __launch_bounds__(32, tiled_warps(kMode))
+    step_tiled_ensemble_kernel(const StepArgs<float> *table, const int *base, const int n, const int s0, const int want_hmax)
+{
+    __shared__ TiledSmem<kMode> sm;
+    __shared__ StepArgs<float> a;
+    const int item = blockIdx.x, lo = grid_of_item(base, n, item);
     static_assert(sizeof(StepArgs<float>) % 8 == 0, "copied in 8-byte words");
     for (int w = threadIdx.x; w < (int)(sizeof(StepArgs<float>) / 8); w += 32)
         reinterpret_cast<unsigned long long *>(&a)[w] = reinterpret_cast<const unsigned long long *>(table + lo)[w];
     __syncwarp();
-    const int local = item - base[lo];
-    if (local == 0 && threadIdx.x == 0) tiled_finish<K>(a, s0);
-    // (the items are numbered for the ensemble's K; a shorter launch's strips may be wider)
-    if (local >= tiled_item_count(a.geo.nx, a.geo.ny, out_cols(K, kMode), a.tile_y, a.tile_x)) return;
-    tiled_run<K, kMode, false>(a, s0, local, want_hmax, sm);
+    tiled_run_of_many<K, kMode>(a, s0, item - base[lo], want_hmax, sm);
 }
 
 template <int K, int kMode>
@@ -706,16 +739,29 @@ cudaError_t launch_tiled_mode(const StepArgs<float> &a, cudaStream_t st)
     }
 }
 
-template <int kMode>
-cudaError_t launch_tiled_ensemble_mode(const StepArgs<float> *table, const int *base, int n, int total_items,
-                                       int k_steps, int s0, int want_hmax, cudaStream_t st)
+template <int K, int kMode, int N>
+cudaError_t launch_grids(const GridTable &t, int s0, int want_hmax, cudaStream_t st)
 {
-    if (total_items < 1) return cudaSuccess;
+    GridArgs<N> g = {};
+    for (int k = 0; k < t.n; k++) g.grid[k] = t.host_table[k];
+    for (int k = 0; k <= t.n; k++) g.base[k] = t.host_base[k];
+    step_tiled_grids_kernel<K, kMode, N><<<t.host_base[t.n], 32, 0, st>>>(g, t.n, s0, want_hmax);
+    return cudaGetLastError();
+}
+
+// (The arguments' form is built for K = 4, the steps of nearly every launch.)
+template <int kMode>
+cudaError_t launch_tiled_ensemble_mode(const GridTable &t, int k_steps, int s0, int want_hmax, cudaStream_t st)
+{
+    const int items = t.host_base[t.n];
+    if (items < 1) return cudaSuccess;
+    if (k_steps == 4 && t.n <= kFewGrids) return launch_grids<4, kMode, kFewGrids>(t, s0, want_hmax, st);
+    if (k_steps == 4 && t.n <= kManyGrids) return launch_grids<4, kMode, kManyGrids>(t, s0, want_hmax, st);
     switch (k_steps) {
-    case 1: step_tiled_ensemble_kernel<1, kMode><<<total_items, 32, 0, st>>>(table, base, n, s0, want_hmax); break;
-    case 2: step_tiled_ensemble_kernel<2, kMode><<<total_items, 32, 0, st>>>(table, base, n, s0, want_hmax); break;
-    case 3: step_tiled_ensemble_kernel<3, kMode><<<total_items, 32, 0, st>>>(table, base, n, s0, want_hmax); break;
-    case 4: step_tiled_ensemble_kernel<4, kMode><<<total_items, 32, 0, st>>>(table, base, n, s0, want_hmax); break;
+    case 1: step_tiled_ensemble_kernel<1, kMode><<<items, 32, 0, st>>>(t.table, t.base, t.n, s0, want_hmax); break;
+    case 2: step_tiled_ensemble_kernel<2, kMode><<<items, 32, 0, st>>>(t.table, t.base, t.n, s0, want_hmax); break;
+    case 3: step_tiled_ensemble_kernel<3, kMode><<<items, 32, 0, st>>>(t.table, t.base, t.n, s0, want_hmax); break;
+    case 4: step_tiled_ensemble_kernel<4, kMode><<<items, 32, 0, st>>>(t.table, t.base, t.n, s0, want_hmax); break;
     default: return cudaErrorInvalidValue;
     }
     return cudaGetLastError();

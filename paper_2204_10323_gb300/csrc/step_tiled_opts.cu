@@ -16,14 +16,12 @@ cudaError_t launch_step_tiled_opts(const StepArgs<float> &a, int mode, cudaStrea
     }
 }
 
-cudaError_t launch_step_tiled_ensemble_opts(const StepArgs<float> *table, const int *base, int n, int total_items,
-                                            int k_steps, int s0, int want_hmax, int mode,
-                                            cudaStream_t st)
+cudaError_t launch_step_tiled_ensemble_opts(const GridTable &t, int k_steps, int s0, int want_hmax, int mode, cudaStream_t st)
 {
     switch (mode) {
-    case 1: return launch_tiled_ensemble_mode<1>(table, base, n, total_items, k_steps, s0, want_hmax, st);
-    case 2: return launch_tiled_ensemble_mode<2>(table, base, n, total_items, k_steps, s0, want_hmax, st);
-    case 3: return launch_tiled_ensemble_mode<3>(table, base, n, total_items, k_steps, s0, want_hmax, st);
+    case 1: return launch_tiled_ensemble_mode<1>(t, k_steps, s0, want_hmax, st);
+    case 2: return launch_tiled_ensemble_mode<2>(t, k_steps, s0, want_hmax, st);
+    case 3: return launch_tiled_ensemble_mode<3>(t, k_steps, s0, want_hmax, st);
     default: return cudaErrorInvalidValue;
     }
 }
