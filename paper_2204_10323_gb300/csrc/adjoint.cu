@@ -596,8 +596,8 @@ __device__ __forceinline__ float border_lin(int type, float inward, float h, flo
     if (type == kBcInflow) return inward * inflow;
     const float q = outflow_fast(h, sqrtS, n, G.dx_f, G.h_dry_f, G.bc_form);
     if (q > 0.0f) {
-        dh = __fdividef(-inward * (G.bc_form == 0 ? 5.0f / 3.0f : 2.0f / 3.0f) * q, h);
-        dn = __fdividef(inward * q, n);
+        dh = -inward * (G.bc_form == 0 ? 5.0f / 3.0f : 2.0f / 3.0f) * q / h;
+        dn = inward * q / n;
     }
     return -inward * q;
 }
