@@ -349,16 +349,21 @@ __device__ void inflow_body(const Geom &G, const InflowSec *secs, int nsec, cons
         hi = zmin + Hb;
     }
     double lo = zmin;                                  // f, d: at hi
+    // What the section's sum resolves in double: a few roundings of the level.  Newton's step keeps that far from the
+    // bracket's ends (twice as far each time it has to, as the sum's own rounding may hide the root), so that the bracket
+    // closes on the root from both sides.  (Ends 0.9e-12 m apart, the bracket's width, left the level up to that far above.)
+    double least = 1.0;
     for (int it = 0; it < 200 && hi - lo >= 1e-12; it++) {
         const double half = 0.5 * (lo + hi);
         if (!(half > lo && half < hi)) break;          // neighbouring doubles
         double W = half;
-        if (form == 0 && it < 60) {
-            // Newton's step; once it is below the bracket's width, the end of that width from hi (or, where
-            // rounding has left lo at the root, from lo)
+        const double r = least * (sizeof(T) == 8 ? 0x1p-51 * fmax(fabs(hi), hi - zmin) : 0.45e-12);
+        if (form == 0 && it < 60 && hi - lo > 4.0 * r) {
             W = hi - (f - Q) / d;
-            if (W > hi - 0.45e-12) W = hi - 0.9e-12;
-            else if (W <= lo + 0.45e-12) W = lo + 0.9e-12;
+            if (W > hi - r || W < lo + r) {
+                W = W > hi - r ? hi - r : lo + r;
+                least *= 2.0;
+            }
             if (!(W > lo && W < hi)) W = half;
         }
         double dW;

@@ -1,0 +1,53 @@
+"""How closely and in how many evaluations the Eq. 6 level search ends.
+
+Accuracy, FP64: the level itself, from the shares of a section's shallowest and deepest cells (a share's
+relative error is (5/3) dW (1/h - mean 1/h)), against a bisection to neighbouring doubles.  The search
+ends within a few roundings of the level (3 x 4 of the 1.4e-14 m spacing at 100 m): 1.8e-13 m.
+
+Time, FP32 sections beyond one warp's cells: the search of the literal form is the plain halving, about 41
+evaluations of the section; the other form's Newton steps must not need more.
+"""
+import numpy as np
+import pytest
+
+from inputs import INFLOW, XMIN, Options, Problem, Section
+
+pytestmark = pytest.mark.gpu
+
+
+def F():
+    import paper_2204_10323_gb300 as F
+    return F
+
+
+@pytest.mark.parametrize("cells", [13, 60])
+def test_level_of_double_precision_sections(cells):
+    Fm = F()
+    n_sec, nx, dx, S = 40, 4, 5.0, 1e-3
+    ny = n_sec * cells
+    rng = np.random.default_rng(cells)
+    z = 97.0 + rng.uniform(0.0, 0.5, (ny, nx))
+    n = rng.uniform(0.02, 0.06, (ny, nx))
+    Q = 4.0 * cells * rng.uniform(1.0, 4.0, n_sec)
+    secs = [Section.cells(XMIN, k * cells, (k + 1) * cells, INFLOW, S, nx, ny, [0.0, 100.0], [Q[k], Q[k]])
+            for k in range(n_sec)]
+    p = Problem("level", nx, ny, dx, z, n, secs, Options(dt_mode=1, dt_const=0.01, dt_cap=0.01, epoch_steps=1))
+    s = Fm.Sim(p, precision=Fm.F64)
+    s.step(1)
+    qx = s.read(Fm.FIELD_QX)[:, 0]
+    s.close()
+    worst = 0.0
+    for k in range(n_sec):
+        zc, nc, q = (a[k * cells:(k + 1) * cells] for a in (z[:, 0], n[:, 0], qx))
+        share = lambda W: dx * np.maximum(W - zc, 0.0) ** (5.0 / 3.0) * np.sqrt(S) / nc
+        lo, hi = zc.min(), zc.min() + 64.0
+        while lo < 0.5 * (lo + hi) < hi:
+            mid = 0.5 * (lo + hi)
+            lo, hi = (mid, hi) if share(mid).sum() < Q[k] else (lo, mid)
+        h = hi - zc
+        w = share(hi)
+        e = q / (w * (Q[k] / w.sum()) / dx) - 1.0
+        a, b = h.argmin(), h.argmax()
+        assert h[a] > 0.3
+        worst = max(worst, abs((e[a] - e[b]) / (5.0 / 3.0 * (1.0 / h[a] - 1.0 / h[b]))))
+    assert worst <= 1.8e-13, worst
