@@ -51,3 +51,29 @@ def test_level_of_double_precision_sections(cells):
         assert h[a] > 0.3
         worst = max(worst, abs((e[a] - e[b]) / (5.0 / 3.0 * (1.0 / h[a] - 1.0 / h[b]))))
     assert worst <= 1.8e-13, worst
+
+
+def test_long_single_precision_sections_take_no_more_than_the_halving():
+    import torch
+    Fm = F()
+    nx, ny = 6, 1500
+    rng = np.random.default_rng(2)
+    z, n = 50.0 + rng.uniform(0.0, 0.5, (ny, nx)), rng.uniform(0.02, 0.06, (ny, nx))
+    best = []
+    for form in (0, 1):
+        secs = [Section.cells(XMIN, 10, 1410, INFLOW, 1e-3, nx, ny, [0.0, 1e6], [9000.0, 9000.0])]
+        p = Problem("level", nx, ny, 5.0, z, n, secs,
+                    Options(dt_mode=1, dt_const=0.01, dt_cap=0.01, epoch_steps=1, bc_form=form))
+        s = Fm.Sim(p)
+        s.step(20)
+        times = []
+        for _ in range(7):
+            a, b = torch.cuda.Event(enable_timing=True), torch.cuda.Event(enable_timing=True)
+            a.record()
+            s.step(50)
+            b.record()
+            torch.cuda.synchronize()
+            times.append(a.elapsed_time(b))
+        best.append(min(times))
+        s.close()
+    assert best[0] <= 1.1 * best[1], best
