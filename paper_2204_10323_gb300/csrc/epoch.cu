@@ -548,6 +548,18 @@ __global__ void gauges_kernel(Geom G, const T *h, const int64_t *cells, int ng, 
     out[k] = (double)h[(c / G.nx) * G.pitch + (c % G.nx)];
 }
 
+__global__ void __launch_bounds__(128)
+    gauge_rows_kernel(Geom G, const float *rows, int n_rows, const int *row, const int64_t *cells, int ng, int64_t n, double *out)
+{
+    pdl_wait();
+    pdl_launch();
+    for (int64_t x = blockIdx.x * 128LL + threadIdx.x; x < n; x += gridDim.x * 128LL) {
+        const int64_t s = x / ng, c = cells[x - s * ng];
+        const int j = (int)(c / G.nx);
+        out[x] = (double)rows[((size_t)s * n_rows + row[j]) * G.pitch + (c - (int64_t)j * G.nx)];
+    }
+}
+
 }  // namespace
 
 // Parts of a decomposed grid: the largest of their running depth maxima
@@ -678,6 +690,15 @@ cudaError_t launch_gauges(const Geom &g, const T *h, const int64_t *cells, int G
     if (G <= 0) return cudaSuccess;
     gauges_kernel<T><<<(G + 127) / 128, 128, 0, st>>>(g, h, cells, G, out);
     return cudaGetLastError();
+}
+
+cudaError_t launch_gauge_rows(const Geom &g, const float *rows, int n_rows, const int *row, const int64_t *cells, int G,
+                              int n_steps, double *out, cudaStream_t st)
+{
+    const int64_t n = (int64_t)n_steps * G, blocks = (n + 127) / 128;
+    if (n <= 0) return cudaSuccess;
+    return launch_pdl(gauge_rows_kernel, (unsigned)(blocks < 152 * 16 ? blocks : 152 * 16), 128, st, g, rows, n_rows, row, cells, G, n,
+                      out);
 }
 
 #define FLOOD_INST(T)                                                                                      \

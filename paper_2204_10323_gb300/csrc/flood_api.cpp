@@ -254,8 +254,7 @@ flood_status launch_inflow_epoch(flood_handle *h) { return launch_epoch(h, false
 flood_status begin_epoch(flood_handle *h, const double *fixed_dt) { return launch_epoch(h, true, fixed_dt); }
 
 template <typename T>
-StepArgs<T> make_args(flood_handle *h, int s, int k_steps, int want_hmax, const int64_t *gcells,
-                             int ng, double *gout)
+StepArgs<T> make_args(flood_handle *h, int s, int k_steps, int want_hmax, const Gauges &gauges, void *gout)
 {
     StepArgs<T> a;
     std::memset(&a, 0, sizeof(a));
@@ -282,15 +281,21 @@ StepArgs<T> make_args(flood_handle *h, int s, int k_steps, int want_hmax, const 
     a.s = s;
     a.k_steps = k_steps;
     a.want_hmax = want_hmax;
-    a.gauge_cells = gcells;
-    a.n_gauges = ng;
-    a.gauge_out = gout;
+    if (gauges.rows) {
+        a.gauge_row = gauges.row;
+        a.n_gauges = gauges.n_rows;
+        a.gauge_rows = (float *)gout;
+    } else {
+        a.gauge_cells = gauges.cells;
+        a.n_gauges = gauges.n;
+        a.gauge_out = (double *)gout;
+    }
     a.tile_x = h->tile_x;
     a.tile_y = h->tile_y;
     return a;
 }
 
-StepArgs<float> step_args_f32(flood_handle *h, int s) { return make_args<float>(h, s, 1, 0, nullptr, 0, nullptr); }
+StepArgs<float> step_args_f32(flood_handle *h, int s) { return make_args<float>(h, s, 1, 0, {}, nullptr); }
 
 // The FP32 step of the handle's kernel family for prepared arguments.
 static cudaError_t launch_f32(flood_handle *h, const StepArgs<float> &a)
@@ -305,14 +310,20 @@ static cudaError_t launch_f32(flood_handle *h, const StepArgs<float> &a)
 }
 
 // One launch of k steps starting at step-in-epoch s.
-flood_status launch_steps(flood_handle *h, int s, int k, int want_hmax, const int64_t *gcells, int ng,
-                          double *gout)
+flood_status launch_steps(flood_handle *h, int s, int k, int want_hmax, const Gauges &gauges, void *gout)
 {
     cudaError_t e;
-    if (h->prec == FLOOD_F64)
-        e = launch_step_reference<double>(make_args<double>(h, s, 1, want_hmax, gcells, ng, gout), h->stream);
-    else
-        e = launch_f32(h, make_args<float>(h, s, k, want_hmax, gcells, ng, gout));
+    if (h->prec == FLOOD_F64) {
+        e = launch_step_reference<double>(make_args<double>(h, s, 1, want_hmax, gauges, gout), h->stream);
+    } else {
+        StepArgs<float> a = make_args<float>(h, s, k, want_hmax, gauges, gout);
+        if (gout && !gauges.rows && h->kernel == FLOOD_KERNEL_TILED) {   // a single step and a gather
+            a.tile_x = a.tile_y = 0;
+            e = launch_step_stream(a, h->stream);
+        } else {
+            e = launch_f32(h, a);
+        }
+    }
     if (e != cudaSuccess) return cuda_fail(h, e, "step kernel launch");
     h->cur = 1 - h->cur;
     return FLOOD_OK;
@@ -334,11 +345,11 @@ flood_status launch_step_planes(flood_handle *h, int s, int k, const void *const
     cudaError_t e;
     if (h->prec == FLOOD_F64) {
         if (k != 1) return fail(h, FLOOD_ERR_ARG, "FP64 planes advance one step per launch");
-        StepArgs<double> a = make_args<double>(h, s, 1, 0, nullptr, 0, nullptr);
+        StepArgs<double> a = make_args<double>(h, s, 1, 0, {}, nullptr);
         set_planes(a, in, out);
         e = launch_step_reference<double>(a, h->stream);
     } else {
-        StepArgs<float> a = make_args<float>(h, s, k, 0, nullptr, 0, nullptr);
+        StepArgs<float> a = make_args<float>(h, s, k, 0, {}, nullptr);
         set_planes(a, in, out);
         // The temporal-blocking kernel for several steps, and for one on grids below 2^25 cells: us a step tiled
         // K = 1 / TMA / stream 9.7 / 13.9 / 15.9 (1024^2), 28 / 31 / 36 (2048^2), 97 / 99 / 103 (4096^2), but
@@ -355,15 +366,22 @@ flood_status launch_step_planes(flood_handle *h, int s, int k, const void *const
     return FLOOD_OK;
 }
 
-// Advance n steps; if gcells, record gauges after each step into gbuf (device, n x ng).
+// Advance n steps; if gbuf (device, n x gauges.n), record the gauges after each step.
 // epoch_open: the current epoch was begun already (its dt, times and inflow rows
 // are in place), so a first step at an epoch start does not begin it again.
-flood_status advance(flood_handle *h, int64_t n, const int64_t *gcells, int ng, double *gbuf,
-                     const double *fixed_dt_log, bool epoch_open)
+flood_status advance(flood_handle *h, int64_t n, const Gauges &gauges, double *gbuf, const double *fixed_dt_log,
+                     bool epoch_open)
 {
     NvtxRange range("flood: steps");
     const int E = h->geo.epoch_steps;
     int64_t done = 0;
+    int slab = 0;                                      // steps in the slab of rows
+    const auto take_out = [&]() -> flood_status {
+        CK(launch_gauge_rows(h->geo, gauges.rows, gauges.n_rows, gauges.row, gauges.cells, gauges.n, slab,
+                             gbuf + (done - slab) * gauges.n, h->stream));
+        slab = 0;
+        return FLOOD_OK;
+    };
     while (done < n) {
         int s = (int)(h->step % E);
         if (s == 0 && !(epoch_open && done == 0)) {
@@ -373,16 +391,25 @@ flood_status advance(flood_handle *h, int64_t n, const int64_t *gcells, int ng, 
             if (st) return st;
         }
         int k = 1;
-        if (h->prec == FLOOD_F32 && h->kernel == FLOOD_KERNEL_TILED) {
+        if (h->prec == FLOOD_F32 && h->kernel == FLOOD_KERNEL_TILED && (!gbuf || gauges.rows)) {
             k = std::min<int64_t>(h->k_per_launch, std::min<int64_t>(E - s, n - done));
         }
         int want = (s + k == E) ? 1 : 0;
-        flood_status st = launch_steps(h, s, k, want, gcells, ng, gcells ? gbuf + done * ng : nullptr);
+        void *gout = gbuf ? gbuf + done * gauges.n : nullptr;
+        if (gauges.rows) {
+            if (slab + k > gauges.cap) {
+                flood_status st = take_out();
+                if (st) return st;
+            }
+            gout = gauges.rows + (size_t)slab * gauges.n_rows * h->geo.pitch;
+            slab += k;
+        }
+        flood_status st = launch_steps(h, s, k, want, gauges, gout);
         if (st) return st;
         h->step += k;
         done += k;
     }
-    return FLOOD_OK;
+    return slab > 0 ? take_out() : FLOOD_OK;
 }
 
 flood_status check_device_status(flood_handle *h)
@@ -777,7 +804,7 @@ extern "C" flood_status flood_step(flood_handle *h, int64_t n_steps)
     if (n_steps < 0) return fail(h, FLOOD_ERR_ARG, "n_steps must be >= 0");
     if (h->sticky) return fail(h, FLOOD_ERR_STATE, "handle is in an error state; write a new state first");
     if (h->opts.use_graph) return advance_graph(h, n_steps);
-    return advance(h, n_steps, nullptr, 0, nullptr, nullptr);
+    return advance(h, n_steps, {}, nullptr, nullptr);
 }
 
 extern "C" flood_status flood_coarsen(int32_t precision, const void *src, int32_t nx, int32_t ny, int32_t factor,
@@ -848,7 +875,7 @@ extern "C" flood_status flood_advance(flood_handle *h, double t_end, int64_t *st
         int m = s;                                     // steps s .. m-1 end at or before t_end
         while (m < E && tl[m + 1] <= t_end) m++;
         if (m > s) {
-            flood_status st = advance(h, m - s, nullptr, 0, nullptr, nullptr, begun);
+            flood_status st = advance(h, m - s, {}, nullptr, nullptr, begun);
             if (st) return st;
             taken += m - s;
         }
@@ -861,7 +888,7 @@ extern "C" flood_status flood_advance(flood_handle *h, double t_end, int64_t *st
         const double dt = c.dt, dt_last = t_end - tl[m];
         CK(cudaMemcpyAsync(&h->ctrl->dt, &dt_last, sizeof(double), cudaMemcpyHostToDevice, h->stream));
         CK(cudaMemcpyAsync(h->t_list + m + 1, &t_end, sizeof(double), cudaMemcpyHostToDevice, h->stream));
-        flood_status st = advance(h, 1, nullptr, 0, nullptr, nullptr, begun && m == s);
+        flood_status st = advance(h, 1, {}, nullptr, nullptr, begun && m == s);
         if (st) return st;
         taken += 1;
         // the rest of the epoch continues from t_end with the epoch's dt
@@ -1043,6 +1070,17 @@ extern "C" flood_status flood_set_manning(flood_handle *h, const void *manning, 
     return FLOOD_OK;
 }
 
+// Gauges with the temporal-blocking kernel by rows, else by single steps and gathers.  The table of rows is made on the host,
+// some 2.5 ns a gauge and less a row of the grid, and a single step with its gather takes 10 us more than a
+// quarter of a launch of four (1024^2; more on larger grids): few steps with very many gauges, or of a tall narrow grid, do not earn it.
+static bool gauges_by_rows(const flood_handle *h, int64_t n_steps, int64_t n_gauges)
+{
+    const int64_t entries = n_gauges + h->geo.ny;
+    return h->prec == FLOOD_F32 && h->kernel == FLOOD_KERNEL_TILED && (entries <= 16384 || entries <= 4096 * n_steps);
+}
+
+static constexpr size_t kSlab = 64 << 20;
+
 extern "C" flood_status flood_run_gauges(flood_handle *h, int64_t n_steps, const int64_t *gauge_cells,
                                          int32_t n_gauges, double *out, int32_t out_on_device)
 {
@@ -1055,10 +1093,33 @@ extern "C" flood_status flood_run_gauges(flood_handle *h, int64_t n_steps, const
     for (int g = 0; g < n_gauges; g++)
         if (gauge_cells[g] < 0 || gauge_cells[g] >= nc) return fail(h, FLOOD_ERR_ARG, "gauge cell out of range");
     if (n_gauges == 0 || n_steps == 0) return flood_step(h, n_steps);
-    flood_status st = ensure_gauge_buffers(h, n_gauges, (size_t)n_steps * n_gauges);
+    Gauges gauges;
+    gauges.n = n_gauges;
+    std::vector<int64_t> up(gauge_cells, gauge_cells + n_gauges);     // the cells, and the rows' places behind them
+    const bool by_rows = gauges_by_rows(h, n_steps, n_gauges);
+    if (by_rows) {
+        up.resize(n_gauges + ((size_t)h->geo.ny + 1) / 2);
+        int *row = reinterpret_cast<int *>(up.data() + n_gauges);
+        std::fill(row, row + h->geo.ny, -1);
+        for (int g = 0; g < n_gauges; g++) {
+            int &place = row[gauge_cells[g] / h->geo.nx];
+            if (place < 0) place = gauges.n_rows++;
+        }
+    }
+    flood_status st = ensure_gauge_buffers(h, up.size() * sizeof(int64_t), (size_t)n_steps * n_gauges);
     if (st) return st;
-    CK(cudaMemcpyAsync(h->gauge_dev, gauge_cells, n_gauges * sizeof(int64_t), cudaMemcpyHostToDevice, h->stream));
-    st = advance(h, n_steps, h->gauge_dev, n_gauges, h->gauge_buf, nullptr);
+    CK(cudaMemcpyAsync(h->gauge_dev, up.data(), up.size() * sizeof(int64_t), cudaMemcpyHostToDevice, h->stream));
+    gauges.cells = (const int64_t *)h->gauge_dev;
+    if (by_rows) {
+        // a slab of rows for as many steps as kSlab holds, for one launch at least; without it single steps
+        const size_t step_bytes = (size_t)gauges.n_rows * h->geo.pitch * sizeof(float);
+        const int64_t k = std::min<int64_t>(h->k_per_launch, n_steps);
+        gauges.row = reinterpret_cast<const int *>(gauges.cells + n_gauges);
+        gauges.cap = (int)std::max<int64_t>(std::min<int64_t>(n_steps, (int64_t)(kSlab / step_bytes)), k);
+        gauges.rows = (float *)dev_alloc(h, gauges.cap * step_bytes);
+    }
+    st = advance(h, n_steps, gauges, h->gauge_buf, nullptr);
+    dev_free(h, gauges.rows);                          // (back to the pool, for work queued behind this on the stream)
     if (st) return st;
     CK(cudaMemcpyAsync(out, h->gauge_buf, (size_t)n_steps * n_gauges * sizeof(double),
                        out_on_device ? cudaMemcpyDeviceToDevice : cudaMemcpyDeviceToHost, h->stream));
@@ -1068,16 +1129,18 @@ extern "C" flood_status flood_run_gauges(flood_handle *h, int64_t n_steps, const
 
 namespace flood {
 
-flood_status ensure_gauge_buffers(flood_handle *h, int ng, size_t n_values)
+flood_status ensure_gauge_buffers(flood_handle *h, size_t bytes, size_t n_values)
 {
-    if (ng > h->gauge_cap) {
+    if (bytes > h->gauge_cap) {
         dev_free(h, h->gauge_dev);
-        h->gauge_dev = (int64_t *)dev_alloc(h, (size_t)ng * sizeof(int64_t));
+        h->gauge_cap = 0;
+        h->gauge_dev = dev_alloc(h, bytes);
         if (!h->gauge_dev) return fail(h, FLOOD_ERR_OOM, "gauge list allocation");
-        h->gauge_cap = ng;
+        h->gauge_cap = bytes;
     }
     if (n_values > h->gauge_buf_cap) {
         dev_free(h, h->gauge_buf);
+        h->gauge_buf_cap = 0;
         h->gauge_buf = (double *)dev_alloc(h, n_values * sizeof(double));
         if (!h->gauge_buf) return fail(h, FLOOD_ERR_OOM, "gauge series allocation");
         h->gauge_buf_cap = n_values;

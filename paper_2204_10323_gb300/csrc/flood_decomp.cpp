@@ -416,7 +416,7 @@ extern "C" flood_status flood_decomp_step(flood_decomp *d, int64_t n_steps)
             for (int k_done = 0; k_done < m;) {
                 int k = 1;
                 if (h->prec == FLOOD_F32 && h->kernel == FLOOD_KERNEL_TILED) k = std::min(h->k_per_launch, m - k_done);
-                flood_status st = launch_steps(h, s + k_done, k, 0, nullptr, 0, nullptr);
+                flood_status st = launch_steps(h, s + k_done, k, 0, {}, nullptr);
                 if (st) return part_fail(d, r, st);
                 k_done += k;
             }

@@ -18,7 +18,7 @@ static flood_status capture_epoch(flood_handle *h, int parity)
     h->cur = parity;
     e = cudaStreamBeginCapture(cap, cudaStreamCaptureModeThreadLocal);
     flood_status st = FLOOD_OK;
-    if (e == cudaSuccess) st = advance(h, h->geo.epoch_steps, nullptr, 0, nullptr, nullptr);
+    if (e == cudaSuccess) st = advance(h, h->geo.epoch_steps, {}, nullptr, nullptr);
     cudaGraph_t graph = nullptr;
     cudaError_t e2 = cudaStreamEndCapture(cap, &graph);
     h->stream = user;
@@ -47,7 +47,7 @@ flood_status advance_graph(flood_handle *h, int64_t n)
         int s = (int)(h->step % E);
         if (s != 0 || n < E) {
             int64_t k = s != 0 ? std::min<int64_t>(E - s, n) : n;
-            flood_status st = advance(h, k, nullptr, 0, nullptr, nullptr);
+            flood_status st = advance(h, k, {}, nullptr, nullptr);
             if (st) return st;
             n -= k;
             continue;

@@ -81,9 +81,18 @@ struct StepArgs {
     int s;                        // step index inside the epoch (first step of the launch)
     int k_steps;                  // steps done by this launch (1 except the tiled kernel)
     int want_hmax;                // 1: record max depth after the launch's last step
-    const int64_t *gauge_cells;   // flat j*nx+i; h after each step -> gauge_out
+    // Gauges after every step: n_gauges cells (flat j*nx+i) into n_gauges values of gauge_out (null: none).  Tiled:
+    // whole rows of depths instead, row r into place gauge_row[r] (< 0: none) of the step's n_gauges rows of `pitch`
+    // floats in gauge_rows (k_steps x n_gauges rows; null: none).
+    union {
+        const int64_t *gauge_cells;
+        const int *gauge_row;
+    };
     int n_gauges;
-    double *gauge_out;            // k_steps x n_gauges values of this launch, or null
+    union {
+        double *gauge_out;
+        float *gauge_rows;
+    };
     int tile_x, tile_y;           // launch shape (stream/TMA: warps, rows; tiled: rows per item of the edge
                                   // strips and of the others; on its way in: cap on pipelines, rows per item)
 };
@@ -234,6 +243,9 @@ cudaError_t launch_padding(void *a, size_t esz, int rows, int cols, int pitch, b
 // *gave_up (device) = 1 when the bounded wait gave up (the expected outcome).
 cudaError_t launch_wait_probe(uint64_t budget_ns, int *gave_up, cudaStream_t st);
 
+// The same from rows of depths (StepArgs::gauge_rows) of n_steps steps into out[n_steps][G].
+cudaError_t launch_gauge_rows(const Geom &g, const float *rows, int n_rows, const int *row, const int64_t *cells, int G,
+                              int n_steps, double *out, cudaStream_t st);
 // Gather h at gauge cells into out[0..G).
 template <typename T>
 cudaError_t launch_gauges(const Geom &g, const T *h, const int64_t *cells, int G, double *out,

@@ -50,8 +50,8 @@ struct flood_handle {
     double *vol_partials = nullptr, *vol_out = nullptr;
     int *flag = nullptr;                  // device word for the non-finite check of flood_write_state
     int n_partials = 1024;
-    int64_t *gauge_dev = nullptr;
-    int gauge_cap = 0;
+    void *gauge_dev = nullptr;             // the cells, and (temporal blocking) the rows' places
+    size_t gauge_cap = 0;                  // bytes
     double *gauge_buf = nullptr;
     size_t gauge_buf_cap = 0;
 
@@ -129,19 +129,29 @@ flood_status refresh_hmax(flood_handle *h);
 flood_status launch_inflow_epoch(flood_handle *h);
 flood_status begin_epoch(flood_handle *h, const double *fixed_dt = nullptr);
 EpochArgs<float> epoch_args_f32(flood_handle *h);
-flood_status launch_steps(flood_handle *h, int s, int k, int want_hmax, const int64_t *gcells, int ng,
-                          double *gout);
+// Gauges to record, on the device; rows, n_rows, row and cap (a slab of that many steps) where the temporal-blocking
+// kernel leaves the rows they lie in.
+struct Gauges {
+    const int64_t *cells = nullptr;
+    int n = 0;
+    const int *row = nullptr;
+    int n_rows = 0;
+    float *rows = nullptr;
+    int cap = 0;
+};
+// gout: the step's values, or (gauges.rows) rows.
+flood_status launch_steps(flood_handle *h, int s, int k, int want_hmax, const Gauges &gauges, void *gout);
 // One step at step-in-epoch s reading the state planes in[] = {h, qx, qy} and
 // writing out[] (pitched like the handle's state; the handle's own buffers and
 // its current index are not touched).
 // k steps (k > 1: FP32, Eq. 3 as printed, at most 4 and within the epoch) from the planes `in`
 // into the planes `out`, starting at step-in-epoch s.
 flood_status launch_step_planes(flood_handle *h, int s, int k, const void *const in[3], void *const out[3]);
-flood_status advance(flood_handle *h, int64_t n, const int64_t *gcells, int ng, double *gbuf,
-                     const double *fixed_dt_log, bool epoch_open = false);
+flood_status advance(flood_handle *h, int64_t n, const Gauges &gauges, double *gbuf, const double *fixed_dt_log,
+                     bool epoch_open = false);
 flood_status check_device_status(flood_handle *h);
 StepArgs<float> step_args_f32(flood_handle *h, int s);
-flood_status ensure_gauge_buffers(flood_handle *h, int ng, size_t n_values);
+flood_status ensure_gauge_buffers(flood_handle *h, size_t bytes, size_t n_values);
 
 // CUDA-graph epochs (flood_graph.cpp)
 flood_status advance_graph(flood_handle *h, int64_t n);

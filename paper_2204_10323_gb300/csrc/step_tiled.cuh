@@ -186,7 +186,6 @@ struct alignas(16) TiledSmem {
     float qy[kMode ? 4 : kAhead][128];   // and qy (the scheme options read it one row further on)
     float z[kRowsZ][128];
     float c[4][4][128];                  // face_c and the higher bed of a row's west and south faces, for levels 2 .. K
-    int gauge[32][3];                    // gauges in the item's own cells: row, staged column, index
 };
 
 // One work item: strip `strip`, rows [y0, y1) of grid a, steps s0 .. s0 + K - 1 of the epoch.
@@ -196,7 +195,10 @@ struct alignas(16) TiledSmem {
 // (4 more per option and level), the old qy of the row above is the row that level s - 1 has just
 // computed (level 1: the next row in flight).  A lane at the strip's edge takes its missing
 // neighbour column as garbage, like the plain arithmetic's edge lanes: it stays inside the halo.
-// kGauge: the depth of the item's gauges after each of the K steps goes to a.gauge_out.
+// kGauge: rows with gauges (a.gauge_row) go to a.gauge_rows after each of the K steps, the strip's own columns of them;
+// one launch takes the gauges out after many steps.  So the kernel knows rows only, whatever the gauges' number and
+// order.  (Recording from lists, every item testing all gauges, a crowded one scanning them at every tick, took
+// 194 ms for 64 steps of 1024^2 with 4096 gauges in a 64 x 64 patch, 0.60 so, and 0.56 with one gauge, 0.55 so.)
 template <int K, int kMode, bool kGauge>
 __device__ __forceinline__ void tiled_item(const StepArgs<float> &a, const int s0, const int strip, const int y0,
                                            const int y1, const int want_hmax, TiledSmem<kMode> &sm)
@@ -274,30 +276,12 @@ __device__ __forceinline__ void tiled_item(const StepArgs<float> &a, const int s
     };
     border_fetch(jb - bl);
 
-    // the item's gauges; one with more than 32 scans them all at every tick
-    int ng = 0;
-    auto gauge_at = [&](int g, int &row, int &col) {   // false: not in the item
-        const int64_t flat = a.gauge_cells[g];
-        row = (int)(flat / nx);
-        const int c = (int)(flat - (int64_t)row * nx);
-        col = c - x0;
-        return row >= y0 && row < y1 && c >= own_lo && c < own_hi;
+    unsigned gm = 0;                                   // (kGauge) bit s - 1 at tick j: row j - s has a place
+    const bool keep = c0 >= own_lo && c0 < own_hi;     // (a lane with the grid's last columns stores some padding too)
+    auto gauge_store = [&](int s, int r, const Row4 &v) {
+        if (((gm >> (s - 1)) & 1) && keep)
+            row_store(a.gauge_rows + ((size_t)(s - 1) * a.n_gauges + __ldg(a.gauge_row + r)) * P + lane_off, v);
     };
-    if constexpr (kGauge) {
-        for (int g0 = 0; g0 < a.n_gauges; g0 += 32) {
-            int row = 0, col = 0;
-            const bool mine = g0 + lane < a.n_gauges && gauge_at(g0 + lane, row, col);
-            const unsigned m = __ballot_sync(0xffffffffu, mine);
-            const int slot = ng + __popc(m & ((1u << lane) - 1));
-            if (mine && slot < 32) {
-                sm.gauge[slot][0] = row;
-                sm.gauge[slot][1] = col;
-                sm.gauge[slot][2] = g0 + lane;
-            }
-            ng += __popc(m);
-        }
-        __syncwarp();
-    }
 
     Row4 sh[K], sx[K], sy[K];                          // per level: the previous row's old depth and new faces
     Row4 ox[K], oy[K];                                 // the sums of its neighbouring old qx (kVec), its old qy (kTheta)
@@ -311,7 +295,8 @@ __device__ __forceinline__ void tiled_item(const StepArgs<float> &a, const int s
     auto tick = [&](auto steady_t, auto edge_t, const int j) {
         constexpr bool kSteady = decltype(steady_t)::value, kEdge = decltype(edge_t)::value;
         Row4 ch{0, 0}, cx{0, 0}, cy{0, 0}, cyn{0, 0};  // the current level's input row, and the old qy of the row above it
-        Row4 last{0, 0};                               // the row that level K finished (kGauge)
+        int place = -1;                                // of row j
+        if (kGauge && j >= y0 && j < y1) place = __ldg(a.gauge_row + j);
         copy_wait<kAhead - 1>();
 #pragma unroll
         for (int s = 1; s <= K; s++) {
@@ -430,11 +415,11 @@ __device__ __forceinline__ void tiled_item(const StepArgs<float> &a, const int s
                                 }
                             fin = row_pack(v[0], v[1], v[2], v[3]);
                         }
-                        if (kGauge && s == K) last = fin;
                         if (s == K && rr >= y0 && (kSteady || rr < y1)) {
                             const float2 g0 = f2unpack(fin.a), g1 = f2unpack(fin.b);
                             const size_t ro = (size_t)rr * P + lane_off;
                             const bool north = !kSteady && rr == ny - 1;   // the grid's north face row too
+                            if (kGauge) gauge_store(K, rr, fin);
                             const bool maximum = want_hmax && rr >= G.led_j0 && rr < G.led_j1;   // a part's own rows
                             if (kEdge ? full : lane >= 1 && lane <= kOut / 4) {
                                 if (maximum) hmax = max_nan(max_nan(hmax, max_nan(g0.x, g0.y)), max_nan(g1.x, g1.y));
@@ -499,23 +484,12 @@ __device__ __forceinline__ void tiled_item(const StepArgs<float> &a, const int s
             }
         }
         if constexpr (kGauge) {
-            // level s finished row j - s: the next level's previous row (level K's: last)
-            const int n_scan = ng > 32 ? a.n_gauges : ng;
-            for (int x = 0; x < n_scan; x++) {
-                int row, col, idx = x;
-                if (ng <= 32) {
-                    row = sm.gauge[x][0];
-                    col = sm.gauge[x][1];
-                    idx = sm.gauge[x][2];
-                } else if (!gauge_at(x, row, col)) continue;
-                const int k = col & 3;
+            // level s finished row j - s, the next level's previous row (level K stored its own above)
+            if (gm & ((1u << (K - 1)) - 1)) {
 #pragma unroll
-                for (int s = 1; s <= K; s++) {
-                    const Row4 v = s < K ? sh[s < K ? s : 0] : last;
-                    if (row == j - s && lane == col >> 2)
-                        a.gauge_out[(size_t)(s - 1) * a.n_gauges + idx] = (double)row_get(v, k);
-                }
+                for (int s = 1; s < K; s++) gauge_store(s, j - s, sh[s]);
             }
+            gm = gm << 1 | (place >= 0 ? 1u : 0u);
         }
         if (kEdge && (west || east)) {
             float h = 0.0f;
@@ -587,7 +561,6 @@ __device__ __forceinline__ void tiled_item(const StepArgs<float> &a, const int s
         }
     }
     copy_wait<0>();
-    if constexpr (kGauge) __syncwarp();                // before the next item's list
     if (lane == 0) {
         if (led_q != 0.0) atomicAdd(&a.ctrl->V_out, a.ctrl->dt * led_q * G.dx);
         if (led_c != 0.0) atomicAdd(&a.ctrl->V_clip, led_c * G.dx * G.dx);
@@ -722,7 +695,7 @@ cudaError_t launch_k(const StepArgs<float> &a0, cudaStream_t st)
     blocks = a0.tile_x > 0 && a0.tile_x < items ? a0.tile_x : items;    // caller's cap on pipelines
     a.tile_x = edge;
     a.tile_y = rows;
-    return launch_pdl(a.gauge_out && a.n_gauges > 0 ? step_tiled_kernel<K, kMode, true> : step_tiled_kernel<K, kMode, false>,
+    return launch_pdl(a.gauge_rows ? step_tiled_kernel<K, kMode, true> : step_tiled_kernel<K, kMode, false>,
                       blocks, 32, st, a);
 }
 
