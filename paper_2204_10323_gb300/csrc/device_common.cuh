@@ -185,6 +185,29 @@ __device__ __forceinline__ void atomic_max_nonneg(unsigned long long *addr, doub
     atomicMax(addr, (unsigned long long)__double_as_longlong(v));
 }
 
+// The first of n gauges (in the order of rows and columns) from position x on that does not lie before (row, col), by a
+// warp: among the next 32, where it mostly lies, else by 32 probes a round.
+__device__ __forceinline__ int gauge_seek(const int4 *__restrict__ list, int n, int x, int row, int col)
+{
+    const auto before = [&](int k) {                   // how many of the warp's probes come before
+        const int4 g = k < n ? __ldg(list + k) : make_int4(row, col, 0, 0);
+        return __popc(__ballot_sync(0xffffffffu, g.x < row || (g.x == row && g.y < col)));
+    };
+    const int lane = threadIdx.x & 31;
+    int m = before(x + lane);
+    x += m;
+    if (m < 32) return x;
+#pragma unroll 1
+    while (n - x > 32) {
+        const int step = (n - x + 31) >> 5;
+        m = before(x + lane * step);
+        if (m == 0) return x;
+        n = min(n, x + m * step);
+        x += (m - 1) * step + 1;
+    }
+    return x + before(x + lane);
+}
+
 // Inward unit sign of a side: +1 on xmin / ymin, -1 on xmax / ymax.
 __device__ __forceinline__ int inward_sign(int side) { return (side == 0 || side == 2) ? 1 : -1; }
 

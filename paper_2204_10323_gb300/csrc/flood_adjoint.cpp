@@ -14,6 +14,7 @@
 
 #include <algorithm>
 #include <cstring>
+#include <utility>
 #include <vector>
 
 #include "flood_internal.h"
@@ -55,6 +56,18 @@ int64_t revolve_cost(int64_t l, int64_t c)
 }
 
 namespace {
+
+// (row, column, index) of every gauge, in that order.
+std::vector<int4> gauge_list(const int64_t *cells, int n, int nx)
+{
+    std::vector<std::pair<int64_t, int>> order(n);
+    for (int g = 0; g < n; g++) order[g] = {cells[g], g};
+    if (!std::is_sorted(order.begin(), order.end())) std::sort(order.begin(), order.end());
+    std::vector<int4> list(n);
+    for (int k = 0; k < n; k++)
+        list[k] = make_int4((int)(order[k].first / nx), (int)(order[k].first % nx), order[k].second, 0);
+    return list;
+}
 
 #define CKA(expr)                                                     \
     do {                                                              \
@@ -105,7 +118,7 @@ struct Sweep {
     int64_t log_first = 0;        // global step of the log's first entry
     int cur_l = 0;
     const int64_t *cells = nullptr;
-    const int2 *cells_rc = nullptr;
+    const int4 *list = nullptr;
     int G = 0;
     const double *seed = nullptr;    // device, N x G
     int64_t fwd_steps = 0;
@@ -331,7 +344,7 @@ flood_status reverse_step_t(Sweep &S)
     A.sec_cells = h->sec_cells;
     A.inflow_W = h->inflow_W;
     A.gauge_cells = S.cells;
-    A.gauge_rc = S.cells_rc;
+    A.gauge_list = S.list;
     A.n_gauges = S.G;
     A.seed = S.seed + (size_t)k * S.G;      // dL/dh after step k, added to lambda_{k+1}
     A.scratch = (T *)S.scratch;
@@ -538,14 +551,13 @@ extern "C" flood_status flood_adjoint(flood_handle *h, int64_t n_steps, const in
         }
     }
     double *seed_dev = (double *)alloc(std::max<size_t>((size_t)n_steps * n_gauges, 1) * sizeof(double));
-    int64_t *cells_dev = (int64_t *)alloc(std::max(n_gauges, 1) * (sizeof(int64_t) + sizeof(int2)));
-    int2 *rc_dev = (int2 *)(cells_dev + std::max(n_gauges, 1));
-    std::vector<int2> rc(n_gauges);
-    for (int g = 0; g < n_gauges; g++)
-        rc[g] = make_int2((int)(gauge_cells[g] / h->geo.nx), (int)(gauge_cells[g] % h->geo.nx));
+    void *cells_dev = alloc(std::max(n_gauges, 1) * sizeof(int4));
+    const bool listed = h->prec == FLOOD_F32 && !opts;   // the row walk takes a list, the other reverse steps the cells
+    std::vector<int4> list;
+    if (listed) list = gauge_list(gauge_cells, n_gauges, h->geo.nx);
     for (void *p : {(void *)S.dt_log, (void *)S.tl_log, S.iq_log, (void *)S.iQ_log, (void *)S.iW_log, S.lh[0],
                     S.lh[1], S.lqx[0], S.lqx[1], S.lqy[0], S.lqy[1], S.lhu, (void *)S.gn, (void *)seed_dev,
-                    (void *)cells_dev})
+                    cells_dev})
         if (!p) {
             release();
             return fail(h, FLOOD_ERR_OOM, "adjoint buffer allocation");
@@ -591,8 +603,8 @@ extern "C" flood_status flood_adjoint(flood_handle *h, int64_t n_steps, const in
     if (n_gauges > 0) {
         CKF(cudaMemcpyAsync(seed_dev, dLdh, (size_t)n_steps * n_gauges * sizeof(double), cudaMemcpyHostToDevice,
                             h->stream));
-        CKF(cudaMemcpyAsync(cells_dev, gauge_cells, n_gauges * sizeof(int64_t), cudaMemcpyHostToDevice, h->stream));
-        CKF(cudaMemcpyAsync(rc_dev, rc.data(), n_gauges * sizeof(int2), cudaMemcpyHostToDevice, h->stream));
+        if (listed) CKF(cudaMemcpyAsync(cells_dev, list.data(), n_gauges * sizeof(int4), cudaMemcpyHostToDevice, h->stream));
+        else CKF(cudaMemcpyAsync(cells_dev, gauge_cells, n_gauges * sizeof(int64_t), cudaMemcpyHostToDevice, h->stream));
     }
     // the adjoint after the last step; every reverse step writes the other half whole (and lhu before it is read)
     CKF(cudaMemsetAsync(S.lh[0], 0, S.plane, h->stream));
@@ -600,8 +612,8 @@ extern "C" flood_status flood_adjoint(flood_handle *h, int64_t n_steps, const in
     CKF(cudaMemsetAsync(S.lqy[0], 0, S.plane_y, h->stream));
     CKF(cudaMemsetAsync(S.gn, 0, P * h->geo.ny * sizeof(double), h->stream));
     if (S.gn_in) CKF(cudaMemsetAsync(S.gn_in, 0, (size_t)S.n_in_cells * sizeof(double), h->stream));
-    S.cells = cells_dev;
-    S.cells_rc = rc_dev;
+    S.cells = listed ? nullptr : (const int64_t *)cells_dev;
+    S.list = listed ? (const int4 *)cells_dev : nullptr;
     S.G = n_gauges;
     S.seed = seed_dev;
     // FP32 forward replays run the arithmetic the adjoint linearises: launches of up to four steps

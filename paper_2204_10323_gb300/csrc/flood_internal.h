@@ -192,7 +192,7 @@ struct AdjArgs {
     const int64_t *sec_cells;
     const double *inflow_W;       // E x n_sec levels of this epoch
     const int64_t *gauge_cells;   // flat j*nx+i of the loss's gauges
-    const int2 *gauge_rc;         // the same as (row, column)
+    const int4 *gauge_list;       // FP32, Eq. 3 as printed: the same as (row, column, index), in that order
     int n_gauges;
     const double *seed;           // dL/d(depth at gauge g after this step), n_gauges values (device)
     T *scratch;                   // scheme options only: 11 planes of pitch x (ny + 1) elements (face

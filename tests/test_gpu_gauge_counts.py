@@ -1,12 +1,13 @@
 """Gauges in any number: spread over the grid or all in one patch, repeated, in random order, recorded through the
 temporal-blocking kernel and its scheme options over whole launches and a short one, against the single-step
-kernel's gather (bit for bit), and the time of a run with thousands of them in one patch against the same
-run with one.
+kernel's gather (bit for bit); their seeds in the FP32 reverse step against the FP64 one; and the time of a run
+with thousands of them in one patch against the same run with one.
 """
 import numpy as np
 import pytest
 
 import inputs
+from inputs import OUTFLOW, XMAX, Options, Problem, Section
 
 pytestmark = pytest.mark.gpu
 
@@ -101,6 +102,29 @@ def test_series_with_any_launch_shape(k, tile):
     assert np.array_equal(out[0], out[1])
 
 
+@pytest.mark.parametrize("kind,count", [("spread", 33), ("patch", 1600), ("row", 250), ("spread", 3000)])
+def test_seeds_of_many_gauges(kind, count):
+    """Wet land, 0.6-0.8 m, steps of 0.1 s: no decision flips, and a reverse step rounds some twenty operations (6e-8
+    each) that the friction derivative amplifies by 7/3: 1e-5 a step, 1e-4 of the largest gradient over 8 steps."""
+    Fm = F()
+    nx, ny, steps = 190, 70, 8
+    rng = np.random.default_rng(7)
+    f = lambda a: a.astype(np.float32).astype(np.float64)
+    z = f(1.0 - 1e-3 * np.arange(nx)[None, :] + rng.uniform(-0.02, 0.02, (ny, nx)))
+    p = Problem("seeds", nx, ny, 4.0, z, f(rng.uniform(0.03, 0.06, (ny, nx))),
+                [Section.cells(XMAX, 0, ny, OUTFLOW, 2e-3, nx, ny)],
+                Options(dt_mode=1, dt_const=0.1, dt_cap=0.1, epoch_steps=8), h0=f(0.6 + rng.uniform(0.0, 0.2, (ny, nx))))
+    at = gauges(kind, count, nx, ny, count)
+    w = rng.standard_normal((steps, count))
+    out = []
+    for prec in (Fm.F64, Fm.F32):
+        s = Fm.Sim(p, precision=prec)
+        out.append(s.adjoint(steps, at, w, n_checkpoints=8, want_dh0=True))
+        s.close()
+    for a, b in zip(*out):
+        assert np.abs(b - a).max() <= 1e-4 * np.abs(a).max()
+
+
 def test_time_with_thousands_of_gauges_in_a_patch():
     """Single steps and a gather take about twice the launches of four steps on this grid, and each of them a few
     microseconds more for the gauges: five times one gauge's time is well above either way, a scan of all gauges by
@@ -124,4 +148,22 @@ def test_time_with_thousands_of_gauges_in_a_patch():
         return min(times)
     patch = np.stack([400 + np.arange(4096) % 64, 400 + np.arange(4096) // 64], 1)
     assert best(patch) <= 5.0 * best(patch[:1])
+    s.close()
+
+
+def test_time_of_reverse_steps_with_thousands_of_gauges_in_a_patch():
+    """A row of the patch takes 64 additions in turn, a few times what the row takes without; a scan of all gauges a row
+    took 250 times as long as a step with one gauge."""
+    Fm = F()
+    s = Fm.Sim(inputs.lake_at_rest(1024, 1024))
+    patch = np.stack([400 + np.arange(4096) % 64, 400 + np.arange(4096) // 64], 1)
+    s.adjoint_profile(True)
+    best = []
+    for at in (patch, patch[:1]):
+        times = []
+        for _ in range(4):
+            s.adjoint(16, at, np.ones((16, len(at))), n_checkpoints=16)
+            times.append(s.adjoint_times()["reverse_ms"] / 16)
+        best.append(min(times))
+    assert best[0] <= 8.0 * best[1], best
     s.close()
