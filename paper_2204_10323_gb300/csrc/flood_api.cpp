@@ -6,6 +6,7 @@
 
 #include <c10/cuda/CUDACachingAllocator.h>
 #include <c10/cuda/CUDAStream.h>
+#include <cuda.h>
 #include <cuda_runtime.h>
 
 #include <algorithm>
@@ -176,18 +177,40 @@ void field_shape(const flood_handle *h, int field, int *rows, int *cols)
     *cols = h->geo.nx + (field == FLOOD_FIELD_QX ? 1 : 0);
 }
 
+// Bytes from p to the end of its allocation on the device (0: not known).
+static size_t allocation_left(const void *p)
+{
+    using Range = CUresult (*)(CUdeviceptr *, size_t *, CUdeviceptr);
+    static const Range range = [] {
+        void *f = nullptr;
+        cudaDriverEntryPointQueryResult q = cudaDriverEntryPointSymbolNotFound;
+        if (cudaGetDriverEntryPointByVersion("cuMemGetAddressRange", &f, 12000, cudaEnableDefault, &q) == cudaSuccess &&
+            q == cudaDriverEntryPointSuccess)
+            return reinterpret_cast<Range>(f);
+        return (Range) nullptr;
+    }();
+    CUdeviceptr base = 0;
+    size_t size = 0;
+    if (!range || range(&base, &size, (CUdeviceptr)p) != CUDA_SUCCESS) return 0;
+    return size - (size_t)((CUdeviceptr)p - base);
+}
+
 cudaError_t copy_rows(void *dst, size_t dpitch, const void *src, size_t spitch, size_t width, size_t rows, int on_device,
                       bool to_device, int device, cudaStream_t st)
 {
     if (!on_device)
         return cudaMemcpy2DAsync(dst, dpitch, src, spitch, width, rows,
                                  to_device ? cudaMemcpyHostToDevice : cudaMemcpyDeviceToHost, st);
-    // memory of this device: the copy kernel; anything else that the caller calls device memory is
-    // left to the runtime's copy, which checks it
+    // memory of this device: the copy kernel, if the rows end inside its allocation, an error if not; anything
+    // else that the caller calls device memory is left to the runtime's copy, which checks it
+    const void *mine = to_device ? src : dst;
     cudaPointerAttributes at;
-    const cudaError_t e = cudaPointerGetAttributes(&at, to_device ? src : dst);
-    if (e == cudaSuccess && at.type == cudaMemoryTypeDevice && at.device == device)
-        return launch_copy_rows(dst, dpitch, src, spitch, width, rows, st);
+    const cudaError_t e = cudaPointerGetAttributes(&at, mine);
+    if (e == cudaSuccess && at.type == cudaMemoryTypeDevice && at.device == device) {
+        const size_t bytes = rows ? (rows - 1) * (to_device ? spitch : dpitch) + width : 0, left = allocation_left(mine);
+        if (left && bytes > left) return cudaErrorInvalidValue;
+        if (left) return launch_copy_rows(dst, dpitch, src, spitch, width, rows, st);
+    }
     if (e != cudaSuccess) (void)cudaGetLastError();
     return cudaMemcpy2DAsync(dst, dpitch, src, spitch, width, rows, cudaMemcpyDeviceToDevice, st);
 }
