@@ -14,6 +14,7 @@
 
 #include <algorithm>
 #include <cstring>
+#include <new>
 #include <utility>
 #include <vector>
 
@@ -554,7 +555,12 @@ extern "C" flood_status flood_adjoint(flood_handle *h, int64_t n_steps, const in
     void *cells_dev = alloc(std::max(n_gauges, 1) * sizeof(int4));
     const bool listed = h->prec == FLOOD_F32 && !opts;   // the row walk takes a list, the other reverse steps the cells
     std::vector<int4> list;
-    if (listed) list = gauge_list(gauge_cells, n_gauges, h->geo.nx);
+    try {
+        if (listed) list = gauge_list(gauge_cells, n_gauges, h->geo.nx);
+    } catch (const std::bad_alloc &) {
+        release();
+        return fail(h, FLOOD_ERR_OOM, "gauge list");
+    }
     for (void *p : {(void *)S.dt_log, (void *)S.tl_log, S.iq_log, (void *)S.iQ_log, (void *)S.iW_log, S.lh[0],
                     S.lh[1], S.lqx[0], S.lqx[1], S.lqy[0], S.lqy[1], S.lhu, (void *)S.gn, (void *)seed_dev,
                     cells_dev})
