@@ -14,6 +14,7 @@
 #include <cmath>
 #include <cstdio>
 #include <cstring>
+#include <new>
 #include <string>
 #include <vector>
 
@@ -1118,10 +1119,17 @@ extern "C" flood_status flood_run_gauges(flood_handle *h, int64_t n_steps, const
     if (n_gauges == 0 || n_steps == 0) return flood_step(h, n_steps);
     Gauges gauges;
     gauges.n = n_gauges;
-    std::vector<int64_t> up(gauge_cells, gauge_cells + n_gauges);     // the cells, and the rows' places behind them
-    const bool by_rows = gauges_by_rows(h, n_steps, n_gauges);
+    std::vector<int64_t> up;                           // the cells, and the rows' places behind them
+    bool by_rows = gauges_by_rows(h, n_steps, n_gauges);
     if (by_rows) {
-        up.resize(n_gauges + ((size_t)h->geo.ny + 1) / 2);
+        try {
+            up.resize(n_gauges + ((size_t)h->geo.ny + 1) / 2);
+        } catch (const std::bad_alloc &) {
+            by_rows = false;
+        }
+    }
+    if (by_rows) {
+        std::copy(gauge_cells, gauge_cells + n_gauges, up.begin());
         int *row = reinterpret_cast<int *>(up.data() + n_gauges);
         std::fill(row, row + h->geo.ny, -1);
         for (int g = 0; g < n_gauges; g++) {
@@ -1129,9 +1137,10 @@ extern "C" flood_status flood_run_gauges(flood_handle *h, int64_t n_steps, const
             if (place < 0) place = gauges.n_rows++;
         }
     }
-    flood_status st = ensure_gauge_buffers(h, up.size() * sizeof(int64_t), (size_t)n_steps * n_gauges);
+    const size_t up_bytes = (by_rows ? up.size() : (size_t)n_gauges) * sizeof(int64_t);
+    flood_status st = ensure_gauge_buffers(h, up_bytes, (size_t)n_steps * n_gauges);
     if (st) return st;
-    CK(cudaMemcpyAsync(h->gauge_dev, up.data(), up.size() * sizeof(int64_t), cudaMemcpyHostToDevice, h->stream));
+    CK(cudaMemcpyAsync(h->gauge_dev, by_rows ? up.data() : gauge_cells, up_bytes, cudaMemcpyHostToDevice, h->stream));
     gauges.cells = (const int64_t *)h->gauge_dev;
     if (by_rows) {
         // a slab of rows for as many steps as kSlab holds, for one launch at least; without it single steps
