@@ -467,6 +467,17 @@ flood_status flood_debug_padding(flood_handle *h, int32_t fill, int64_t *bad);
 flood_status flood_debug_tiled_split(int32_t nx, int32_t ny, int32_t k_steps, int32_t mode, int32_t resident,
                                      int32_t *chunk_rows, int32_t *blocks, int32_t *n_items);
 
+/*
+ * flood_debug_tiled_rows: rows per work item that the temporal-blocking kernel
+ * takes on n grids of nx[k] x ny[k] cells (host only, no device): each alone on
+ * the GPU (most_rows 0) or all in an ensemble whose launch shape has most_rows
+ * rows.  k_steps 1..4, mode as above.  rows[k] for inner strips, rows_edge[k] for
+ * the one or two strips with the borders x = 0 and x = nx, items[k] the grid's
+ * items.  FLOOD_ERR_ARG (no message) for arguments out of range.
+ */
+flood_status flood_debug_tiled_rows(int32_t n, const int32_t *nx, const int32_t *ny, int32_t k_steps, int32_t mode,
+                                    int32_t most_rows, int32_t *rows, int32_t *rows_edge, int32_t *items);
+
 /* Library version string. */
 const char *flood_version(void);
 

@@ -138,6 +138,8 @@ def _load():
     L.flood_debug_padding.restype = C.c_int
     L.flood_debug_tiled_split.argtypes = [i32, i32, i32, i32, i32, C.POINTER(C.c_int32), C.POINTER(C.c_int32),
                                           C.POINTER(C.c_int32)]
+    L.flood_debug_tiled_rows.argtypes = [i32, vp, vp, i32, i32, i32, vp, vp, vp]
+    L.flood_debug_tiled_rows.restype = C.c_int
     for name in ("flood_decomp_plan", "flood_decomp_combine_ledgers", "flood_decomp_create", "flood_decomp_step",
                  "flood_decomp_read", "flood_decomp_write_state", "flood_decomp_sync", "flood_decomp_destroy"):
         getattr(L, name).restype = C.c_int
@@ -250,8 +252,19 @@ def flood_debug_fail_alloc_after(n: int) -> None:
     lib().flood_debug_fail_alloc_after(int(n))
 
 
+def flood_debug_tiled_rows(shapes, k_steps: int = 4, mode: int = 0, most_rows: int = 0):
+    """(rows, edge rows, items) of the temporal-blocking kernel for each (nx, ny), alone on the GPU or (most_rows > 0) in an
+    ensemble (host only; see include/flood.h)."""
+    n = len(shapes)
+    a = (C.c_int32 * n)
+    nx, ny, out = a(*[s[0] for s in shapes]), a(*[s[1] for s in shapes]), [a(), a(), a()]
+    _check(lib().flood_debug_tiled_rows(n, nx, ny, int(k_steps), int(mode), int(most_rows), *out), None)
+    return list(zip(*out))
+
+
 def flood_debug_tiled_split(nx: int, ny: int, k_steps: int = 4, mode: int = 0, resident: int = 912) -> dict:
-    """The temporal-blocking kernel's work items for an nx x ny grid (host only)."""
+    """The temporal-blocking kernel's work items for an nx x ny grid held to `resident` pipelines that walk them in turn
+    (flood_opts.tile_x; host only)."""
     rows, blocks, items = C.c_int32(), C.c_int32(), C.c_int32()
     _check(lib().flood_debug_tiled_split(int(nx), int(ny), int(k_steps), int(mode), int(resident), C.byref(rows),
                                          C.byref(blocks), C.byref(items)), None)

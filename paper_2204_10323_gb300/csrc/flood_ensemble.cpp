@@ -86,34 +86,33 @@ void drop_graphs(flood_ensemble *e)
 // by the square root of the grid's cells over that, at least 8 and at most the
 // grid's rows.  The grids come largest first, so the items shrink towards the end of
 // a launch, where the small ones fill the tail.
-int item_rows(const flood_ensemble *e, const Geom &g)
+int item_rows(int base_rows, const Geom &g)
 {
     const double cells = (double)g.nx * g.ny;
-    const int r = (int)(e->base_rows * std::sqrt(cells / (double)(1 << 20)) + 0.5);
+    const int r = (int)(base_rows * std::sqrt(cells / (double)(1 << 20)) + 0.5);
     return std::min(std::max(r, 8), g.ny);
 }
 
 int edge_rows(int rows) { return (5 * rows + 7) / 8; }
 
-// base_rows, at most the launch shape's rows: each item repeats 2K rows, and the launch ends
+// base_rows, at most `most` (the launch shape's rows): each item repeats 2K rows, and the launch ends
 // with its longest items' last rows, so few rows cost work and many leave warps idle.  The cost is
-// the items' ticks over the warps that the GPU holds, or the longest item if that is more, and a tenth of the
-// longest item for the tail (two groups fill each other's).  20 scenarios of 256^2 .. 2048^2, us a step at 32 / 48 /
-// 64 / 96 / 128 / 256 rows: 72.4 / 68.0 / 66.4 / 79.9 / 94.6 / 157.  (With the arguments in the launch 61.2 at the
-// 64 chosen.)
-void choose_rows(flood_ensemble *e)
+// the items' ticks over the warps that the GPU holds (8 an SM with the theta weighting, else 12), or the longest item
+// if that is more, and a tenth of the longest item for the tail (two groups fill each other's).  20 scenarios of
+// 256^2 .. 2048^2, us a step at most 16 / 24 / 32 / 40 / 48 / 64 rows: 78.6 / 70.6 / 66.3 / 63.8 / 63.7 / 60.9, the 64 chosen
+// (128: 94.6 before the arguments travelled with the launch, against 66.4).  Theta scenarios by 8 warps / by 12: 10.7 / 11.7 (3 of
+// them), 24.4 / 25.1 (5), 39.6 / 42.6 (20 uneven ones), the same rows and time for 10, 20 and 40.
+int choose_rows(const std::vector<Geom> &grids, int K, int mode, int most)
 {
-    const double resident = 152.0 * 12.0;      // one-warp items the GPU holds at once
-    const int K = e->k_steps;
+    const double resident = tiled_resident(mode);
     double best = -1.0;
-    int rows = e->rows;
-    for (int b : {8, 12, 16, 20, 24, 32, 40, 48, 64, 80, 96, 128, 160, 192, 256, 320, 384, 512, e->rows}) {
-        if (b > e->rows) continue;
-        e->base_rows = b;
+    int rows = most;
+    for (int b : {8, 12, 16, 20, 24, 32, 40, 48, 64, 80, 96, 128, 160, 192, 256, 320, 384, 512, most}) {
+        if (b > most) continue;
         double ticks = 0.0, longest = 0.0;
-        for (const flood_handle *h : e->members) {
-            const int r = item_rows(e, h->geo);
-            ticks += (double)tiled_items(h->geo, r, edge_rows(r), K) * (r + 2 * K);
+        for (const Geom &g : grids) {
+            const int r = item_rows(b, g);
+            ticks += (double)tiled_items(g, r, edge_rows(r), K) * (r + 2 * K);
             longest = std::max(longest, (double)(r + 2 * K));
         }
         const double cost = std::max(ticks / resident, longest) + 0.1 * longest;
@@ -122,18 +121,20 @@ void choose_rows(flood_ensemble *e)
             rows = b;
         }
     }
-    e->base_rows = rows;
+    return rows;
 }
 
 flood_status build_tables(flood_ensemble *e)
 {
     const int n = (int)e->members.size();
-    choose_rows(e);
+    std::vector<Geom> grids;
+    for (const flood_handle *h : e->members) grids.push_back(h->geo);
+    e->base_rows = choose_rows(grids, e->k_steps, e->mode, e->rows);
     std::vector<int> base(n + 1, 0), tbase(n + 1, 0);
     for (int k = 0; k < n; k++) {
         const Geom &g = e->members[e->order[k]]->geo;
         base[k + 1] = base[k] + stream_blocks(g, e->warps, e->rows);
-        tbase[k + 1] = tbase[k] + tiled_items(g, item_rows(e, g), edge_rows(item_rows(e, g)), e->k_steps);
+        tbase[k + 1] = tbase[k] + tiled_items(g, item_rows(e->base_rows, g), edge_rows(item_rows(e->base_rows, g)), e->k_steps);
     }
     e->total_blocks = base[n];
     e->total_items = tbase[n];
@@ -144,7 +145,7 @@ flood_status build_tables(flood_ensemble *e)
             const int cur = h->cur;
             h->cur = p;
             t[k] = step_args_f32(h, 0);
-            t[k].tile_y = item_rows(e, h->geo);
+            t[k].tile_y = item_rows(e->base_rows, h->geo);
             t[k].tile_x = edge_rows(t[k].tile_y);
             h->cur = cur;
         }
@@ -172,7 +173,7 @@ flood_status build_tables(flood_ensemble *e)
             gb.assign(ng + 1, 0);
             for (int i = 0; i < ng; i++) {
                 const Geom &G = e->members[members[g][i]]->geo;
-                gb[i + 1] = gb[i] + tiled_items(G, item_rows(e, G), edge_rows(item_rows(e, G)), e->k_steps);
+                gb[i + 1] = gb[i] + tiled_items(G, item_rows(e->base_rows, G), edge_rows(item_rows(e->base_rows, G)), e->k_steps);
             }
             e->gn[g] = ng;
             for (int p = 0; p < 2; p++) {
@@ -183,7 +184,7 @@ flood_status build_tables(flood_ensemble *e)
                     const int cur = h->cur;
                     h->cur = p;
                     t[i] = step_args_f32(h, 0);
-                    t[i].tile_y = item_rows(e, h->geo);
+                    t[i].tile_y = item_rows(e->base_rows, h->geo);
                     t[i].tile_x = edge_rows(t[i].tile_y);
                     h->cur = cur;
                 }
@@ -551,4 +552,30 @@ extern "C" flood_status flood_ensemble_destroy(flood_ensemble *e)
 extern "C" const char *flood_ensemble_last_error(const flood_ensemble *e)
 {
     return e ? e->err.c_str() : g_ens_error.c_str();
+}
+
+extern "C" flood_status flood_debug_tiled_rows(int32_t n, const int32_t *nx, const int32_t *ny, int32_t k_steps, int32_t mode,
+                                               int32_t most_rows, int32_t *rows, int32_t *rows_edge, int32_t *items)
+{
+    if (n < 1 || !nx || !ny || k_steps < 1 || k_steps > 4 || mode < 0 || mode > 3 || most_rows < 0 || !rows || !rows_edge || !items)
+        return FLOOD_ERR_ARG;
+    std::vector<Geom> grids(n);
+    for (int k = 0; k < n; k++) {
+        if (nx[k] < 1 || ny[k] < 1 || (int64_t)nx[k] * ny[k] > (int64_t)1 << 34) return FLOOD_ERR_ARG;
+        grids[k].nx = nx[k];
+        grids[k].ny = ny[k];
+        grids[k].theta = (mode & 1) ? 0.9 : 1.0;
+        grids[k].friction = mode >> 1;
+    }
+    const int base = most_rows > 0 ? choose_rows(grids, k_steps, mode, most_rows) : 0;
+    for (int k = 0; k < n; k++) {
+        if (most_rows > 0) {
+            rows[k] = item_rows(base, grids[k]);
+            rows_edge[k] = edge_rows(rows[k]);
+        } else {
+            tiled_rows(nx[k], ny[k], k_steps, mode, &rows[k], &rows_edge[k]);
+        }
+        items[k] = tiled_items(grids[k], rows[k], rows_edge[k], k_steps);
+    }
+    return FLOOD_OK;
 }

@@ -114,6 +114,9 @@ cudaError_t launch_step_tma(const StepArgs<float> &a, cudaStream_t st);
 // Temporal blocking over many grids, k_steps steps from s0: the items of grid k are base[k] .. base[k+1] - 1
 // (tiled_items per grid, table[k].tile_y rows per item, tile_x in the edge strips).
 int tiled_items(const Geom &g, int rows, int rows_edge, int k_steps);
+// Multiprocessors of the GPU (152 where there is none), and the one-warp items of a scheme mode that it holds at once.
+int sm_count();
+int tiled_resident(int mode);
 // Rows per work item (inner strips, and the one or two strips with the borders x = 0 and x = nx) for a grid
 // alone on the GPU.
 void tiled_rows(int nx, int ny, int K, int mode, int *rows, int *rows_edge);

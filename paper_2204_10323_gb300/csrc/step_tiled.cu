@@ -5,6 +5,20 @@
 
 namespace flood {
 
+int sm_count()
+{
+    static const int n = [] {
+        int dev = 0, v = 0;
+        if (cudaGetDevice(&dev) == cudaSuccess && cudaDeviceGetAttribute(&v, cudaDevAttrMultiProcessorCount, dev) == cudaSuccess && v > 0)
+            return v;
+        (void)cudaGetLastError();
+        return 152;
+    }();
+    return n;
+}
+
+int tiled_resident(int mode) { return sm_count() * tiled_warps(mode); }
+
 // Rows per item.  An item of r rows takes r + 2K ticks; a tick of a warp alone on its quarter of an SM
 // takes about 1650 cycles, beside others about 1150 + 490 per warp (K = 4, measured with the clock
 // register at 1024^2 .. 4096^2), and 1000 more in an edge strip, whose items are therefore shorter.  The
@@ -25,7 +39,7 @@ void tiled_rows_for(int n_strips, int ny, int repeat, int warps, double base, do
 {
     static constexpr int kTry[] = {2,  3,  4,  6,  8,  10, 12, 14, 16,  18,  20,  22,  24,  28,  32, 36,
                                    40, 44, 48, 56, 64, 80, 96, 112, 128, 144, 160, 192, 256};
-    const int sms = 152, resident = sms * warps, n_edge = n_strips < 2 ? n_strips : 2;
+    const int sms = sm_count(), resident = sms * warps, n_edge = n_strips < 2 ? n_strips : 2;
     const auto tick = [&](double w) { return base + slope * (w > 1.0 ? w : 1.0); };
     const auto even = [&](int r) { return (ny + (ny + r - 1) / r - 1) / ((ny + r - 1) / r); };   // equal chunks of at most r
     double best = -1.0;
