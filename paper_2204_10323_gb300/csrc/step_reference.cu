@@ -199,14 +199,16 @@ __global__ void __launch_bounds__(32) step_reference_kernel(const __grid_constan
     }
 }
 
-// Rows per item: an item of r rows computes 2 r + 1 rows of faces, but the FP64 pipes even out over many
-// short items, whose wet ones cluster.  us a step (with the ordinary division by dx) at 1 / 2 / 3 / 4 / 8 rows: 15.3 / 21.5 / 25.8 / 31.8 / 53.1
-// (128^2), 59 / 68 / 66 / 67 / 85 (512^2), 142 / 130 / 142 / 134 / 139 (1001 x 777), 117 / 107 / 105 / 109 /
-// 112 (1200^2, 10 % wet), 298 / 261 / 251 / 255 / 255 (1001 x 777, 90 % wet).
+// Rows per item: an item of r rows computes 2 r + 1 rows of faces, but the FP64 pipes even out over many short items,
+// whose wet ones cluster.  us a step at 1 / 2 / 3 rows, 30 % and 90 % wet: 17.7 / 26.0 / 34.6 and 19.5 / 26.1 / 34.6
+// (128^2), 32 / 29 / 36 and 42 / 38 / 44 (256^2), 38 / 49 / 40 and 65 / 66 / 66 (360^2), 58 / 58 / 70 and 103 / 102 / 90 (512^2),
+// 78 / 70 / 79 and 150 / 140 / 141 (640^2), 94 / 88 / 82 and 186 / 161 / 158 (720^2), 136 / 116 / 121 and 269 / 232 / 218
+// (1001 x 777), 173 / 143 / 137 and 357 / 299 / 283 (1024^2), 228 / 184 / 175 and 475 / 395 / 371 (1200^2): one row up to where
+// two draw level for good, three from where they lead at either wetness.
 int reference_rows(int nx, int ny)
 {
     const int64_t cells = (int64_t)nx * ny;
-    return cells < (1 << 19) ? 1 : cells < (1 << 20) ? 2 : 3;
+    return cells < (1 << 18) ? 1 : cells < (1 << 20) ? 2 : 3;
 }
 
 }  // namespace
