@@ -34,12 +34,9 @@ struct flood_ensemble {
     StepArgs<float> *table[2] = {nullptr, nullptr};   // per parity of the ping-pong buffers
     int *base = nullptr;                   // block prefix, n + 1
     int total_blocks = 0;
-    int *tbase = nullptr;                  // tiled item prefix, n + 1
-    int total_items = 0;
     // tiled: the members in two groups of about equal cells, each launched on a stream of its
     // own from one epoch start to the next, so that one group's launches fill the other's tails
     static constexpr int kGroups = 2;
-    std::vector<int> group_of;             // per member
     StepArgs<float> *gtable[kGroups][2] = {{nullptr, nullptr}, {nullptr, nullptr}};   // [group][parity]
     int *gtbase[kGroups] = {nullptr, nullptr};
     std::vector<StepArgs<float>> gargs[kGroups][2];          // the same on the host
@@ -130,14 +127,12 @@ flood_status build_tables(flood_ensemble *e)
     std::vector<Geom> grids;
     for (const flood_handle *h : e->members) grids.push_back(h->geo);
     e->base_rows = choose_rows(grids, e->k_steps, e->mode, e->rows);
-    std::vector<int> base(n + 1, 0), tbase(n + 1, 0);
+    std::vector<int> base(n + 1, 0);
     for (int k = 0; k < n; k++) {
         const Geom &g = e->members[e->order[k]]->geo;
         base[k + 1] = base[k] + stream_blocks(g, e->warps, e->rows);
-        tbase[k + 1] = tbase[k] + tiled_items(g, item_rows(e->base_rows, g), edge_rows(item_rows(e->base_rows, g)), e->k_steps);
     }
     e->total_blocks = base[n];
-    e->total_items = tbase[n];
     for (int p = 0; p < 2; p++) {
         std::vector<StepArgs<float>> t(n);
         for (int k = 0; k < n; k++) {
@@ -154,8 +149,6 @@ flood_status build_tables(flood_ensemble *e)
         if (c != cudaSuccess) return efail(e, FLOOD_ERR_CUDA, cudaGetErrorString(c));
     }
     cudaError_t c = cudaMemcpyAsync(e->base, base.data(), (n + 1) * sizeof(int), cudaMemcpyHostToDevice, e->stream);
-    if (c != cudaSuccess) return efail(e, FLOOD_ERR_CUDA, cudaGetErrorString(c));
-    c = cudaMemcpyAsync(e->tbase, tbase.data(), (n + 1) * sizeof(int), cudaMemcpyHostToDevice, e->stream);
     if (c != cudaSuccess) return efail(e, FLOOD_ERR_CUDA, cudaGetErrorString(c));
     // the groups: largest member first into the group with fewer cells so far
     {
@@ -401,7 +394,6 @@ extern "C" flood_status flood_ensemble_create(int32_t n, const flood_grid *grids
         }
     }
     e->base = (int *)dev_alloc(e->owner, (n + 1) * sizeof(int));
-    e->tbase = (int *)dev_alloc(e->owner, (n + 1) * sizeof(int));
     for (int g = 0; g < flood_ensemble::kGroups; g++) {
         for (int p = 0; p < 2; p++) e->gtable[g][p] = (StepArgs<float> *)dev_alloc(e->owner, n * sizeof(StepArgs<float>));
         e->gtbase[g] = (int *)dev_alloc(e->owner, (n + 1) * sizeof(int));
@@ -432,7 +424,7 @@ extern "C" flood_status flood_ensemble_create(int32_t n, const flood_grid *grids
     }
     e->n_tasks = (int)tk.size();
     e->tasks = (int2 *)dev_alloc(e->owner, std::max<size_t>(tk.size(), 1) * sizeof(int2));
-    if (!e->base || !e->tbase || !e->etab || !e->tasks ||
+    if (!e->base || !e->etab || !e->tasks ||
         cudaMemcpyAsync(e->etab, et.data(), n * sizeof(EpochArgs<float>), cudaMemcpyHostToDevice, e->stream) ||
         (tk.size() &&
          cudaMemcpyAsync(e->tasks, tk.data(), tk.size() * sizeof(int2), cudaMemcpyHostToDevice, e->stream))) {
@@ -528,7 +520,6 @@ extern "C" flood_status flood_ensemble_destroy(flood_ensemble *e)
         for (int p = 0; p < 2; p++)
             if (e->table[p]) dev_free(e->owner, e->table[p]);
         if (e->base) dev_free(e->owner, e->base);
-        if (e->tbase) dev_free(e->owner, e->tbase);
         for (int g = 0; g < flood_ensemble::kGroups; g++) {
             for (int p = 0; p < 2; p++)
                 if (e->gtable[g][p]) dev_free(e->owner, e->gtable[g][p]);
