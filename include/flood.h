@@ -101,7 +101,7 @@ typedef enum {
     FLOOD_KERNEL_AUTO = 0,       /* TILED (K = 4) with E a multiple of 4 and no launch shape given (Eq. 3
                                     as printed and the scheme options alike); else TMA below 2^27 cells,
                                     else STREAM */
-    FLOOD_KERNEL_REFERENCE = 1,  /* one thread per cell, IEEE ops in the oracle's order */
+    FLOOD_KERNEL_REFERENCE = 1,  /* one warp per strip of 31 columns and a few rows, IEEE ops in the oracle's order */
     FLOOD_KERNEL_ROWS = 2,       /* one warp per 128-column strip, float4 row streaming */
     FLOOD_KERNEL_TILED = 3,      /* one warp per strip and chunk, K steps per launch in registers (temporal blocking) */
     FLOOD_KERNEL_STREAM = 4,     /* one warp per 128-column strip, rows staged by bulk copies (default) */

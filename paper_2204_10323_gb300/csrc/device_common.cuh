@@ -43,9 +43,9 @@ template <> struct R<double> {
 // FP64: q0 = RN(a y) with y = RN(1 / b), r = a - q0 b (exact by fma), RN(q0 + r y), which is RN(a / b) by Markstein's
 // theorem (IBM J. Res. Dev. 34, 1990: a faithful q0 and a correctly rounded y suffice, nothing under- or
 // overflowing).  q0 is faithful where |y b - 1| <= 2^-54: then a y lies less than half a unit in the last place of a / b
-// from it (a quarter just above a power of two).  That holds for 1, 3, 5 and their multiples by powers of two;
-// elsewhere, and for tiny or huge dividends, the ordinary division, which takes about eight operations
-// of the FP64 pipe (two a cycle and SM) for the three here.
+// from it (a quarter just above a power of two).  That holds for all powers of two, for most whole numbers (93 of 1 .. 100; 49 is
+// one of the others) and about seven divisors in ten; elsewhere, and for tiny or huge dividends, the ordinary division,
+// which takes about eight operations of the FP64 pipe (two a cycle and SM) for the three here.
 template <typename T> struct Divisor {
     T b;
     __device__ explicit Divisor(T b_) : b(b_) {}

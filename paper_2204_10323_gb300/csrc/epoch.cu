@@ -131,8 +131,9 @@ __device__ double section_total_warp(const InflowSec &S, const T *sz, const T *s
 }
 
 // The level search.  The section's discharge is increasing in the level W and, for the cross-section form
-// (h^(5/3)), convex: Newton's method from above falls monotonically to the root in a handful of evaluations,
-// where the halvings took 25 (FP32) or 41 and more (FP64), each a chain of powers and a sum over the section.
+// (h^(5/3)), convex: Newton's method from above falls monotonically to the root in a handful of evaluations (in double
+// and on one warp in single precision; 26 on longer single-precision sections), where the halvings took 25 (FP32, one
+// warp) or 41 and more, each a chain of powers and a sum over the section.
 // An iteration that leaves the bracket is replaced by a halving, as are all of them for the literal form
 // (h^(2/3): its slope is infinite where a cell falls dry).
 

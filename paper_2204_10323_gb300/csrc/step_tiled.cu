@@ -62,7 +62,8 @@ void tiled_rows_for(int n_strips, int ny, int repeat, int warps, double base, do
 
 // Row chunks for the items of a grid of n_strips strips and ny rows on `resident` pipelines that walk
 // them in turn (a caller's cap on the pipelines): the chunk count minimises the ticks of the busiest
-// pipeline, (items per pipeline) x (chunk rows + 3K - 1).
+// pipeline, (items per pipeline) x (chunk rows + 3K - 1).  (An item runs 2K ticks more than it has rows by now; callers of
+// flood_debug_tiled_split rely on the values of this form, and the choice between them is a matter of a per cent.)
 static void tiled_split(int n_strips, int ny, int resident, int K, int *chunk_rows, int *blocks)
 {
     static thread_local int memo[4] = {-1, -1, -1, -1}, memo_rows = 0;   // per thread: no race between handles
