@@ -87,8 +87,9 @@ __global__ void __launch_bounds__(128) coarsen_small_kernel(const T *__restrict_
             if ((count & (count - 1)) == 0) {           // a scaling, exact (a sum near zero is not taken)
                 out = __fmul_rn(s, __int_as_float((127 - (31 - __clz(count))) << 23));
             } else {
-                const float q = __fdiv_rn(s, n);
-                out = __fadd_rn(q, __fdiv_rn(__fadd_rn(__fmaf_rn(-q, n, s), c), n));
+                // the quotient by an approximate reciprocal, its remainder (exact) divided likewise
+                const float y = __fdividef(1.0f, n), q = __fmul_rn(s, y);
+                out = __fmaf_rn(__fadd_rn(__fmaf_rn(-q, n, s), c), y, q);
             }
             // the error's bound against 2^-31 of the mean, both times 2^31 n
             const bool close = __fmul_rn((float)((kRows ? f : f * f) + 8) * 0x1p-17f, m) <= __fmul_rn(fabsf(out), n);
