@@ -674,15 +674,34 @@ __device__ __forceinline__ void adj_rows_item(const AdjArgs<float> &A, const int
     };
     for (int j = jb; j < jb + kAhead; j++) issue(j);
 
-    // The next gauge of the list (by row, column and index) that may lie in the staged cells, and its row.  (Crowded items
-    // that scanned all gauges at every row took 5.0 ms a step of 1024^2 with 4096 gauges in a 64 x 64 patch, the tile kernel
-    // before them 0.76; following the list 0.105, and 0.019 with one gauge as before.)
-    int gp = 0, grow = 0x7fffffff;
-    auto gauge_from = [&](int x, int row) {
-        gp = gauge_seek(A.gauge_list, A.n_gauges, x, row, x0);
-        grow = gp < A.n_gauges ? A.gauge_list[gp].x : 0x7fffffff;
+    // The gauges, from a list in the order of rows, columns and indexes: each lane holds one of a window of 32, with its seed;
+    // `pending` are those in the staged cells yet to come, grow the row of the first.  (Crowded items that scanned all gauges at
+    // every row took 5.0 ms a step of 1024^2 with 4096 gauges in a 64 x 64 patch, the tile kernel before them 0.76; so 0.092,
+    // and 0.019 with one gauge as before.)
+    int wx = 0, wrow = 0, wcol = 0, grow = 0x7fffffff;
+    float wseed = 0.0f;
+    unsigned pending = 0;
+    auto window = [&](int x, int row) {                // from x on, or from the first one at (row, x0) or after it
+#pragma unroll 1
+        for (;;) {
+            wx = x;
+            const int4 g = x + lane < A.n_gauges ? __ldg(A.gauge_list + x + lane) : make_int4(0x7fffffff, 0, 0, 0);
+            const bool mine = g.x >= row && g.x <= jhi && g.y >= x0 && g.y < x0 + 64;
+            wrow = g.x;
+            wcol = g.y - x0;
+            pending = __ballot_sync(0xffffffffu, mine);
+            if (pending) {
+                wseed = mine ? (float)A.seed[g.z] : 0.0f;
+                grow = __shfl_sync(0xffffffffu, wrow, __ffs(pending) - 1);
+                return;
+            }
+            grow = 0x7fffffff;
+            const int last = __shfl_sync(0xffffffffu, wrow, 31);
+            if (last > jhi) return;
+            x = gauge_seek(A.gauge_list, A.n_gauges, x + 32, max(row, last), x0);
+        }
     };
-    gauge_from(0, jb);
+    window(A.n_gauges > 32 ? gauge_seek(A.gauge_list, A.n_gauges, 0, jb, x0) : 0, jb);
 
     Pair hp = 0, zp = 0, np_ = 0;                // row j - 1: depth, bed, n
     Pair xp = 0, yp = 0;                           // its new faces
@@ -742,26 +761,26 @@ __device__ __forceinline__ void adj_rows_item(const AdjArgs<float> &A, const int
             const float2 u0 = f2unpack(f2fma(f2dup(Kc.dtdx), dv, hp));
             const float u[2] = {u0.x, u0.y};
             float v[2] = {f2unpack(lu).x, f2unpack(lu).y};
-            if (grow == j - 1) {                       // their seeds, 32 at a time (repeated gauges add up in order)
-                int x = gauge_seek(A.gauge_list, A.n_gauges, gp, j - 1, x0);
-                const int x1 = gauge_seek(A.gauge_list, A.n_gauges, x, j - 1, x0 + 64);
-                for (; x < x1; x += 32) {
-                    int4 g = make_int4(0, 0, 0, 0);
-                    float sd = 0.0f;
-                    if (x + lane < x1) {
-                        g = A.gauge_list[x + lane];
-                        sd = (float)A.seed[g.z];
-                    }
-                    const int m = min(32, x1 - x);
-                    for (int q = 0; q < m; q++) {
-                        const int gc = __shfl_sync(0xffffffffu, g.y, q) - c0;
-                        const float sq = __shfl_sync(0xffffffffu, sd, q);
+            if (grow == j - 1) {                       // the row's seeds, in the list's order (repeated gauges add up in theirs)
+#pragma unroll 1
+                for (;;) {
+                    unsigned now = pending & __ballot_sync(0xffffffffu, wrow == j - 1);
+                    pending &= ~now;
+#pragma unroll 1
+                    for (; now; now &= now - 1) {
+                        const int q = __ffs(now) - 1, gc = __shfl_sync(0xffffffffu, wcol, q) - 2 * lane;
+                        const float sd = __shfl_sync(0xffffffffu, wseed, q);
 #pragma unroll
                         for (int k = 0; k < 2; k++)
-                            if (gc == k) v[k] = v[k] + sq;
+                            if (gc == k) v[k] = v[k] + sd;
                     }
+                    if (pending) {
+                        grow = __shfl_sync(0xffffffffu, wrow, __ffs(pending) - 1);
+                        break;
+                    }
+                    window(wx + 32, j - 1);
+                    if (grow != j - 1) break;
                 }
-                gauge_from(x1, j);
             }
 #pragma unroll
             for (int k = 0; k < 2; k++) {
