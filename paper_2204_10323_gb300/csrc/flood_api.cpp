@@ -1103,7 +1103,7 @@ static bool gauges_by_rows(const flood_handle *h, int64_t n_steps, int64_t n_gau
     return h->prec == FLOOD_F32 && h->kernel == FLOOD_KERNEL_TILED && (entries <= 16384 || entries <= 4096 * n_steps);
 }
 
-static constexpr size_t kSlab = 64 << 20;
+static constexpr size_t kSlab = 64 << 20, kSlabKept = 8 << 20;
 
 extern "C" flood_status flood_run_gauges(flood_handle *h, int64_t n_steps, const int64_t *gauge_cells,
                                          int32_t n_gauges, double *out, int32_t out_on_device)
@@ -1148,10 +1148,22 @@ extern "C" flood_status flood_run_gauges(flood_handle *h, int64_t n_steps, const
         const int64_t k = std::min<int64_t>(h->k_per_launch, n_steps);
         gauges.row = reinterpret_cast<const int *>(gauges.cells + n_gauges);
         gauges.cap = (int)std::max<int64_t>(std::min<int64_t>(n_steps, (int64_t)(kSlab / step_bytes)), k);
-        gauges.rows = (float *)dev_alloc(h, gauges.cap * step_bytes);
+        const size_t need = gauges.cap * step_bytes;
+        if (need <= h->gauge_slab_cap) {
+            gauges.rows = (float *)h->gauge_slab;
+        } else {
+            dev_free(h, h->gauge_slab);
+            h->gauge_slab = dev_alloc(h, need);
+            h->gauge_slab_cap = h->gauge_slab ? need : 0;
+            gauges.rows = (float *)h->gauge_slab;
+        }
     }
     st = advance(h, n_steps, gauges, h->gauge_buf, nullptr);
-    dev_free(h, gauges.rows);                          // (back to the pool, for work queued behind this on the stream)
+    if (h->gauge_slab_cap > kSlabKept) {               // (back to the pool, for work queued behind this on the stream)
+        dev_free(h, h->gauge_slab);
+        h->gauge_slab = nullptr;
+        h->gauge_slab_cap = 0;
+    }
     if (st) return st;
     CK(cudaMemcpyAsync(out, h->gauge_buf, (size_t)n_steps * n_gauges * sizeof(double),
                        out_on_device ? cudaMemcpyDeviceToDevice : cudaMemcpyDeviceToHost, h->stream));

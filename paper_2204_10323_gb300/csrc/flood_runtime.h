@@ -52,6 +52,8 @@ struct flood_handle {
     int n_partials = 1024;
     void *gauge_dev = nullptr;             // the cells, and (temporal blocking) the rows' places
     size_t gauge_cap = 0;                  // bytes
+    void *gauge_slab = nullptr;            // small slabs of rows are kept
+    size_t gauge_slab_cap = 0;
     double *gauge_buf = nullptr;
     size_t gauge_buf_cap = 0;
 
