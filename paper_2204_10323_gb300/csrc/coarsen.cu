@@ -52,9 +52,10 @@ template <typename T, int V> struct alignas(sizeof(T) * V) Vec {
 };
 
 template <typename T, int V, bool kRows>
-__global__ void __launch_bounds__(128) coarsen_small_kernel(const T *__restrict__ src, int nx, int ny, int f, T *__restrict__ dst,
+__global__ void __launch_bounds__(128) coarsen_small_kernel(const T *__restrict__ src, int nx, int ny, int factor, T *__restrict__ dst,
                                                             int mx, int my)
 {
+    const int f = !kRows && V == 4 ? 4 : factor;       // (vectors of four and rows of at most four)
     const int I = blockIdx.x * blockDim.x + threadIdx.x;
     if (I >= mx) return;
     const int i0 = I * f, i1 = min(i0 + f, nx);
