@@ -61,7 +61,7 @@ static_assert(out_cols(1, 1) % 4 == 0 && out_cols(2, 1) % 4 == 0 && out_cols(3, 
 
 // Items resident per SM that the launch bounds ask for: 8, 12 or 16 (255, 168 or 128 registers; the
 // compiler knows no steps between).  Gcell/s at 12 / 16, Eq. 3 as printed, 16384^2: 577 / 563 (16 spills
-// 176 bytes).  At 12 / 8, vector norm, 8192^2: 414 / 393 (12 spills 200 bytes and still leads); theta,
+// 176 bytes).  At 12 / 8, vector norm, 8192^2: 414 / 393 (12 spilled 200 bytes then, 48 now, and leads); theta,
 // 8192^2: 424 / 434 and 1500 x 701: 100 / 111.
 __host__ __device__ constexpr int tiled_warps(int mode) { return (mode & 1) ? 8 : 12; }
 
