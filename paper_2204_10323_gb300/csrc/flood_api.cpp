@@ -178,8 +178,8 @@ void field_shape(const flood_handle *h, int field, int *rows, int *cols)
     *cols = h->geo.nx + (field == FLOOD_FIELD_QX ? 1 : 0);
 }
 
-// Bytes from p to the end of its allocation, if that is ordinary memory of this device (else 0).  One query of the driver for all of
-// it: the runtime's for the kind and the driver's for the range, one after the other, cost a small read 0.5 us more.
+// Bytes from p to the end of its allocation, if that is ordinary memory of this device (else 0).  One query of the CUDA
+// driver for all of it: one of the runtime for the kind and another for the range cost a small read 0.5 us more.
 static size_t device_bytes(const void *p, int device)
 {
     using Query = CUresult (*)(unsigned, CUpointer_attribute *, void **, CUdeviceptr);
