@@ -235,6 +235,8 @@ flood_status flood_set_manning(flood_handle *h, const void *manning, int32_t src
  * Advance n_steps and record the depth at n_gauges gauge cells after every
  * step: out[k*n_gauges + g] = h(gauge g) after step k, as doubles.  gauge_cells
  * are flat cell indices j*nx + i (host array).  out is host or device memory.
+ * The temporal-blocking kernel records whole rows into scratch of up to 64 MB
+ * (or four steps' rows); without memory for it the call takes single steps.
  */
 flood_status flood_run_gauges(flood_handle *h, int64_t n_steps, const int64_t *gauge_cells,
                               int32_t n_gauges, double *out, int32_t out_on_device);
